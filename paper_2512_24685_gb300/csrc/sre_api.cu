@@ -14,6 +14,8 @@
 
 #include "sre_batched.h"
 #include "sre_internal.h"
+#include "sre_one.h"
+#include "sre_two.h"
 
 namespace {
 
@@ -50,6 +52,7 @@ struct sre_plan_s {
     sre_tuning_t user = {-1, -1, -1, -1, -1, -1, -1};           // sre_plan_set_tuning
     sre::LargeCfg tuned[SRE_MAX_QUBITS + 1];        // sre_plan_autotune results
     bool has_tuned[SRE_MAX_QUBITS + 1] = {};
+    sre_mode_t tuned_mode[SRE_MAX_QUBITS + 1] = {};  // the mode it was tuned in
     void *tune_state = nullptr;                     // synthetic state for autotuning
     sre::LargeCfg batch_cfg[SRE_MAX_QUBITS + 1];    // configurations handed to batches
     double *d_series = nullptr;                     // one step's M2 values (time series)
@@ -219,8 +222,10 @@ sre_status_t sre_plan_destroy(sre_plan_t p) {
 // Configuration of the halved shifts for N > 12: the library default, then
 // the autotuned one, then the caller's explicit fields.
 static sre::LargeCfg plan_cfg(sre_plan_t p, int N) {
-    const int eb = elem_bytes_for_mode(p->mode);
-    sre::LargeCfg c = p->has_tuned[N] ? p->tuned[N] : sre::choose_large_cfg(p->dev, N, eb, 1);
+    // a tuned configuration serves the kernel it was timed on: the FP32 modes'
+    // kernels count items and lag differently
+    const bool tuned = p->has_tuned[N] && (p->tuned_mode[N] == SRE_MODE_FP32) == (p->mode == SRE_MODE_FP32);
+    sre::LargeCfg c = tuned ? p->tuned[N] : sre::choose_main_cfg(p->dev, p->ws, N, p->mode);
     if (p->user.x_batch_log >= 0) c.C_log = p->user.x_batch_log;
     if (p->user.ring_slots >= 0) c.R = p->user.ring_slots;
     if (p->user.lag >= 0) c.D = p->user.lag;
@@ -243,7 +248,7 @@ static sre_status_t enqueue_plan(sre_plan_t p, const void *d_state, int N, uint6
     sre::LargeCfg *cp = nullptr;
     if (N > sre::kTileBits) {
         c = plan_cfg(p, N);
-        if (!sre::large_cfg_fits(p->ws, c, N, 1)) return SRE_EINVAL;
+        if (!sre::main_cfg_fits(p->ws, c, N, p->mode)) return SRE_EINVAL;
         cp = &c;
     }
     return enqueue_plan_cfg(p, d_state, N, xb, xe, st, d_m2, d_per_x, cp, alpha);
@@ -293,8 +298,10 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
                                double *ms_out) {
     if (!p || N < 1 || N > p->N) return SRE_EINVAL;
     if (N <= sre::kTileBits) return SRE_OK;
-    // halved shifts taken by the single-pass kernel: nothing to tune
-    if (sre::mid_applies(N, 1, elem_bytes_for_mode(p->mode)) && !sre::tc_mode_available(p->mode)) return SRE_OK;
+    // N <= 15 in FP32 and N <= 14 in FP64 run in a single pass: nothing to tune
+    if (sre::mid_applies(N, 1, elem_bytes_for_mode(p->mode)) ||
+        (p->mode == SRE_MODE_FP32 && N < 16 && sre::one_applies(N, 8)))
+        return SRE_OK;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if (!p->tune_state) {
@@ -307,7 +314,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
     // once (one lag step claims the P1 + P2 items of a chunk) or the largest
     // ring 2 D + 1 the scratch holds
     const int eb = elem_bytes_for_mode(p->mode);
-    const sre::LargeCfg base = sre::choose_large_cfg(p->dev, N, eb, 1);
+    const sre::LargeCfg base = sre::choose_main_cfg(p->dev, p->ws, N, p->mode);
     const int h2 = N - sre::kTileBits - 1;
     // the tensor-core kernel runs one CTA per SM and always stages its
     // copies, so its lag steps are counted over the SMs, its lag is tried at
@@ -320,9 +327,26 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
             if (o.C_log == c.C_log && o.G2_log == c.G2_log && o.B1_log == c.B1_log && o.D == c.D &&
                 o.R == c.R && o.stage1 == c.stage1 && o.stage2 == c.stage2)
                 return;
-        if (sre::large_cfg_fits(p->ws, c, N, 1)) cands.push_back(c);
+        if (sre::main_cfg_fits(p->ws, c, N, p->mode)) cands.push_back(c);
     };
-    for (int C_log = 0; C_log <= 3; ++C_log)
+    // the FP32 kernel of sre_two.cu has no item sizes or copy paths to vary:
+    // shifts per item and ring alone
+    const bool two = p->mode == SRE_MODE_FP32 && sre::two_applies(N, eb);
+    // N = 16 in FP32 runs in a single pass: nothing to vary, its time alone
+    const bool one = p->mode == SRE_MODE_FP32 && sre::one_applies(N, eb);
+    if (one) add(base);
+    for (int C_log = 0; two && C_log <= 3; ++C_log) {
+        sre::LargeCfg c = base;
+        c.C_log = C_log;
+        const size_t chunk = ((size_t)eb << (N - 1)) << C_log;
+        const int fit = (int)std::min<size_t>(p->ws.scratch_bytes / chunk, sre::kMaxRing);
+        for (int R : {fit, fit * 3 / 4, fit / 2, fit / 4, base.R}) {
+            c.R = R;
+            c.D = R - 1;
+            add(c);
+        }
+    }
+    for (int C_log = 0; !two && !one && C_log <= 3; ++C_log)
         for (int g = 0; g <= 3; ++g)
             for (int b = 2; b <= 3; ++b)
                 for (int dm = 0; dm <= (tc ? 6 : 3); ++dm) {
@@ -421,6 +445,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
     if (s != SRE_OK) return s;
     p->tuned[N] = best_c;
     p->has_tuned[N] = true;
+    p->tuned_mode[N] = p->mode;
     if (best) {
         best->x_batch_log = best_c.C_log;
         best->ring_slots = best_c.R;

@@ -165,7 +165,17 @@ cudaError_t batched_run(BatchedContext *ctx, const Workspace &ws, const DeviceIn
         int j = k;
         while (j < count && Ns[order[j]] == Ns[order[k]]) ++j;
         const int N = Ns[order[k]];
-        classes.push_back(batch_class_layout(dev, ws, N, j - k, mode, tuned_half ? tuned_half[N] : nullptr));
+        // split modes: a class whose halved shifts fit the tensor-core kernel
+        // (16 <= N <= 20) and whose states are all 16-byte aligned takes it
+        // (converted copies are aligned)
+        int tc_kind = 0;
+        if (tc_mode_available(mode) && N > kTileBits && tc_applies(N, 1, 2, nullptr)) {
+            bool aligned = true;
+            for (int q = k; q < j; ++q) aligned &= dtype != SRE_C64 || ((uintptr_t)d_states[order[q]] & 15) == 0;
+            if (aligned) tc_kind = mode == SRE_MODE_BF16_SPLIT ? 1 : 2;
+        }
+        classes.push_back(
+            batch_class_layout(dev, ws, N, j - k, mode, tuned_half ? tuned_half[N] : nullptr, tc_kind));
         k = j;
     }
     size_t parts_total = 0, chunk_cap = 1;
@@ -232,23 +242,10 @@ cudaError_t batched_run(BatchedContext *ctx, const Workspace &ws, const DeviceIn
         sptr[k] = convert ? (const void *)((char *)g.conv + off) : d_states[order[k]];
         if (convert) off += (size_t)(fp64 ? 16 : 8) << sNs[k];
     }
-    // split modes: a class whose halved shifts fit the tensor-core kernel
-    // (16 <= N <= 20) and whose states are all 16-byte aligned takes it
     {
         size_t tc_need = 0;
-        int k = 0;
-        for (BatchClass &L : classes) {
-            L.tc_kind = 0;
-            if (tc_mode_available(mode) && L.N > kTileBits && tc_applies(L.N, 1, 2, sptr[k])) {
-                bool aligned = true;
-                for (int q = 0; q < L.S; ++q) aligned &= ((uintptr_t)sptr[k + q] & 15) == 0;
-                if (aligned) {
-                    L.tc_kind = mode == SRE_MODE_BF16_SPLIT ? 1 : 2;
-                    tc_need = std::max(tc_need, (size_t)L.S << (L.N - kTileBits));
-                }
-            }
-            k += L.S;
-        }
+        for (const BatchClass &L : classes)
+            if (L.tc_kind) tc_need = std::max(tc_need, (size_t)L.S << (L.N - kTileBits));
         const size_t tc0 = ctx->tc_e_cap + ctx->tc_bn_cap;
         if (tc_need && ((e = grow(&ctx->tc_e, &ctx->tc_e_cap, tc_need)) != cudaSuccess ||
                         (e = grow(&ctx->tc_bn, &ctx->tc_bn_cap, tc_need)) != cudaSuccess)) {

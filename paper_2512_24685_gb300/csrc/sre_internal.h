@@ -14,6 +14,7 @@ constexpr int kThreads = 256;              // threads per tile CTA
 constexpr int kPerThread = kTile / kThreads;  // 16 entries per thread (4 register bits)
 constexpr int kNormBlocks = 264;           // fixed grid of the norm reduction
 constexpr int kFinalThreads = 256;
+constexpr size_t kWorkBytes = 1024;               // work-queue counters of a workspace
 constexpr int kMaxRing = 64;                      // ring slots a tuned configuration may use
 constexpr size_t kTuneScratch = (size_t)192 << 20;  // scratch floor for N > 12 plans (tuned rings)
 constexpr size_t kSlotScratch = (size_t)96 << 20;   // scratch floor for server slots (default rings)
@@ -85,6 +86,12 @@ cudaError_t query_device(DeviceInfo *info);
 // shifts, x >= 4096).
 LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half);
 
+// The library's two-pass configuration for the main shift range of an
+// arithmetic mode (the halved shifts, or all shifts where sre_two.cu takes
+// them), and whether a configuration fits a workspace.
+LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode);
+bool main_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, sre_mode_t mode);
+
 // Tensor-core two-pass kernel (sre_tc.cu) for the halved shifts of one
 // state: tc_kind 1 = BF16 hi/lo pieces, 2 = FP16 hi/lo pieces.  tc_applies
 // says whether it covers (N, half, Renyi order, state alignment); the launch
@@ -133,8 +140,9 @@ struct BatchClass {
     int tc_kind = 0;                       // split modes: the halved shifts on the tensor cores
 };
 
+// tc_kind: the class takes the tensor-core kernel for its halved shifts.
 BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N, int S,
-                              sre_mode_t mode, const LargeCfg *tuned_half);
+                              sre_mode_t mode, const LargeCfg *tuned_half, int tc_kind);
 cudaError_t enqueue_batch_class(const Workspace &ws, const DeviceInfo &dev, const BatchClass &L,
                                 const void *const *d_ptrs, double *parts, unsigned *counters,
                                 size_t chunk_cap, sre_mode_t mode, cudaStream_t st,
@@ -175,11 +183,9 @@ cudaError_t evolve_tfim_step(void *d_states, void *d_buf, void *d_acc, int N, in
 // Bounded-wait self test (see sre_selftest_wait_timeout).
 cudaError_t run_wait_selftest(long long wait_ns, cudaStream_t st, int *status_out);
 
-// FP32 M2 of a complex64 state with given two-pass configurations for the
-// shifts below 4096 and the halved shifts; allocates nothing (the workspace
+// FP32 M2 of a complex64 state, N <= 16; allocates nothing (the workspace
 // pointers may point into preassigned memory).
-cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N,
-                             const LargeCfg &cfg_full, const LargeCfg &cfg_half, cudaStream_t st,
+cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N, cudaStream_t st,
                              double *d_m2, long long wait_ns);
 
 // Copy the result block to d_out2 = {S, n2} (for the range API).

@@ -32,6 +32,8 @@
 #include "sre_internal.h"
 #include "sre_large.cuh"
 #include "sre_tile.cuh"
+#include "sre_one.h"
+#include "sre_two.h"
 
 namespace sre {
 using namespace dev;
@@ -273,6 +275,16 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half
     return c;
 }
 
+LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode) {
+    const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
+    return mode == SRE_MODE_FP32 && two_applies(N, eb) ? choose_two_cfg(dev, ws, N) : choose_large_cfg(dev, N, eb, 1);
+}
+
+bool main_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, sre_mode_t mode) {
+    return mode == SRE_MODE_FP32 && two_applies(N, ws.elem_bytes) ? two_cfg_fits(ws, c, N)
+                                                                   : large_cfg_fits(ws, c, N, 1);
+}
+
 size_t workspace_scratch_bytes(const DeviceInfo &dev, int N_max, int elem_bytes, sre_mode_t mode) {
     (void)mode;
     if (N_max <= kTileBits) return 0;
@@ -322,7 +334,7 @@ cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int
     SRE_TRY(cudaMalloc(&ws->flags, sizeof(int)));
     ws->part_cap = kTile;  // one partial per tile of an N <= 12 state
     SRE_TRY(cudaMalloc(&ws->part, sizeof(double) * ws->part_cap));
-    SRE_TRY(cudaMalloc(&ws->work, sizeof(unsigned long long) * 2));
+    SRE_TRY(cudaMalloc(&ws->work, kWorkBytes));
     SRE_TRY(cudaMalloc(&ws->status, sizeof(int)));
     SRE_TRY(cudaMalloc(&ws->result, sizeof(Result)));
     if (N_max > kTileBits) {
@@ -448,6 +460,18 @@ static cudaError_t launch_large_h(const LargeArgs &a, int grid, cudaStream_t st)
 
 template <typename R, bool HALF>
 static cudaError_t launch_large(const LargeArgs &a, int grid, cudaStream_t st) {
+    if constexpr (sizeof(R) == 4) {
+        // smaller sizes: sre_one.cu and sre_two.cu
+        switch (a.h2) {
+            case 8: return HALF ? launch_large_h<R, 8, true>(a, grid, st) : cudaErrorInvalidValue;
+#define SRE_CASE(n) \
+    case n: return launch_large_h<R, n, HALF>(a, grid, st);
+            SRE_CASE(9) SRE_CASE(10) SRE_CASE(11)
+#undef SRE_CASE
+            case 12: return HALF ? cudaErrorInvalidValue : launch_large_h<R, 12, false>(a, grid, st);
+            default: return cudaErrorInvalidValue;
+        }
+    }
     switch (a.h2) {
 #define SRE_CASE(n) \
     case n: return launch_large_h<R, n, HALF>(a, grid, st);
@@ -544,9 +568,40 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         const uint64_t split = std::min<uint64_t>(std::max<uint64_t>(x_begin, kTile), x_end);
         if ((e = cudaMemsetAsync(ws.counters, 0, sizeof(unsigned) * 3 * ws.chunk_cap, st)) != cudaSuccess)
             return e;
-        if ((e = cudaMemsetAsync(ws.work, 0, sizeof(unsigned long long) * 2, st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;
         size_t chunks = 0;
-        for (int half = 0; half <= 1; ++half) {
+        // FP32, 13 <= N <= 20: one launch (sre_one.cu up to N = 16, sre_two.cu
+        // above) takes every shift, or with the tensor-core kernel on the
+        // halved ones the shifts below 4096
+        int first_half = 0;
+        if constexpr (sizeof(R) == 4) {
+            if (one_applies(N, eb) || two_applies(N, eb)) {
+                const bool all = !(tc_kind && tc_applies(N, 1, alpha, psi));
+                const uint64_t xe = all ? x_end : split;
+                first_half = all ? 2 : 1;
+                if (x_begin < xe) {
+                    const bool timed = xe == x_end;
+                    if (timed && ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
+                    if (one_applies(N, eb)) {
+                        chunks = (size_t)(xe - x_begin);
+                        if (chunks > ws.chunk_cap) return cudaErrorInvalidValue;
+                        e = launch_one(N, psi, nullptr, 1, x_begin, xe, alpha, ws.chunk_sum, d_per_x, ws.work + 2, ws.status,
+                                       wait_ns, dev, st);
+                    } else {
+                        const LargeCfg c = all && !tc_kind && cfg_override ? *cfg_override : choose_two_cfg(dev, ws, N);
+                        e = launch_two(ws, c, N, psi, nullptr, 1, x_begin, xe, alpha, ws.chunk_sum, ws.counters,
+                                       ws.chunk_cap, ws.chunk_cap, ws.work + 2, d_per_x, wait_ns, st);
+                        chunks = (size_t)two_layout(ws, c, N, x_begin, xe).n_chunks;
+                    }
+                    if (e != cudaSuccess) return e;
+                    if (timed && ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
+                    if (timed) ws.main_kernel = one_applies(N, eb) ? "k_one" : "k_two";
+                    ws.launches += 1;
+                    if (!all) seg1 = (long long)chunks;
+                }
+            }
+        }
+        for (int half = first_half; half <= 1; ++half) {
             const uint64_t xb = half ? split : x_begin;
             const uint64_t xe = half ? x_end : split;
             if (xb >= xe) continue;
@@ -556,11 +611,11 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
             const bool timed = half == 1 || split >= x_end;
             if (timed && !tc_here && ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess)
                 return e;
-            if (!tc_here && mid_applies(N, half, eb)) {
-                // one or two blocks per shift: single pass, one partial per shift
+            if (mid_applies(N, half, eb)) {
+                // FP64, one or two blocks per shift: single pass, one partial per shift
                 const long long ns = (long long)(xe - xb);
                 if (chunks + (size_t)ns > ws.chunk_cap) return cudaErrorInvalidValue;
-                if ((e = launch_mid<R>(N, half, psi, nullptr, 1, ns, xb, alpha, ws.chunk_sum + chunks,
+                if ((e = launch_mid<double>(N, half, psi, nullptr, 1, ns, xb, alpha, ws.chunk_sum + chunks,
                                        d_per_x ? d_per_x + (xb - x_begin) : nullptr, dev, st)) != cudaSuccess)
                     return e;
                 if (timed && ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
@@ -600,14 +655,9 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
     return cudaGetLastError();
 }
 
-// M2 of one complex64 state in FP32 with fixed two-pass configurations for
-// both shift ranges (no allocation, no autotuning): used by callers that
-// hand in preassigned scratch.  It shares the norm and finalize kernels
-// with the single-state path and, like it, takes the single-pass kernel for
-// the shift ranges of N = 13..15; larger N run the two-pass kernel with the
-// given fixed configuration (no autotuned plan).
-cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N,
-                             const LargeCfg &cfg_full, const LargeCfg &cfg_half, cudaStream_t st,
+// M2 of one complex64 state in FP32 for N <= 16 (no allocation): the
+// single-state path's kernels, on scratch that the caller hands in.
+cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N, cudaStream_t st,
                              double *d_m2, long long wait_ns) {
     using R = float;
     cudaError_t e;
@@ -617,47 +667,25 @@ cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const v
     k_norm<R><<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart,
                                                 ws.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    long long nparts = 0, seg1 = 0;
+    long long nparts = 0;
     const double *parts = nullptr;
     if (N <= kTileBits) {
         int np = 0;
         if ((e = launch_small<R>(N, psi, nullptr, 1, 0, d, ws.part, ws.part_cap, dev, st, &np)) != cudaSuccess)
             return e;
         parts = ws.part;
-        nparts = seg1 = np;
+        nparts = np;
     } else {
-        if ((e = cudaMemsetAsync(ws.counters, 0, sizeof(unsigned) * 3 * ws.chunk_cap, st)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(ws.work, 0, sizeof(unsigned long long) * 2, st)) != cudaSuccess) return e;
-        size_t chunks = 0;
-        for (int half = 0; half <= 1; ++half) {
-            const uint64_t xb = half ? (uint64_t)kTile : 0, xe = half ? d : (uint64_t)kTile;
-            if (mid_applies(N, half, 8)) {
-                // one, two or four blocks per shift: the single-pass kernel,
-                // one partial per shift, no ring and no waits
-                const long long ns = (long long)(xe - xb);
-                if (chunks + (size_t)ns > ws.chunk_cap) return cudaErrorInvalidValue;
-                if ((e = launch_mid<R>(N, half, psi, nullptr, 1, ns, xb, 2, ws.chunk_sum + chunks, nullptr, dev,
-                                       st)) != cudaSuccess)
-                    return e;
-                chunks += (size_t)ns;
-                if (!half) seg1 = (long long)chunks;
-                continue;
-            }
-            LargeArgs a;
-            int grid = 0;
-            if ((e = make_large_args(&a, ws, dev, psi, N, xb, xe, half, 8, chunks, nullptr, wait_ns,
-                                     half ? &cfg_half : &cfg_full, &grid)) != cudaSuccess)
-                return e;
-            e = half ? launch_large<R, true>(a, grid, st) : launch_large<R, false>(a, grid, st);
-            if (e != cudaSuccess) return e;
-            chunks += (size_t)a.n_chunks;
-            if (!half) seg1 = (long long)chunks;
-        }
+        if (!one_applies(N, 8) || d > ws.chunk_cap) return cudaErrorInvalidValue;
+        if ((e = cudaMemsetAsync(ws.work, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
+        if ((e = launch_one(N, psi, nullptr, 1, 0, d, 2, ws.chunk_sum, nullptr, ws.work, ws.status, wait_ns, dev,
+                            st)) != cudaSuccess)
+            return e;
         parts = ws.chunk_sum;
-        nparts = (long long)chunks;
+        nparts = (long long)d;
     }
-    k_finalize<<<1, 32, 0, st>>>(parts, 0, seg1, seg1, nparts - seg1, ws.npart, kNormBlocks, N, ws.flags,
-                                 ws.status, ws.result, d_m2, 2);
+    k_finalize<<<1, 32, 0, st>>>(parts, 0, nparts, nparts, 0, ws.npart, kNormBlocks, N, ws.flags, ws.status,
+                                 ws.result, d_m2, 2);
     return cudaGetLastError();
 }
 
@@ -779,8 +807,9 @@ static size_t small_grid_for(const DeviceInfo &dev, int N, int S) {
 }
 
 BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N, int S,
-                              sre_mode_t mode, const LargeCfg *tuned_half) {
+                              sre_mode_t mode, const LargeCfg *tuned_half, int tc_kind) {
     BatchClass L;
+    L.tc_kind = tc_kind;
     L.N = N;
     L.S = S;
     const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
@@ -789,6 +818,30 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         const long long tps = (long long)((((1ull << N) << N) + kTile - 1) >> kTileBits);
         L.cps_full = tps;  // tiles (= partials) per state
         L.parts_n = (size_t)S * (size_t)tps;
+        return L;
+    }
+    if (one_applies(N, eb)) {
+        // one partial per shift, all shifts or those below 4096 beside the
+        // tensor-core kernel
+        L.cfg_half = tuned_half ? *tuned_half : choose_large_cfg(dev, N, eb, 1);
+        L.cps_full = tc_kind ? (long long)kTile : 0;
+        L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)
+                             : 1ll << N;
+        L.parts_n = (size_t)S * (size_t)(L.cps_full + L.cps_half);
+        L.chunks_max = tc_kind ? (size_t)S * (size_t)L.cps_half : 1;
+        return L;
+    }
+    if (two_applies(N, eb)) {
+        // every shift in one launch, or the shifts below 4096 beside the
+        // tensor-core kernel
+        L.cfg_full = choose_two_cfg(dev, ws, N);
+        L.cfg_half = mode == SRE_MODE_FP32 && tuned_half ? *tuned_half : L.cfg_full;
+        if (tc_kind) L.cfg_half = tuned_half ? *tuned_half : choose_large_cfg(dev, N, eb, 1);
+        L.cps_full = tc_kind ? two_layout(ws, L.cfg_full, N, 0, kTile).n_chunks : 0;
+        L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)
+                             : two_layout(ws, L.cfg_half, N, 0, 1ull << N).n_chunks;
+        L.parts_n = (size_t)S * (size_t)(L.cps_full + L.cps_half);
+        L.chunks_max = (size_t)S * (size_t)std::max(L.cps_full, L.cps_half);
         return L;
     }
     L.cfg_full = choose_large_cfg(dev, N, eb, 0);
@@ -825,9 +878,33 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
         const LargeCfg &c = half ? L.cfg_half : L.cfg_full;
         const long long cps = half ? L.cps_half : L.cps_full;
         const uint64_t xb = half ? (uint64_t)kTile : 0, xe = half ? (1ull << N) : (uint64_t)kTile;
+        if constexpr (sizeof(R) == 4) {
+            if (one_applies(N, 8) && !(half && L.tc_kind)) {
+                if (cps == 0) continue;
+                if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;
+                if ((e = launch_one(N, nullptr, d_ptrs, L.S, 0, (uint64_t)cps, 2, parts + off, nullptr, ws.work + 2,
+                                    ws.status, wait_ns, dev, st)) != cudaSuccess)
+                    return e;
+                ws.launches += 1;
+                off += (size_t)cps * L.S;
+                continue;
+            }
+            if (two_applies(N, 8) && !(half && L.tc_kind)) {
+                if (cps == 0) continue;
+                if ((e = cudaMemsetAsync(counters, 0, sizeof(unsigned) * 3 * chunk_cap, st)) != cudaSuccess) return e;
+                if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;
+                if ((e = launch_two(ws, c, N, nullptr, d_ptrs, L.S, 0, half ? 1ull << N : (uint64_t)kTile, 2,
+                                    parts + off, counters, chunk_cap, chunk_cap, ws.work + 2, nullptr, wait_ns, st)) !=
+                    cudaSuccess)
+                    return e;
+                ws.launches += 1;
+                off += (size_t)cps * L.S;
+                continue;
+            }
+        }
         if (mid_applies(N, half, (int)sizeof(v2_t<R>))) {
             // cps = shifts per state (the layout gave this range one chunk per shift)
-            if ((e = launch_mid<R>(N, half, nullptr, d_ptrs, L.S, cps, xb, 2, parts + off, nullptr, dev, st)) !=
+            if ((e = launch_mid<double>(N, half, nullptr, d_ptrs, L.S, cps, xb, 2, parts + off, nullptr, dev, st)) !=
                 cudaSuccess)
                 return e;
             ws.launches += 1;

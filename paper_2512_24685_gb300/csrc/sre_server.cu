@@ -390,8 +390,7 @@ sre_status_t sre_server_create(const sre_server_cfg_t *cfg, sre_server_t *out) {
 
 sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t) {
     if (!s || !t || N <= sre::kTileBits || N > s->cfg.max_N) return SRE_EINVAL;
-    const int eb = s->cfg.mode == SRE_MODE_FP64 ? 16 : 8;
-    sre::LargeCfg c = sre::choose_large_cfg(s->dev, N, eb, 1);
+    sre::LargeCfg c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode);
     if (t->x_batch_log >= 0) c.C_log = t->x_batch_log;
     if (t->ring_slots >= 0) c.R = t->ring_slots;
     if (t->lag >= 0) c.D = t->lag;
@@ -403,7 +402,7 @@ sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t)
     c.B1_log = std::min(c.B1_log, N - sre::kTileBits - 1);
     std::lock_guard<std::mutex> lk(s->mu);
     for (const Slot &sl : s->slots)
-        if (!sre::large_cfg_fits(sl.ws, c, N, 1)) return SRE_EINVAL;
+        if (!sre::main_cfg_fits(sl.ws, c, N, s->cfg.mode)) return SRE_EINVAL;
     s->tuned[N] = c;
     s->has_tuned[N] = true;
     return SRE_OK;
