@@ -299,7 +299,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
     if (!p || N < 1 || N > p->N) return SRE_EINVAL;
     if (N <= sre::kTileBits) return SRE_OK;
     // N <= 15 in FP32 and N <= 14 in FP64 run in a single pass: nothing to tune
-    if (sre::mid_applies(N, 1, elem_bytes_for_mode(p->mode)) ||
+    if (sre::mid_applies(N, elem_bytes_for_mode(p->mode)) ||
         (p->mode == SRE_MODE_FP32 && N < 16 && sre::one_applies(N, 8)))
         return SRE_OK;
     cudaStream_t st = (cudaStream_t)stream;

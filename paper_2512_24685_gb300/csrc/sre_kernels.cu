@@ -8,17 +8,13 @@
 // Kernels
 //   k_convert   element-type conversion of the state (complex128 <-> complex64)
 //   k_norm      n2 = <psi|psi> in FP64 + NaN/Inf detection (fixed grid)
-//   k_small     N <= 12: one 2^12-entry tile holds 2^(12-N) whole shifts; the
-//               state sits in shared memory; static tile->CTA assignment
-//   k_large     N  > 12: persistent two-pass kernel.  Pass 1 (one work item
-//               per chunk of C shifts and high index block t_h) forms the
-//               products of a 2^12 block, transforms its 12 low bits and
-//               writes the block to an L2-sized ring of scratch; pass 2 (work
-//               items of whole-z-block tiles) gathers the 2^(N-12) blocks of
-//               a z-range, transforms the high bits and reduces |A|^4.  Items
-//               are claimed in order from one counter; pass 2 of a chunk waits
-//               (bounded, %globaltimer) for its pass-1 items, and pass 1 of a
-//               chunk waits for the ring slot to be released.
+//   k_small     N <= 12, FP32: one 2^12-entry tile holds 2^(13-N) whole shifts
+//               (halved form); the state sits in shared memory; static
+//               tile->CTA assignment.  k_small_fx: the same in fixed point
+//   k_fx_*      fixed point: unit exponents of a state, block or shift
+//   k_large     fixed point N >= 15, FP32 N >= 21: persistent two-pass kernel
+//               (sre_large.cuh); the sizes between run in sre_mid.cu,
+//               sre_one.cu and sre_two.cu
 //   k_finalize  fixed-order FP64 sums of the partials, M2 and the status.
 // Every reduction has a fixed order, so results are bitwise reproducible and
 // do not depend on what else runs on the device.
@@ -28,6 +24,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "sre_internal.h"
 #include "sre_large.cuh"
@@ -53,8 +50,8 @@ __global__ void k_convert(const In *__restrict__ src, Out *__restrict__ dst, uin
 }
 
 // n2 = sum_t |phi_t|^2 (FP64), per-block partials in a fixed grid.
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_norm(const v2_t<R> *__restrict__ psi, uint64_t d,
+template <typename V>
+__global__ void __launch_bounds__(kThreads) k_norm(const V *__restrict__ psi, uint64_t d,
                                                    double *__restrict__ npart,
                                                    int *__restrict__ flags) {
     __shared__ double red[kThreads / 32];
@@ -62,7 +59,7 @@ __global__ void __launch_bounds__(kThreads) k_norm(const v2_t<R> *__restrict__ p
     int bad = 0;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < d;
          t += (uint64_t)gridDim.x * blockDim.x) {
-        const v2_t<R> v = psi[t];
+        const V v = psi[t];
         const double re = (double)v.x, im = (double)v.y;
         if (!isfinite(re) || !isfinite(im)) bad = 1;
         s += re * re + im * im;
@@ -72,11 +69,76 @@ __global__ void __launch_bounds__(kThreads) k_norm(const v2_t<R> *__restrict__ p
     if (threadIdx.x == 0) npart[blockIdx.x] = b;
 }
 
+// Bounds (256 log2) of n entries by one CTA: largest |phi|^2 and squared l2 norm
+// (in thread 0).
+__device__ int2 fx_norm_max(const double2 *__restrict__ p, int n) {
+    __shared__ double red[kThreads / 32], mx[kThreads / 32];
+    double s = 0.0, m = 0.0;
+    for (int t = threadIdx.x; t < n; t += kThreads) {
+        const double2 v = p[t];
+        const double q = v.x * v.x + v.y * v.y;
+        s += q;
+        m = fmax(m, q);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) mx[threadIdx.x >> 5] = m;
+    s = block_sum(s, red);  // its barriers also order mx
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kThreads / 32; ++w) m = fmax(m, mx[w]);
+    return make_int2(fx_log(m), fx_log(s));
+}
+
+// N <= 12, one CTA per state: the unit exponents of the FP64 mode.
+__global__ void __launch_bounds__(kThreads) k_fx_exponent(const double2 *__restrict__ psi, const void *const *psis,
+                                                          const int *__restrict__ Ns, int N,
+                                                          FxUnits *__restrict__ units) {
+    const int n = Ns ? Ns[blockIdx.x] : N;
+    if (n > kTileBits) return;
+    const int2 b = fx_norm_max(psis ? reinterpret_cast<const double2 *>(psis[blockIdx.x]) : psi, 1 << n);
+    if (threadIdx.x == 0) units[blockIdx.x] = fx_units(b, kFxNonFinite);
+}
+
+// N > 12: bounds of every 4096-entry block (blockIdx.y: state).
+__global__ void __launch_bounds__(kThreads) k_fx_block_norms(const double2 *__restrict__ psi,
+                                                             const void *const *psis, int2 *__restrict__ bn) {
+    const double2 *base = psis ? reinterpret_cast<const double2 *>(psis[blockIdx.y]) : psi;
+    const int2 b = fx_norm_max(base + ((size_t)blockIdx.x << kTileBits), kTile);
+    if (threadIdx.x == 0) bn[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = b;
+}
+
+// Unit exponent per x_h = x >> 12: one warp sums the bounds of the shift's blocks.
+__global__ void k_fx_scales(const int2 *__restrict__ bn_all, int nb, int *__restrict__ e_all) {
+    const int xh = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (xh >= nb) return;
+    const int2 *bn = bn_all + (size_t)blockIdx.y * nb;
+    double s = 0.0;
+    for (int tp = lane; tp < nb / 2; tp += 32) {
+        const int l = fx_bound(bn, nb, (uint64_t)xh << kTileBits, tp).y;
+        s += l >= kFxNonFinite / 2 ? __longlong_as_double(0x7ff0000000000000ll) : exp2((double)l / 256.0);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) e_all[(size_t)blockIdx.y * nb + xh] = fx_exponent(fx_log(s));
+}
+
+cudaError_t enqueue_fx_scales(const void *psi, const void *const *psis, int nstates, int N, int2 *bn, int *e,
+                              cudaStream_t st) {
+    const int nb = 1 << (N - kTileBits);
+    k_fx_block_norms<<<dim3(nb, (unsigned)nstates), kThreads, 0, st>>>(reinterpret_cast<const double2 *>(psi), psis,
+                                                                       bn);
+    cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    k_fx_scales<<<dim3((nb + 7) / 8, (unsigned)nstates), 256, 0, st>>>(bn, nb, e);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------- N <= 12: k_small
 
-// Tile g covers flat indices [g*4096, (g+1)*4096) of the (x - x_begin, t)
-// space: x = x_begin + (flat >> N), t = flat & (d - 1).  The transform runs
-// over the low NB = N bits of the tile index.
+// Tile g covers flat indices [g*4096, (g+1)*4096) of the (x - x_begin, t')
+// space: x = x_begin + (flat >> NB), t' = flat & (2^NB - 1), NB = N - 1: every
+// shift in the halved form, t' being t without the pivot bit (the highest set
+// bit of x; x = 0 pairs the two halves of g_0).
 template <typename R, int NB>
 __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ psi,
                                                     const void *const *__restrict__ psis,
@@ -94,10 +156,11 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
     V *bufA = psi_s + kTileSlots;
     V *bufB = bufA + kTileSlots;
     __shared__ double red[kThreads / 32];
-    constexpr int N = NB;
+    constexpr int N = NB + 1;
     constexpr int d = 1 << N;
     const int tid = threadIdx.x;
 
+    const double hfac = half_factor<R>(alpha, 0);
     long long cur = -1;
     for (long long g = blockIdx.x; g < ntiles; g += gridDim.x) {
         const long long sidx = psis ? g / tiles_per_state : 0;
@@ -113,19 +176,65 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const uint64_t flat = ((uint64_t)gl << kTileBits) | (uint64_t)elem<0>(tid, i);
-            const uint64_t x = x_begin + (flat >> N);
-            const int t = (int)(flat & (d - 1));
+            const uint64_t x = x_begin + (flat >> NB);
             if (x < x_end) {
-                const V a = psi_s[pad(t)];
-                const V b = psi_s[pad(t ^ (int)x)];
-                v[i] = conj_mul<R>(b.x, b.y, a.x, a.y);  // conj(phi_{t^x}) * phi_t
+                const int xe = x ? (int)x : d >> 1;
+                const int lo = (int)(flat & ((1u << NB) - 1)) & ((1 << (31 - __clz(xe))) - 1);
+                const int t = (((int)(flat & ((1u << NB) - 1)) - lo) << 1) | lo;
+                v[i] = x ? pair_value<R, false>(psi_s[pad(t ^ xe)], psi_s[pad(t)], 0)
+                         : pair_value<R, true>(psi_s[pad(t ^ xe)], psi_s[pad(t)], 0);
             } else {
                 v[i] = Cx<R>::zero();
             }
         }
         tile_fwht<NB, R>(v, bufA, bufB, tid);
         // block_sum's barriers also protect bufB before the next tile
-        const double s = block_sum((double)sum_order<R, false>(v, alpha), red);
+        const double s = block_sum(hfac * (double)sum_order<R>(v, alpha), red);
+        if (tid == 0) part[g] = s;
+    }
+}
+
+// The same in the fixed-point mode: factors straight from global memory (the
+// state stays in L1), bits 8-11 first, one move buffer, so that two CTAs fit
+// an SM.
+template <int NB>
+__global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restrict__ psi0,
+                                                          const void *const *__restrict__ psis,
+                                                          long long tiles_per_state, uint64_t x_begin, uint64_t x_end,
+                                                          long long ntiles, double *__restrict__ part, int alpha,
+                                                          const FxUnits *__restrict__ units) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double2 *buf = reinterpret_cast<double2 *>(smem_raw);
+    __shared__ double red[kThreads / 32];
+    constexpr int d = 2 << NB;
+    const int tid = threadIdx.x;
+    for (long long g = blockIdx.x; g < ntiles; g += gridDim.x) {
+        const long long sidx = psis ? g / tiles_per_state : 0;
+        const long long gl = g - sidx * tiles_per_state;
+        const double2 *psi = psis ? reinterpret_cast<const double2 *>(psis[sidx]) : psi0;
+        const FxUnits un = units[sidx];
+        cx_t<fx> v[16];
+        auto value = [&](int i, auto with_zero) {
+            const uint64_t flat = ((uint64_t)gl << kTileBits) | (uint64_t)elem<2>(tid, i);
+            const uint64_t x = x_begin + (flat >> NB);
+            if (x >= x_end) return Cx<fx>::zero();
+            const int xe = x ? (int)x : d >> 1, tt = (int)(flat & ((1u << NB) - 1));
+            const int lo = tt & ((1 << (31 - __clz(xe))) - 1), t = ((tt - lo) << 1) | lo;
+            const double2 b = __ldg(psi + (t ^ xe)), a = __ldg(psi + t);
+            if constexpr (decltype(with_zero)::value)
+                if (!x) return pair_value<fx, true>(b, a, un.a);
+            return pair_value<fx, false>(b, a, un.a);
+        };
+        // the first tile alone holds x = 0
+        if (gl == 0 && x_begin == 0) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = value(i, std::true_type());
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = value(i, std::false_type());
+        }
+        fx_tile<NB>(v, buf, tid, un);
+        const double s = block_sum(half_factor<fx>(alpha, un.c) * sum_order<fx>(v, alpha), red);
         if (tid == 0) part[g] = s;
     }
 }
@@ -207,8 +316,6 @@ cudaError_t query_device(DeviceInfo *info) {
                                   info->device);
 }
 
-static size_t tile_smem_bytes(int elem_bytes) { return (size_t)3 * kTileSlots * elem_bytes; }
-
 // deterministic pseudo-random amplitudes for timing runs (values irrelevant)
 template <typename V>
 __global__ void k_fill_synthetic(V *p, uint64_t n) {
@@ -256,8 +363,7 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half
     const int h2 = N - kTileBits - half;
     const double per_x = (double)elem_bytes * (double)(1ull << (N - half));
     const double budget = std::max(24.0 * (1 << 20), 0.6 * (double)dev.l2_bytes);
-    const int occ = elem_bytes == 8 ? 2 : 1;
-    c.grid = std::max(1, dev.sms * occ);
+    c.grid = std::max(1, dev.sms * 2);
     const int P1 = 1 << h2;
     const int inflight = (c.grid + P1 - 1) / P1;
     c.D = std::min(inflight + 1, kMaxRing / 2 - 1);
@@ -312,6 +418,7 @@ void workspace_free(Workspace *ws) {
     cudaFree(ws->conv);
     cudaFree(ws->tc_e);
     cudaFree(ws->tc_bn);
+    cudaFree(ws->fx_k);
     *ws = Workspace();
 }
 
@@ -336,6 +443,7 @@ cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int
     SRE_TRY(cudaMalloc(&ws->part, sizeof(double) * ws->part_cap));
     SRE_TRY(cudaMalloc(&ws->work, kWorkBytes));
     SRE_TRY(cudaMalloc(&ws->status, sizeof(int)));
+    SRE_TRY(cudaMalloc(&ws->fx_k, sizeof(FxUnits)));
     SRE_TRY(cudaMalloc(&ws->result, sizeof(Result)));
     if (N_max > kTileBits) {
         // sizes for every N up to N_max and both halves of the shift range,
@@ -372,21 +480,28 @@ template <typename R, int NB>
 static cudaError_t launch_small_nb(const void *psi, const void *const *psis, int nstates,
                                    uint64_t x_begin, uint64_t x_end, double *part, int part_cap,
                                    const DeviceInfo &dev, cudaStream_t st, int *nparts,
-                                   int forced_grid = 0, int alpha = 2) {
-    const size_t smem = tile_smem_bytes(sizeof(v2_t<R>));
-    auto kern = k_small<R, NB>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                   int forced_grid, int alpha, const int *fx_k) {
+    constexpr bool kFx = sizeof(cx_t<R>) == 16;
+    const size_t smem = (size_t)(kFx ? 1 : 3) * kTileSlots * sizeof(v2_t<R>);
+    cudaError_t e;
+    if constexpr (kFx)
+        e = cudaFuncSetAttribute(k_small_fx<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    else
+        e = cudaFuncSetAttribute(k_small<R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const uint64_t flat = (x_end - x_begin) << NB;
     const long long tps = (long long)((flat + kTile - 1) >> kTileBits);
     const long long ntiles = tps * nstates;
     if (ntiles > part_cap) return cudaErrorInvalidValue;
-    const int occ = sizeof(R) == 4 ? 2 : 1;
     const int grid = forced_grid > 0 ? forced_grid
-                                     : (int)std::min<long long>(ntiles, (long long)dev.sms * occ);
+                                     : (int)std::min<long long>(ntiles, (long long)dev.sms * 2);
     if (grid < 1) return cudaErrorInvalidValue;
-    kern<<<grid, kThreads, smem, st>>>(reinterpret_cast<const v2_t<R> *>(psi), psis, tps, x_begin,
-                                       x_end, ntiles, part, alpha);
+    if constexpr (kFx)
+        k_small_fx<NB><<<grid, kThreads, smem, st>>>(reinterpret_cast<const double2 *>(psi), psis, tps, x_begin, x_end,
+                                                     ntiles, part, alpha, reinterpret_cast<const FxUnits *>(fx_k));
+    else
+        k_small<R, NB><<<grid, kThreads, smem, st>>>(reinterpret_cast<const float2 *>(psi), psis, tps, x_begin, x_end,
+                                                     ntiles, part, alpha);
     *nparts = (int)ntiles;
     return cudaGetLastError();
 }
@@ -395,10 +510,10 @@ template <typename R>
 static cudaError_t launch_small(int N, const void *psi, const void *const *psis, int nstates,
                                 uint64_t xb, uint64_t xe, double *part, int part_cap,
                                 const DeviceInfo &dev, cudaStream_t st, int *nparts,
-                                int forced_grid = 0, int alpha = 2) {
+                                int forced_grid, int alpha, const int *fx_k) {
     switch (N) {
 #define SRE_CASE(n) \
-    case n: return launch_small_nb<R, n>(psi, psis, nstates, xb, xe, part, part_cap, dev, st, nparts, forced_grid, alpha);
+    case n: return launch_small_nb<R, n - 1>(psi, psis, nstates, xb, xe, part, part_cap, dev, st, nparts, forced_grid, alpha, fx_k);
         SRE_CASE(1) SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6)
         SRE_CASE(7) SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11) SRE_CASE(12)
 #undef SRE_CASE
@@ -429,7 +544,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 cudaError_t encode_p2_tmap(LargeArgs &a) {
     auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
-    if (a.h2 < 5 || a.h2 > 8 || ((uintptr_t)a.scratch & 15)) return cudaErrorInvalidValue;
+    if (a.h2 != 8 || ((uintptr_t)a.scratch & 15)) return cudaErrorInvalidValue;
     const cuuint64_t rows = (cuuint64_t)a.R << (a.C_log + a.h2);
     if (rows > 0xFFFFFFFFull) return cudaErrorInvalidValue;
     const cuuint64_t dims[2] = {2ull * kTile, rows};
@@ -442,10 +557,10 @@ cudaError_t encode_p2_tmap(LargeArgs &a) {
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <typename R, int H2, bool HALF>
+template <typename R, int H2>
 static cudaError_t launch_large_h(const LargeArgs &a, int grid, cudaStream_t st) {
     const size_t smem = large_smem_bytes<R, H2>();
-    auto kern = k_large<R, H2, HALF>;
+    auto kern = k_large<R, H2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if constexpr (large_uses_tma<R, H2>()) {
@@ -458,28 +573,21 @@ static cudaError_t launch_large_h(const LargeArgs &a, int grid, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <typename R, bool HALF>
+// FP32: N >= 21 (smaller sizes run in sre_one.cu and sre_two.cu); fixed point:
+// N >= 15.
+template <typename R>
 static cudaError_t launch_large(const LargeArgs &a, int grid, cudaStream_t st) {
-    if constexpr (sizeof(R) == 4) {
-        // smaller sizes: sre_one.cu and sre_two.cu
-        switch (a.h2) {
-            case 8: return HALF ? launch_large_h<R, 8, true>(a, grid, st) : cudaErrorInvalidValue;
-#define SRE_CASE(n) \
-    case n: return launch_large_h<R, n, HALF>(a, grid, st);
-            SRE_CASE(9) SRE_CASE(10) SRE_CASE(11)
-#undef SRE_CASE
-            case 12: return HALF ? cudaErrorInvalidValue : launch_large_h<R, 12, false>(a, grid, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
     switch (a.h2) {
 #define SRE_CASE(n) \
-    case n: return launch_large_h<R, n, HALF>(a, grid, st);
-        SRE_CASE(0) SRE_CASE(1) SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6)
-        SRE_CASE(7) SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11) SRE_CASE(12)
+    case n: return launch_large_h<R, n>(a, grid, st);
+        SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11)
 #undef SRE_CASE
-        default: return cudaErrorInvalidValue;
+#define SRE_CASE(n) \
+    case n: if constexpr (sizeof(cx_t<R>) == 16) return launch_large_h<R, n>(a, grid, st); break;
+        SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6) SRE_CASE(7)
+#undef SRE_CASE
     }
+    return cudaErrorInvalidValue;
 }
 
 // Fill LargeArgs for the shift range [xb, xe) (all of it halved or not).
@@ -492,6 +600,8 @@ static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const Devi
     A.psi = psi;
     A.psis = nullptr;
     A.chunks_per_state = 0;
+    A.fx_bn = reinterpret_cast<const int2 *>(ws.tc_bn);
+    A.tc_e = ws.tc_e;
     A.N = N;
     A.half = half;
     A.h2 = N - kTileBits - half;
@@ -540,112 +650,96 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                                 double *d_per_x, long long wait_ns, LargeCfg *cfg_override,
                                 int tc_kind, int alpha) {
     cudaError_t e;
+    constexpr bool kFx = sizeof(cx_t<R>) == 16;
     const uint64_t d = 1ull << N;
     if ((e = cudaMemsetAsync(ws.flags, 0, sizeof(int), st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(ws.status, 0, sizeof(int), st)) != cudaSuccess) return e;
-    k_norm<R><<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart,
-                                                ws.flags);
+    k_norm<<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart, ws.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ws.launches += 2;  // k_norm + k_finalize
+    if constexpr (kFx) {
+        if (N <= kTileBits) {
+            k_fx_exponent<<<1, kThreads, 0, st>>>(reinterpret_cast<const double2 *>(psi), nullptr, nullptr, N,
+                                                  reinterpret_cast<FxUnits *>(ws.fx_k));
+            e = cudaGetLastError();
+        } else {
+            e = enqueue_fx_scales(psi, nullptr, 1, N, reinterpret_cast<int2 *>(ws.tc_bn), ws.tc_e, st);
+        }
+        if (e != cudaSuccess) return e;
+        ws.launches += N <= kTileBits ? 1 : 2;
+    }
     const double *parts = nullptr;
-    long long nparts = 0, seg1 = 0;  // large path: [0, seg1) full shifts, [seg1, nparts) halved
+    long long nparts = 0, seg1 = 0;  // [0, seg1) shifts below 4096 beside the tensor-core kernel's [seg1, nparts)
     if (N <= kTileBits) {
         int np = 0;
         if (ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
         if ((e = launch_small<R>(N, psi, nullptr, 1, x_begin, x_end, ws.part, ws.part_cap, dev, st,
-                                 &np, 0, alpha)) != cudaSuccess)
+                                 &np, 0, alpha, kFx ? ws.fx_k : nullptr)) != cudaSuccess)
             return e;
         if (ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
         ws.main_kernel = "k_small";
         ws.launches += 1;
         parts = ws.part;
         nparts = np;
-        seg1 = np;
     } else {
-        // shifts below 4096 (pivot bit inside the 12-bit block): full
-        // transform; shifts from 4096 up: conjugate-symmetry halving
         const int eb = (int)sizeof(v2_t<R>);
-        const uint64_t split = std::min<uint64_t>(std::max<uint64_t>(x_begin, kTile), x_end);
         if ((e = cudaMemsetAsync(ws.counters, 0, sizeof(unsigned) * 3 * ws.chunk_cap, st)) != cudaSuccess)
             return e;
         if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;
+        // every shift in one launch, or with the tensor-core kernel on the
+        // shifts from 4096 up those below it
+        const bool tc = tc_kind && tc_applies(N, 1, alpha, psi);
+        const uint64_t split = tc ? std::min<uint64_t>(std::max<uint64_t>(x_begin, kTile), x_end) : x_end;
         size_t chunks = 0;
-        // FP32, 13 <= N <= 20: one launch (sre_one.cu up to N = 16, sre_two.cu
-        // above) takes every shift, or with the tensor-core kernel on the
-        // halved ones the shifts below 4096
-        int first_half = 0;
-        if constexpr (sizeof(R) == 4) {
-            if (one_applies(N, eb) || two_applies(N, eb)) {
-                const bool all = !(tc_kind && tc_applies(N, 1, alpha, psi));
-                const uint64_t xe = all ? x_end : split;
-                first_half = all ? 2 : 1;
-                if (x_begin < xe) {
-                    const bool timed = xe == x_end;
-                    if (timed && ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
-                    if (one_applies(N, eb)) {
-                        chunks = (size_t)(xe - x_begin);
-                        if (chunks > ws.chunk_cap) return cudaErrorInvalidValue;
-                        e = launch_one(N, psi, nullptr, 1, x_begin, xe, alpha, ws.chunk_sum, d_per_x, ws.work + 2, ws.status,
-                                       wait_ns, dev, st);
-                    } else {
-                        const LargeCfg c = all && !tc_kind && cfg_override ? *cfg_override : choose_two_cfg(dev, ws, N);
-                        e = launch_two(ws, c, N, psi, nullptr, 1, x_begin, xe, alpha, ws.chunk_sum, ws.counters,
-                                       ws.chunk_cap, ws.chunk_cap, ws.work + 2, d_per_x, wait_ns, st);
-                        chunks = (size_t)two_layout(ws, c, N, x_begin, xe).n_chunks;
-                    }
-                    if (e != cudaSuccess) return e;
-                    if (timed && ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
-                    if (timed) ws.main_kernel = one_applies(N, eb) ? "k_one" : "k_two";
-                    ws.launches += 1;
-                    if (!all) seg1 = (long long)chunks;
-                }
-            }
-        }
-        for (int half = first_half; half <= 1; ++half) {
-            const uint64_t xb = half ? split : x_begin;
-            const uint64_t xe = half ? x_end : split;
-            if (xb >= xe) continue;
-            const bool tc_here = tc_kind && tc_applies(N, half, alpha, psi);
-            // the profiling events bracket the dominant launch: the halved
-            // shifts, or the full-transform range when there are none
-            const bool timed = half == 1 || split >= x_end;
-            if (timed && !tc_here && ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess)
-                return e;
-            if (mid_applies(N, half, eb)) {
-                // FP64, one or two blocks per shift: single pass, one partial per shift
-                const long long ns = (long long)(xe - xb);
-                if (chunks + (size_t)ns > ws.chunk_cap) return cudaErrorInvalidValue;
-                if ((e = launch_mid<double>(N, half, psi, nullptr, 1, ns, xb, alpha, ws.chunk_sum + chunks,
-                                       d_per_x ? d_per_x + (xb - x_begin) : nullptr, dev, st)) != cudaSuccess)
+        if (x_begin < split) {
+            const bool timed = split == x_end;
+            if (timed && ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
+            const char *name;
+            if (one_applies(N, eb) || mid_applies(N, eb)) {
+                // a shift in one CTA, one partial per shift
+                name = kFx ? "k_mid" : "k_one";
+                chunks = (size_t)(split - x_begin);
+                if (chunks > ws.chunk_cap) return cudaErrorInvalidValue;
+                if constexpr (kFx)
+                    e = launch_mid(N, psi, nullptr, 1, (long long)chunks, x_begin, alpha, ws.chunk_sum, d_per_x,
+                                   reinterpret_cast<const int2 *>(ws.tc_bn), ws.tc_e, dev, st);
+                else
+                    e = launch_one(N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, d_per_x, ws.work + 2,
+                                   ws.status, wait_ns, dev, st);
+            } else if (two_applies(N, eb)) {
+                name = "k_two";
+                const LargeCfg c = !tc_kind && cfg_override ? *cfg_override : choose_two_cfg(dev, ws, N);
+                e = launch_two(ws, c, N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, ws.counters,
+                               ws.chunk_cap, ws.chunk_cap, ws.work + 2, d_per_x, wait_ns, st);
+                chunks = (size_t)two_layout(ws, c, N, x_begin, split).n_chunks;
+            } else {
+                name = "k_large";
+                LargeArgs a;
+                int grid = 0;
+                if ((e = make_large_args(&a, ws, dev, psi, N, x_begin, split, 1, eb, 0, d_per_x, wait_ns,
+                                         cfg_override, &grid)) != cudaSuccess)
                     return e;
-                if (timed && ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
-                if (timed) ws.main_kernel = "k_mid";
-                ws.launches += 1;
-                chunks += (size_t)ns;
-                if (!half) seg1 = (long long)chunks;
-                continue;
+                a.alpha = alpha;
+                e = launch_large<R>(a, grid, st);
+                chunks = (size_t)a.n_chunks;
             }
+            if (e != cudaSuccess) return e;
+            if (timed && ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
+            if (timed) ws.main_kernel = name;
+            ws.launches += 1;
+            if (tc) seg1 = (long long)chunks;
+        }
+        if (tc && split < x_end) {
             LargeArgs a;
             int grid = 0;
-            if ((e = make_large_args(&a, ws, dev, psi, N, xb, xe, half, eb, chunks,
-                                     d_per_x ? d_per_x + (xb - x_begin) : nullptr, wait_ns,
-                                     cfg_override && half ? cfg_override : nullptr, &grid)) != cudaSuccess)
+            if ((e = make_large_args(&a, ws, dev, psi, N, split, x_end, 1, eb, chunks,
+                                     d_per_x ? d_per_x + (split - x_begin) : nullptr, wait_ns, cfg_override,
+                                     &grid)) != cudaSuccess)
                 return e;
             a.alpha = alpha;
-            if (tc_here)
-                e = launch_large_tc(a, ws, dev, grid, st, tc_kind);
-            else if (half)
-                e = launch_large<R, true>(a, grid, st);
-            else
-                e = launch_large<R, false>(a, grid, st);
-            if (e != cudaSuccess) return e;
-            if (timed && !tc_here) {
-                if (ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
-                ws.main_kernel = "k_large";
-            }
+            if ((e = launch_large_tc(a, ws, dev, grid, st, tc_kind)) != cudaSuccess) return e;
             ws.launches += 1;
             chunks += (size_t)a.n_chunks;
-            if (!half) seg1 = (long long)chunks;
         }
         parts = ws.chunk_sum;
         nparts = (long long)chunks;
@@ -664,14 +758,14 @@ cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const v
     const uint64_t d = 1ull << N;
     if ((e = cudaMemsetAsync(ws.flags, 0, sizeof(int), st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(ws.status, 0, sizeof(int), st)) != cudaSuccess) return e;
-    k_norm<R><<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart,
-                                                ws.flags);
+    k_norm<<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart, ws.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     long long nparts = 0;
     const double *parts = nullptr;
     if (N <= kTileBits) {
         int np = 0;
-        if ((e = launch_small<R>(N, psi, nullptr, 1, 0, d, ws.part, ws.part_cap, dev, st, &np)) != cudaSuccess)
+        if ((e = launch_small<R>(N, psi, nullptr, 1, 0, d, ws.part, ws.part_cap, dev, st, &np, 0, 2,
+                                 nullptr)) != cudaSuccess)
             return e;
         parts = ws.part;
         nparts = np;
@@ -714,7 +808,7 @@ cudaError_t enqueue_m2(const Workspace &ws, const DeviceInfo &dev, const void *d
     }
     const int tc_kind = mode == SRE_MODE_BF16_SPLIT ? 1 : mode == SRE_MODE_FP16_SPLIT ? 2 : 0;
     if (fp64)
-        return enqueue_m2_t<double>(ws, dev, psi, N, x_begin, x_end, stream, d_m2, d_per_x, wait_ns,
+        return enqueue_m2_t<fx>(ws, dev, psi, N, x_begin, x_end, stream, d_m2, d_per_x, wait_ns,
                                     cfg_override, 0, alpha);
     return enqueue_m2_t<float>(ws, dev, psi, N, x_begin, x_end, stream, d_m2, d_per_x, wait_ns,
                                cfg_override, tc_kind, alpha);
@@ -800,10 +894,9 @@ __global__ void k_finalize_batch(const longlong4 *__restrict__ seg, const double
 
 template <typename R>
 static size_t small_grid_for(const DeviceInfo &dev, int N, int S) {
-    const uint64_t flat = (1ull << N) << N;
+    const uint64_t flat = (1ull << N) << (N - 1);
     const long long tps = (long long)((flat + kTile - 1) >> kTileBits);
-    const int occ = sizeof(R) == 4 ? 2 : 1;
-    return (size_t)std::min<long long>(tps * S, (long long)dev.sms * occ);
+    return (size_t)std::min<long long>(tps * S, (long long)dev.sms * 2);
 }
 
 BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N, int S,
@@ -814,8 +907,8 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
     L.S = S;
     const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
     if (N <= kTileBits) {
-        L.small_grid = (int)(eb == 8 ? small_grid_for<float>(dev, N, S) : small_grid_for<double>(dev, N, S));
-        const long long tps = (long long)((((1ull << N) << N) + kTile - 1) >> kTileBits);
+        L.small_grid = (int)(eb == 8 ? small_grid_for<float>(dev, N, S) : small_grid_for<fx>(dev, N, S));
+        const long long tps = (long long)((((1ull << N) << (N - 1)) + kTile - 1) >> kTileBits);
         L.cps_full = tps;  // tiles (= partials) per state
         L.parts_n = (size_t)S * (size_t)tps;
         return L;
@@ -844,16 +937,12 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         L.chunks_max = (size_t)S * (size_t)std::max(L.cps_full, L.cps_half);
         return L;
     }
-    L.cfg_full = choose_large_cfg(dev, N, eb, 0);
     L.cfg_half = tuned_half ? *tuned_half : choose_large_cfg(dev, N, eb, 1);
-    // ranges taken by the single-pass kernel have one partial per shift
-    if (mid_applies(N, 0, eb)) L.cfg_full.C_log = 0;
-    if (mid_applies(N, 1, eb)) L.cfg_half.C_log = 0;
-    L.cps_full = (long long)(((uint64_t)kTile + (1ull << L.cfg_full.C_log) - 1) >> L.cfg_full.C_log);
-    const uint64_t span = (1ull << N) - kTile;
-    L.cps_half = (long long)((span + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log);
-    L.parts_n = (size_t)S * (size_t)(L.cps_full + L.cps_half);
-    L.chunks_max = (size_t)S * (size_t)std::max(L.cps_full, L.cps_half);
+    // the single-pass kernel has one partial per shift
+    if (mid_applies(N, eb)) L.cfg_half.C_log = 0;
+    L.cps_full = 0;
+    L.cps_half = 1ll << (N - L.cfg_half.C_log);
+    L.parts_n = L.chunks_max = (size_t)S * (size_t)L.cps_half;
     (void)ws;
     return L;
 }
@@ -863,22 +952,27 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
                                          const BatchClass &L, const void *const *d_ptrs,
                                          double *parts, unsigned *counters, size_t chunk_cap,
                                          cudaStream_t st, long long wait_ns, int *tc_e, double *tc_bn,
-                                         size_t tc_cap) {
+                                         size_t tc_cap, const int *fx_k) {
     cudaError_t e;
     const int N = L.N;
     if (N <= kTileBits) {
         int np = 0;
         e = launch_small<R>(N, nullptr, d_ptrs, L.S, 0, 1ull << N, parts + L.parts_off,
-                            (int)L.parts_n, dev, st, &np, L.small_grid);
+                            (int)L.parts_n, dev, st, &np, L.small_grid, 2, fx_k);
         ws.launches += 1;
         return e;
+    }
+    if constexpr (sizeof(cx_t<R>) == 16) {
+        if (!tc_e || !tc_bn || (size_t)L.S << (N - kTileBits) > tc_cap) return cudaErrorInvalidValue;
+        if ((e = enqueue_fx_scales(nullptr, d_ptrs, L.S, N, reinterpret_cast<int2 *>(tc_bn), tc_e, st)) != cudaSuccess) return e;
+        ws.launches += 2;
     }
     size_t off = L.parts_off;
     for (int half = 0; half <= 1; ++half) {
         const LargeCfg &c = half ? L.cfg_half : L.cfg_full;
         const long long cps = half ? L.cps_half : L.cps_full;
-        const uint64_t xb = half ? (uint64_t)kTile : 0, xe = half ? (1ull << N) : (uint64_t)kTile;
-        if constexpr (sizeof(R) == 4) {
+        const uint64_t xb = half && L.cps_full ? (uint64_t)kTile : 0, xe = half ? (1ull << N) : (uint64_t)kTile;
+        if constexpr (sizeof(cx_t<R>) == 8) {
             if (one_applies(N, 8) && !(half && L.tc_kind)) {
                 if (cps == 0) continue;
                 if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;
@@ -902,19 +996,25 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
                 continue;
             }
         }
-        if (mid_applies(N, half, (int)sizeof(v2_t<R>))) {
-            // cps = shifts per state (the layout gave this range one chunk per shift)
-            if ((e = launch_mid<double>(N, half, nullptr, d_ptrs, L.S, cps, xb, 2, parts + off, nullptr, dev, st)) !=
-                cudaSuccess)
-                return e;
-            ws.launches += 1;
-            off += (size_t)cps * L.S;
-            continue;
+        if (cps == 0) continue;
+        if constexpr (sizeof(cx_t<R>) == 16) {
+            if (mid_applies(N, 16)) {
+                // one partial per shift
+                if ((e = launch_mid(N, nullptr, d_ptrs, L.S, cps, 0, 2, parts + off, nullptr,
+                                    reinterpret_cast<const int2 *>(tc_bn), tc_e, dev, st)) !=
+                    cudaSuccess)
+                    return e;
+                ws.launches += 1;
+                off += (size_t)cps * L.S;
+                continue;
+            }
         }
         if (!large_cfg_fits(ws, c, N, half)) return cudaErrorInvalidValue;
         LargeArgs A;
         A.psi = nullptr;
         A.psis = d_ptrs;
+        A.fx_bn = reinterpret_cast<const int2 *>(tc_bn);
+        A.tc_e = tc_e;
         A.chunks_per_state = cps;
         A.N = N;
         A.half = half;
@@ -952,7 +1052,7 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
         if (half && L.tc_kind)
             e = launch_large_tc(A, ws, dev, grid, st, L.tc_kind, tc_e, tc_bn, tc_cap);
         else
-            e = half ? launch_large<R, true>(A, grid, st) : launch_large<R, false>(A, grid, st);
+            e = launch_large<R>(A, grid, st);
         if (e != cudaSuccess) return e;
         ws.launches += 1;
         off += (size_t)A.n_chunks;
@@ -963,16 +1063,16 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
 cudaError_t enqueue_batch_class(const Workspace &ws, const DeviceInfo &dev, const BatchClass &L,
                                 const void *const *d_ptrs, double *parts, unsigned *counters,
                                 size_t chunk_cap, sre_mode_t mode, cudaStream_t st,
-                                long long wait_ns, int *tc_e, double *tc_bn, size_t tc_cap) {
+                                long long wait_ns, int *tc_e, double *tc_bn, size_t tc_cap, const int *fx_k) {
     if (mode == SRE_MODE_FP64)
-        return enqueue_batch_class_t<double>(ws, dev, L, d_ptrs, parts, counters, chunk_cap, st, wait_ns, nullptr,
-                                             nullptr, 0);
+        return enqueue_batch_class_t<fx>(ws, dev, L, d_ptrs, parts, counters, chunk_cap, st, wait_ns, tc_e,
+                                         tc_bn, tc_cap, fx_k);
     return enqueue_batch_class_t<float>(ws, dev, L, d_ptrs, parts, counters, chunk_cap, st, wait_ns, tc_e, tc_bn,
-                                        tc_cap);
+                                        tc_cap, nullptr);
 }
 
 cudaError_t enqueue_batch_norm(const Workspace &ws, const void *const *d_ptrs, const int *d_Ns,
-                               int count, double *npart, int *flags, sre_mode_t mode,
+                               int count, double *npart, int *flags, int *fx_k, sre_mode_t mode,
                                cudaStream_t st) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(flags, 0, sizeof(int) * count, st)) != cudaSuccess) return e;
@@ -982,6 +1082,9 @@ cudaError_t enqueue_batch_norm(const Workspace &ws, const void *const *d_ptrs, c
         k_norm_batch<double><<<grid, kThreads, 0, st>>>(d_ptrs, d_Ns, npart, flags);
     else
         k_norm_batch<float><<<grid, kThreads, 0, st>>>(d_ptrs, d_Ns, npart, flags);
+    ws.launches += 1;
+    if ((e = cudaGetLastError()) != cudaSuccess || mode != SRE_MODE_FP64) return e;
+    k_fx_exponent<<<count, kThreads, 0, st>>>(nullptr, d_ptrs, d_Ns, 0, reinterpret_cast<FxUnits *>(fx_k));
     ws.launches += 1;
     return cudaGetLastError();
 }

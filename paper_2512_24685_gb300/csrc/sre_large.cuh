@@ -1,5 +1,6 @@
-// sre_large.cuh -- the persistent two-pass CUDA-core kernel of libsre
-// (N > 12), and the work-item order and bounded waits it shares with the
+// sre_large.cuh -- the persistent two-pass CUDA-core kernel of libsre (fixed
+// point: N >= 15; FP32: N >= 21, smaller sizes run in sre_one.cu and
+// sre_two.cu), and the work-item order and bounded waits it shares with the
 // tensor-core kernel of sre_tc.cu.
 #pragma once
 #include <cuda.h>
@@ -39,16 +40,16 @@ using namespace dev;
 // released by chunk c - R (D < R keeps this deadlock-free: every item waits
 // only on items claimed before it).
 //
-// Halving (half = 1, shifts x >= 4096).  With pivot j = the highest set bit
-// of x, g_x(t ^ x) = conj(g_x(t)) pairs every t with t_j = 1 to one with
+// Halving.  With pivot j = the highest set bit of x, g_x(t ^ x) = conj(g_x(t)) pairs every t with t_j = 1 to one with
 // t_j = 0, and sum_z |A_x(z)|^4 = 16 sum_{z'} [(Re W(z'))^4 + (Im W(z'))^4]
 // where W is the (N-1)-bit transform of g_x restricted to t_j = 0 (A is
 // 2 Re W or 2i Im W, so at Renyi order alpha the exponents are 2 alpha and
-// the factor 2^(2 alpha)).  Since
-// j >= 12, the restriction removes one high bit: block t'_h maps to
-// t_h = t'_h with a zero inserted at bit j - 12, and h2 = N - 13.
+// the factor 2^(2 alpha)).  For
+// j >= 12 the restriction removes one high bit: block t'_h maps to t_h = t'_h
+// with a zero inserted at bit j - 12; below that it removes a bit of the block,
+// and x = 0 pairs the halves of the state (BlockPair).  h2 = N - 13.
 //
-// FP32 launches with 5 <= h2 <= 8 stage pass-2 tiles through TMA
+// FP32 launches with h2 = 8 (N = 21) stage pass-2 tiles through TMA
 // (sre_stage.cuh): tmap then describes the scratch ring as a 2-D FP32 array
 // of 8192 columns (4096 complex per block t'_h) by R * C * 2^h2 rows.  The
 // tensor-core kernel (sre_tc.cu) describes its 16-bit scratch planes there
@@ -56,6 +57,8 @@ using namespace dev;
 struct LargeArgs {
     CUtensorMap tmap;          // pass-2 staging (encode_p2_tmap / tc map), else unused
     const int *tc_e;           // tensor-core kernel: scale exponent per x >> 12
+    const int2 *fx_bn;         // fixed-point mode: bounds per 4096-entry block (fx_bound; tc_e: unit
+                               // exponent per x >> 12)
     const void *psi;           // the state (single-state launch)
     const void *const *psis;   // or: states of one batch class (device array)
     long long chunks_per_state;  // chunks of each state (batch class)
@@ -130,7 +133,7 @@ __device__ __forceinline__ void decode_item(const LargeArgs &a, long long item, 
 // Pass 2 of this instantiation stages its tiles through TMA.
 template <typename R, int H2>
 __host__ __device__ constexpr bool large_uses_tma() {
-    return sizeof(R) == 4 && H2 >= 5 && H2 <= 8;
+    return sizeof(R) == 4 && H2 == 8;
 }
 
 // Pass 1 of this instantiation can take its block pairs by bulk copy (FP32
@@ -145,14 +148,14 @@ __host__ __device__ constexpr bool large_stages_pass1() {
 // double as the TMA stages of pass 2, hence 1024-byte alignment).
 template <typename R, int H2>
 __host__ __device__ constexpr size_t large_smem_bytes() {
-    return (size_t)3 * kTileSlots * sizeof(v2_t<R>) + (large_uses_tma<R, H2>() ? 1024 : 0);
+    return (size_t)(sizeof(cx_t<R>) == 16 ? 1 : 3) * kTileSlots * sizeof(v2_t<R>) + (large_uses_tma<R, H2>() ? 1024 : 0);
 }
 
 // Host: encode LargeArgs::tmap for the launch's scratch ring.
 cudaError_t encode_p2_tmap(LargeArgs &a);
 
-template <typename R, int H2, bool HALF>
-__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(const __grid_constant__ LargeArgs a) {
+template <typename R, int H2>
+__global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ LargeArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using V = v2_t<R>;
     constexpr bool kTma = large_uses_tma<R, H2>();
@@ -160,8 +163,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
     unsigned char *sbase = smem_raw;
     if constexpr (kTma) sbase += (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
     V *bufB = reinterpret_cast<V *>(sbase);  // round 1 -> 2 moves, alternating with
-    V *bufC = bufB + kTileSlots;             //   bufC from tile to tile; pass-2 stages
-    V *bufA = bufC + kTileSlots;             // warp-local moves
+    // (fixed point: one buffer for all, ordered by one more barrier per tile)
+    constexpr bool kFx = sizeof(cx_t<R>) == 16;
+    V *bufC = bufB + (kFx ? 0 : kTileSlots);  //   bufC from tile to tile; pass-2 stages
+    V *bufA = bufC + (kFx ? 0 : kTileSlots);  // warp-local moves
     __shared__ long long s_next[2];
     __shared__ int s_stop[2];
     // stage barriers: [0], [1] the pass-2 tile stages (kTma), [2] the pass-1
@@ -172,16 +177,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
     uint32_t slost = 0;   // barriers whose completion wait expired
 
     const int tid = threadIdx.x;
-    const int lgx = a.N - (HALF ? 1 : 0);        // log2 scratch entries per shift
+    const int lgx = a.N - 1;                      // log2 scratch entries per shift
     const int C = 1 << a.C_log;
     const V *psi0 = reinterpret_cast<const V *>(a.psi);
     V *scratch = reinterpret_cast<V *>(a.scratch);
     constexpr int zsub_bits = kTileBits - H2;     // z entries per block in pass 2
     const int ipx_log = H2 - a.G2_log;            // pass-2 items per shift (log2)
-    // halved shifts: sum_z |A|^(2 alpha) = 2^(2 alpha) sum_z' [(Re W)^(2 alpha) +
-    // (Im W)^(2 alpha)] (16 at alpha = 2)
-    const double hfac = (double)(1ull << (2 * a.alpha));
-
     const int warp = tid >> 5, lane = tid & 31;
     constexpr int kWarps = kThreads / 32;
     // Item claims are prefetched one item ahead through a two-entry slot;
@@ -207,12 +208,21 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
         // batch class: chunk c belongs to state c / chunks_per_state
         long long cl = c;
         const V *psi = psi0;
+        long long sidx = 0;
         if (a.psis) {
-            const long long sidx = c / a.chunks_per_state;
+            sidx = c / a.chunks_per_state;
             cl = c - sidx * a.chunks_per_state;
             psi = reinterpret_cast<const V *>(a.psis[sidx]);
         }
+        // fixed point: block norms of the state and the exponent of the shifts' unit
+        const int2 *bn = nullptr;
+        int fxk = 0;
         const uint64_t xc = a.x0 + ((uint64_t)cl << a.C_log);
+        if constexpr (kFx) {
+            const size_t at = (size_t)sidx << (a.N - kTileBits);
+            bn = a.fx_bn + at;
+            fxk = a.tc_e[at + (xc >> kTileBits)];
+        }
         V *slot_base = scratch + (size_t)slot * ((size_t)C << lgx);
 
         if (pass1) {
@@ -228,8 +238,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
             }
             const uint64_t xh = xc >> kTileBits;
             const int xl0 = (int)(xc & (kTile - 1));
-            const int jh = HALF ? (63 - __clzll((long long)xc)) - kTileBits : 0;
-            if (kStage1 && a.stage1 && C == 1 && ((uintptr_t)psi & 15) == 0) {
+            const int jh = (63 - __clzll((long long)(xc | 1))) - kTileBits;  // pivot above the block: >= 0
+            if (jh >= 0 && kStage1 && a.stage1 && C == 1 && ((uintptr_t)psi & 15) == 0) {
                 // One shift per chunk and a 16-byte aligned state: the block
                 // t_h and its partner t_h ^ x_h arrive by two 32 KB bulk copies
                 // in the two stage buffers.  The products overwrite the own
@@ -244,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
                     const V *par = bufC;
                     auto issue_pair = [&](int kb) {
                         const int tp = (r << a.B1_log) + kb;
-                        const int th = HALF ? (((tp >> jh) << (jh + 1)) | (tp & ((1 << jh) - 1))) : tp;
+                        const int th = ((tp >> jh) << (jh + 1)) | (tp & ((1 << jh) - 1));
                         mbar_arrive_expect_tx(mb, 2u * kStageBytes);
                         bulk_load(smem_u32(own), psi + ((uint64_t)th << kTileBits), kStageBytes, mb);
                         bulk_load(smem_u32(par), psi + (((uint64_t)th ^ xh) << kTileBits), kStageBytes, mb);
@@ -269,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
                         for (int i = 0; i < 16; ++i) {
                             const V b = par[((i ^ q) << 8) | pl];
                             const V va = own[(i << 8) | tid];
-                            v[i] = conj_mul<R>(b.x, b.y, va.x, va.y);  // conj(phi_{t^x}) * phi_t
+                            v[i] = pair_value<R, false>(b, va, 0);  // conj(phi_{t^x}) * phi_t
                         }
                         reg_stages<2, 12, R>(v);
 #pragma unroll
@@ -290,23 +300,44 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
                         for (int i = 0; i < 16; ++i) __stcg(o + (i << 8), Cx<R>::to(v[i]));
                     }
                 }
-            } else
+            } else if (jh < 0 || kFx) {
+                // shifts below 4096: the pivot lies inside the block (x = 0
+                // pairs the halves of g_0), every shift has its own place map
+                for (int kb = 0; kb < (1 << a.B1_log); ++kb) {
+                    const int tp = (r << a.B1_log) + kb;
+                    for (int xl = 0; xl < C; ++xl) {
+                        const uint64_t x = xc + (uint64_t)xl;
+                        if (x < a.x_begin || x >= a.x_end) continue;
+                        cx_t<R> v[16];
+                        if constexpr (kFx) {
+                            const FxUnits un = fx_units(fx_bound(bn, 1 << (a.N - kTileBits), x, tp), fxk);
+                            block_values<R>(v, block_pair(psi, a.N, x, tp), tid, un.a);
+                            fx_tile<12>(v, bufB, tid, un);
+                            fx_rescale(v, fxk - un.c);
+                        } else {
+                            block_values<R>(v, block_pair(psi, a.N, x, tp), tid, 0);
+                            V *bB = (tcount & 1) ? bufC : bufB;
+                            ++tcount;
+                            tile_fwht12_rev<R>(v, bufA, bB, tid);
+                        }
+                        V *o = slot_base + ((size_t)xl << lgx) + ((size_t)tp << kTileBits) + tid;
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) __stcg(o + (i << 8), Cx<R>::to(v[i]));
+                    }
+                }
+            } else if constexpr (!kFx)
             for (int kb = 0; kb < (1 << a.B1_log); ++kb) {
                 const int tp = (r << a.B1_log) + kb;
-                const int th = HALF ? (((tp >> jh) << (jh + 1)) | (tp & ((1 << jh) - 1))) : tp;
+                const int th = ((tp >> jh) << (jh + 1)) | (tp & ((1 << jh) - 1));
                 // Round-2 layout: thread tid holds t_l = i << 8 | tid of block th
                 // (own factors phi_t in registers); its partners t ^ x are
                 // t_l ^ xlow of block th ^ x_h, read coalesced (each warp load
                 // covers one aligned 256-entry run).
-                R ar[16], ai[16];
+                V own[16];
                 {
                     const V *pa = psi + ((uint64_t)th << kTileBits) + tid;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const V va = __ldg(pa + (i << 8));
-                        ar[i] = va.x;
-                        ai[i] = va.y;
-                    }
+                    for (int i = 0; i < 16; ++i) own[i] = __ldg(pa + (i << 8));
                 }
                 const V *pb = psi + (((uint64_t)th ^ xh) << kTileBits);
                 for (int xl = 0; xl < C; ++xl) {
@@ -319,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const V b = __ldg(pbx + ((i ^ q) << 8));
-                        v[i] = conj_mul<R>(b.x, b.y, ar[i], ai[i]);  // conj(phi_{t^x}) * phi_t
+                        v[i] = pair_value<R, false>(b, own[i], 0);  // conj(phi_{t^x}) * phi_t
                     }
                     V *bB = (tcount & 1) ? bufC : bufB;
                     ++tcount;
@@ -344,6 +375,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
             const int zb0 = (j & ((1 << ipx_log) - 1)) << a.G2_log;
             const uint64_t x = xc + (uint64_t)xl;
             double acc = 0.0;
+            const double hfac = half_factor<R>(a.alpha, fxk);
             const bool staged2 = kTma && a.stage2;
             if constexpr (kTma) {
                 // One thread waits for the chunk's pass 1 and keeps two TMA
@@ -392,8 +424,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
                                             ((zb0 + gb) << zsub_bits) + (tid % kLpr) * 16);
                         }
                         const unsigned char *stage = reinterpret_cast<const unsigned char *>(st ? bufC : bufB);
-                        const float s = p2_tile<H2, HALF>(stage, reinterpret_cast<float2 *>(bufA), pl, a.alpha);
-                        acc += (HALF ? hfac : 1.0) * (double)s;
+                        const float s = p2_tile<H2>(stage, reinterpret_cast<float2 *>(bufA), pl, a.alpha);
+                        acc += hfac * (double)s;
                         if (gb + 2 < ntiles) {
                             __syncthreads();  // every thread has read stage st
                             if (tid == 0) {
@@ -424,9 +456,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) k_large(cons
                             __ldcg(xb + ((size_t)tp << kTileBits) + (zb << zsub_bits) + zs));
                     }
                     V *bB = (tcount & 1) ? bufC : bufB;
-                    if (H2 > 8) ++tcount;
+                    if (H2 > 8) {
+                        ++tcount;
+                        if (kFx) __syncthreads();  // one buffer: the previous tile's readers are done
+                    }
                     tile_fwht<H2, R>(v, bufA, bB, tid);
-                    acc += (HALF ? hfac : 1.0) * (double)sum_order<R, HALF>(v, a.alpha);
+                    acc += hfac * (double)sum_order<R>(v, a.alpha);
                 }
             }
             }

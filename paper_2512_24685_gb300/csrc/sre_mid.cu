@@ -1,24 +1,14 @@
-// sre_mid.cu -- FP64 single-pass kernel for shifts whose transform spans one
-// or two 4096-entry blocks: the halved shifts (x >= 4096) of N = 13 and 14
-// and the full shifts (x < 4096) of N = 13.
+// sre_mid.cu -- FP64 single-pass kernel (fixed-point transform, sre_tile.cuh)
+// for N = 13 and 14: the halved transform of a shift is one or two 4096-entry
+// blocks and stays inside one CTA.
 //
-// For such a shift the whole transform stays inside one CTA, so the two-pass
-// machinery (scratch ring, lagged work items, inter-CTA waits) is not needed.
 // A CTA takes whole shifts, grid-strided over (state, shift): it forms the
-// XOR-shifted products of each block, applies the 12-bit tile transform
-// (sre_tile.cuh, bits 8-11 first), parks every block but the last in shared
-// memory at positions only its own thread reads back (i << 8 | tid, no bank
-// conflicts), then applies the butterflies across the blocks (transform bits
-// 12 and up).  The
-// shift's quartic sum (or order-alpha sum; halved shifts with the factor
-// 2^(2 alpha)) is summed per thread in R and across the CTA in FP64 in a
-// fixed tree: one partial per shift, the same in a single or a batched
-// launch.
-//
-// Halving (x >= 4096, pivot j = highest set bit of x, jh = j - 12): the
-// restricted transform runs over t with t_j = 0; block t'_h of it is block
-// t_h = t'_h with a zero inserted at bit jh.  For N = 13 there is one block
-// (jh = 0, t_h = 0); for N = 14, t'_h = 0, 1.
+// XOR-shifted products of each block, applies the 12-bit tile transform (bits
+// 8-11 first), parks the first of two blocks in shared memory at positions
+// only its own thread reads back (i << 8 | tid, no bank conflicts), then applies
+// the butterfly across the blocks (transform bit 12).  The sum of powers is
+// taken per thread and across the CTA in FP64 in a fixed tree: one partial per
+// shift, the same in a single or a batched launch.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -32,63 +22,51 @@ using namespace dev;
 
 namespace {
 
-template <typename R, bool HALF, int NB>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_mid(const v2_t<R> *__restrict__ psi0, const void *const *__restrict__ psis, long long shifts_per_state,
-          uint64_t x_begin, long long n, int alpha, double *__restrict__ part, double *__restrict__ per_x) {
+template <int NB>
+__global__ void __launch_bounds__(kThreads, NB == 1 ? 2 : 1)
+    k_mid(const double2 *__restrict__ psi0, const void *const *__restrict__ psis, long long shifts_per_state,
+          uint64_t x_begin, long long n, int alpha, double *__restrict__ part, double *__restrict__ per_x,
+          const int2 *__restrict__ fx_bn, const int *__restrict__ fx_e) {
     static_assert(NB == 1 || NB == 2, "one or two blocks per shift");
+    constexpr int N = kTileBits + NB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using V = v2_t<R>;
-    V *bufA = reinterpret_cast<V *>(smem_raw);  // warp-local moves
-    V *bufB = bufA + kTileSlots;                 // CTA-wide moves
-    V *park = bufB + kTileSlots;                 // blocks 0 .. NB-2, 4096 entries each
+    double2 *buf = reinterpret_cast<double2 *>(smem_raw);  // moves
+    double2 *park = buf + kTileSlots;                       // block 0 of two
     __shared__ double red[kThreads / 32];
     const int tid = threadIdx.x;
-    const double hfac = HALF ? (double)(1ull << (2 * alpha)) : 1.0;
 
     for (long long g = blockIdx.x; g < n; g += gridDim.x) {
         const long long sidx = psis ? g / shifts_per_state : 0;
-        const V *psi = psis ? reinterpret_cast<const V *>(psis[sidx]) : psi0;
+        const double2 *psi = psis ? reinterpret_cast<const double2 *>(psis[sidx]) : psi0;
         const uint64_t x = x_begin + (uint64_t)(g - sidx * shifts_per_state);
-        const uint64_t xh = x >> kTileBits;
-        const int xlow = (int)(x & (kTile - 1));
-        const int q = xlow >> 8;
-        const int jh = HALF ? (63 - __clzll((long long)x)) - kTileBits : 0;
-        cx_t<R> v[16];
+        // block bounds of the state and the unit's exponent of the shift
+        const int2 *bn = fx_bn + (sidx << NB);
+        const int k = fx_e[(sidx << NB) + (long long)(x >> kTileBits)];
+        cx_t<fx> v[16];
 #pragma unroll
         for (int tp = 0; tp < NB; ++tp) {
-            const int th = HALF ? (((tp >> jh) << (jh + 1)) | (tp & ((1 << jh) - 1))) : tp;
-            const V *pa = psi + ((uint64_t)th << kTileBits) + tid;
-            const V *pb = psi + (((uint64_t)th ^ xh) << kTileBits) + (tid ^ (xlow & 255));
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const V a = __ldg(pa + (i << 8));
-                const V b = __ldg(pb + ((i ^ q) << 8));
-                v[i] = conj_mul<R>(b.x, b.y, a.x, a.y);  // conj(phi_{t^x}) * phi_t
-            }
-            // one CTA-wide buffer: the barrier keeps the previous block's (or
-            // shift's) readers ahead of this block's writers
-            __syncthreads();
-            tile_fwht12_rev<R>(v, bufA, bufB, tid);
+            const FxUnits un = fx_units(fx_bound(bn, 1 << NB, x, tp), k);
+            block_values<fx>(v, block_pair(psi, N, x, tp), tid, un.a);
+            fx_tile<12>(v, buf, tid, un);
+            fx_rescale(v, k - un.c);
             if (tp + 1 < NB) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) park[(tp << kTileBits) + ((i << 8) | tid)] = Cx<R>::to(v[i]);
+                for (int i = 0; i < 16; ++i) park[(i << 8) | tid] = Cx<fx>::to(v[i]);
             }
         }
-        R s;
+        double s = 0.0;
         if constexpr (NB == 2) {
-            cx_t<R> w[16];
+            cx_t<fx> w[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const cx_t<R> a = Cx<R>::from(park[(i << 8) | tid]);
-                w[i] = Cx<R>::sub(a, v[i]);
-                v[i] = Cx<R>::add(a, v[i]);
+                const cx_t<fx> a = Cx<fx>::from(park[(i << 8) | tid]);
+                w[i] = Cx<fx>::sub(a, v[i]);
+                v[i] = Cx<fx>::add(a, v[i]);
             }
-            s = sum_order<R, HALF>(v, alpha) + sum_order<R, HALF>(w, alpha);
-        } else {
-            s = sum_order<R, HALF>(v, alpha);
+            s = sum_order<fx>(w, alpha);
         }
-        const double tot = block_sum(hfac * (double)s, red);
+        s += sum_order<fx>(v, alpha);
+        const double tot = block_sum(half_factor<fx>(alpha, k) * s, red);
         if (tid == 0) {
             part[g] = tot;
             if (per_x) per_x[g] = tot;
@@ -96,41 +74,31 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-template <typename R, bool HALF, int NB>
+template <int NB>
 cudaError_t launch_mid_t(const void *psi, const void *const *psis, int nstates, long long sps, uint64_t x_begin,
-                         int alpha, double *part, double *per_x, const DeviceInfo &dev, cudaStream_t st) {
-    const size_t smem = ((size_t)2 * kTileSlots + (size_t)(NB > 1 ? NB - 1 : 0) * kTile) * sizeof(v2_t<R>);
-    auto kern = k_mid<R, HALF, NB>;
+                         int alpha, double *part, double *per_x, const int2 *fx_bn, const int *fx_e, const DeviceInfo &dev,
+                         cudaStream_t st) {
+    const size_t smem = ((size_t)kTileSlots + (size_t)(NB - 1) * kTile) * sizeof(double2);
+    auto kern = k_mid<NB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long n = sps * (long long)nstates;
     if (n <= 0) return cudaSuccess;
-    const int grid = (int)std::min<long long>(n, (long long)dev.sms);
-    kern<<<grid, kThreads, smem, st>>>(reinterpret_cast<const v2_t<R> *>(psi), psis, sps, x_begin, n, alpha,
-                                       part, per_x);
+    const int grid = (int)std::min<long long>(n, (long long)dev.sms * (NB == 1 ? 2 : 1));
+    kern<<<grid, kThreads, smem, st>>>(reinterpret_cast<const double2 *>(psi), psis, sps, x_begin, n, alpha, part,
+                                       per_x, fx_bn, fx_e);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-bool mid_applies(int N, int half, int elem_bytes) {
-    const int bits = N - (half ? 1 : 0);
-    return elem_bytes == 16 && N > kTileBits && bits >= kTileBits && bits <= kTileBits + 1;
-}
+bool mid_applies(int N, int elem_bytes) { return elem_bytes == 16 && (N == 13 || N == 14); }
 
-template <typename R>
-cudaError_t launch_mid(int N, int half, const void *psi, const void *const *psis, int nstates, long long sps,
-                       uint64_t x_begin, int alpha, double *part, double *per_x, const DeviceInfo &dev,
+cudaError_t launch_mid(int N, const void *psi, const void *const *psis, int nstates, long long sps, uint64_t x_begin,
+                       int alpha, double *part, double *per_x, const int2 *fx_bn, const int *fx_e, const DeviceInfo &dev,
                        cudaStream_t st) {
-    const int nb = 1 << (N - (half ? 1 : 0) - kTileBits);
-    if (half)
-        return nb == 1 ? launch_mid_t<R, true, 1>(psi, psis, nstates, sps, x_begin, alpha, part, per_x, dev, st)
-                       : launch_mid_t<R, true, 2>(psi, psis, nstates, sps, x_begin, alpha, part, per_x, dev, st);
-    return nb == 1 ? launch_mid_t<R, false, 1>(psi, psis, nstates, sps, x_begin, alpha, part, per_x, dev, st)
-                   : launch_mid_t<R, false, 2>(psi, psis, nstates, sps, x_begin, alpha, part, per_x, dev, st);
+    return N == 13 ? launch_mid_t<1>(psi, psis, nstates, sps, x_begin, alpha, part, per_x, fx_bn, fx_e, dev, st)
+                   : launch_mid_t<2>(psi, psis, nstates, sps, x_begin, alpha, part, per_x, fx_bn, fx_e, dev, st);
 }
-
-template cudaError_t launch_mid<double>(int, int, const void *, const void *const *, int, long long, uint64_t,
-                                        int, double *, double *, const DeviceInfo &, cudaStream_t);
 
 }  // namespace sre

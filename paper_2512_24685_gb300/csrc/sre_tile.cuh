@@ -21,7 +21,23 @@
 // FP32 complex values live in one 64-bit register pair and are combined with
 // the packed add/sub/mul/fma.rn.f32x2 instructions of sm_100+ (two IEEE
 // round-to-nearest FP32 operations per instruction: the same results as
-// scalar FP32 at half the instruction count).  FP64 values use double2.
+// scalar FP32 at half the instruction count).
+//
+// The FP64 mode transforms 64-bit fixed point (struct fx): an FP64 product is
+// rounded to a multiple of 2^(k - 63) and every butterfly is an exact integer
+// addition.  2^k bounds the values that the next four bits make, so nothing
+// overflows; the unit follows their growth, rounded every four bits: 16 and
+// 256 times the largest product of the block pair, then the product of the
+// blocks' l2 norms (Cauchy-Schwarz), above the block the sum of those products
+// over the shift's blocks.  The rounding that this leaves is below that of FP64
+// sums (per-shift sums of N = 13..15 states against 80-bit arithmetic).  The
+// reason is the pipe: GB300 runs 2 FP64 operations per clock and SM, against
+// some 40 64-bit integer additions.  FP64 operations are left for the product
+// (4 per entry) and the powers (4 per entry); both conversions are integer
+// code, since F2I and I2F run at the FP64 rate too.  Measured: all shifts of an
+// N = 16 state 46 ms (FP64 butterflies, full transforms below x = 4096: 178 ms),
+// 60 states of N = 12 10.5 ms with their evolution (61.9 ms); the FP64 pipe is
+// busy 65 % of the time.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -32,6 +48,11 @@ namespace dev {
 template <typename R> struct V2;
 template <> struct V2<float> { using T = float2; };
 template <> struct V2<double> { using T = double2; };
+struct fx {};  // FP64 state, fixed-point transform
+template <> struct V2<fx> { using T = double2; };
+template <typename R> struct Real { using T = R; };
+template <> struct Real<fx> { using T = double; };
+template <typename R> using real_t = typename Real<R>::T;  // partial sums within a thread
 template <typename R> using v2_t = typename V2<R>::T;
 
 constexpr int kTileSlots = 4096 + 256;  // padded shared-memory tile
@@ -79,22 +100,17 @@ template <> struct Cx<float> {
     }
 };
 
-template <> struct Cx<double> {
-    using T = double2;
-    static __device__ __forceinline__ T pack(double re, double im) { return make_double2(re, im); }
-    static __device__ __forceinline__ void unpack(T v, double &re, double &im) {
-        re = v.x;
-        im = v.y;
+template <> struct Cx<fx> {
+    using T = longlong2;
+    static __device__ __forceinline__ T add(T a, T b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+    static __device__ __forceinline__ T sub(T a, T b) { return make_longlong2(a.x - b.x, a.y - b.y); }
+    static __device__ __forceinline__ T zero() { return make_longlong2(0, 0); }
+    static __device__ __forceinline__ T from(double2 v) {
+        return make_longlong2(__double_as_longlong(v.x), __double_as_longlong(v.y));
     }
-    static __device__ __forceinline__ T add(T a, T b) { return make_double2(a.x + b.x, a.y + b.y); }
-    static __device__ __forceinline__ T sub(T a, T b) { return make_double2(a.x - b.x, a.y - b.y); }
-    static __device__ __forceinline__ T mul(T a, T b) { return make_double2(a.x * b.x, a.y * b.y); }
-    static __device__ __forceinline__ T fma(T a, T b, T c) {
-        return make_double2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
+    static __device__ __forceinline__ double2 to(T v) {
+        return make_double2(__longlong_as_double(v.x), __longlong_as_double(v.y));
     }
-    static __device__ __forceinline__ T zero() { return make_double2(0.0, 0.0); }
-    static __device__ __forceinline__ T from(double2 v) { return v; }
-    static __device__ __forceinline__ double2 to(T v) { return v; }
 };
 
 template <typename R> using cx_t = typename Cx<R>::T;
@@ -105,12 +121,137 @@ __device__ __forceinline__ cx_t<R> conj_mul(R br, R bi, R ar, R ai) {
     return Cx<R>::pack(br * ar + bi * ai, br * ai - bi * ar);
 }
 
+// Marks a state whose norm is not a finite number.
+constexpr int kFxNonFinite = 0x3fffffff;
+
+// Bounds travel as 256 log2, rounded up, so that the transform kernels derive
+// units without FP64 operations: bound < 2^(l / 256).
+__device__ __forceinline__ int fx_log(double m) {
+    if (!isfinite(m)) return kFxNonFinite;
+    return m > 0.0 ? (int)ceil(256.0 * log2(m)) + 1 : -(1 << 20);
+}
+// Smallest k with 2^(l / 256) <= 2^k.
+__device__ __forceinline__ int fx_exponent(int l) { return l >= kFxNonFinite / 2 ? kFxNonFinite : (l + 255) >> 8; }
+
+// From unit 2^(k1 - 63) to the coarser 2^(k2 - 63), q = k2 - k1, rounded.
+__device__ __forceinline__ long long fx_shift(long long a, int q) {
+    return q <= 0 ? a : q > 62 ? 0 : (a + (1ll << (q - 1))) >> q;
+}
+
+// round(p 2^(63 - k)), |p| < 2^k.  The mantissa, 10 bits up, moves right by
+// what its exponent lacks to the top; half of the last place is added first.
+__device__ __forceinline__ long long fx_from(double p, int k) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(p);
+    const int e = (int)(b >> 52) & 2047;
+    // shift left by e - 1075 + 63 - k in all, 10 of them already done
+    const int q = 1022 - e + k;
+    const unsigned long long m =
+        (((b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull)) << 10) + ((1ull << (q & 63)) >> 1);
+    const long long r = (unsigned)q < 64 ? (long long)(m >> (q & 63)) : 0;  // zero, or below half a unit
+    return (long long)b < 0 ? -r : r;
+}
+
+// |a| 2^-63 as a double (the sign does not matter to even powers), rounded to
+// 53 bits; a carry out of the mantissa moves on into the exponent.
+__device__ __forceinline__ double fx_abs(long long a) {
+    const unsigned long long u = (unsigned long long)(a < 0 ? -a : a);
+    const int lz = __clzll((long long)u);
+    const unsigned long long n = u << (lz & 63);
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1) + ((unsigned long long)(1022 - lz) << 52);
+    return u ? __longlong_as_double((long long)m) : 0.0;
+}
+
+// g_x(t) = conj(phi_{t^x}) phi_t from the factors b = phi_{t^x}, a = phi_t, or
+// for x = 0 (ZERO) W's input ((g0 + g1) / 2, (g0 - g1) / 2) from the two halves
+// of g_0.  k: the fixed-point unit's exponent (fx only).
+template <typename R, bool ZERO>
+__device__ __forceinline__ cx_t<R> pair_value(v2_t<R> b, v2_t<R> a, int k) {
+    using T = real_t<R>;
+    T re, im;
+    if constexpr (ZERO) {
+        const T g0 = a.x * a.x + a.y * a.y, g1 = b.x * b.x + b.y * b.y;
+        re = T(0.5) * (g0 + g1);
+        im = T(0.5) * (g0 - g1);
+    } else {
+        re = b.x * a.x + b.y * a.y;
+        im = b.x * a.y - b.y * a.x;
+    }
+    if constexpr (sizeof(cx_t<R>) == 8)
+        return Cx<R>::pack(re, im);
+    else
+        return make_longlong2(fx_from(re, k), fx_from(im, k));
+}
+
+// Factor of a partial sum of (Re W)^(2 alpha) + (Im W)^(2 alpha): 2^(2 alpha)
+// for the halving, and the fixed-point unit 2^k to the same power (NaN for a
+// state without a finite norm, whose fixed-point values mean nothing).
+template <typename R>
+__device__ __forceinline__ double half_factor(int alpha, int k) {
+    if constexpr (sizeof(cx_t<R>) == 8) return (double)(1ull << (2 * alpha));
+    if (k == kFxNonFinite) return __longlong_as_double(0x7ff8000000000000ll);
+    return scalbn(1.0, 2 * alpha * (1 + k));
+}
+
+// Where one shift finds the factors of a 4096-entry block of t' (t with the
+// pivot bit removed): own entry e at place(e) from `own`, its partner at
+// place(e) ^ xo from `par`.
+template <typename V>
+struct BlockPair {
+    const V *own, *par;
+    int xo, pivot;  // pivot 12: it lies above the block
+    bool zero;      // x = 0: the two halves of g_0
+    __device__ __forceinline__ int place(int e) const {
+        if (pivot == 12) return e;
+        const int lo = e & ((1 << pivot) - 1);
+        return ((e - lo) << 1) | lo;
+    }
+};
+
+template <typename V>
+__device__ __forceinline__ BlockPair<V> block_pair(const V *psi, int N, uint64_t x, int tp) {
+    BlockPair<V> s;
+    s.zero = x == 0;
+    const uint64_t xe = s.zero ? 1ull << (N - 1) : x;
+    const int j = 63 - __clzll((long long)xe);
+    if (j >= 12) {
+        const uint64_t th = (((uint64_t)tp >> (j - 12)) << (j - 11)) | ((uint64_t)tp & ((1ull << (j - 12)) - 1));
+        s.own = psi + (th << 12);
+        s.par = psi + ((th ^ (xe >> 12)) << 12);
+        s.xo = (int)(xe & 4095);
+        s.pivot = 12;
+    } else {
+        s.own = s.par = psi + ((uint64_t)tp << 13);
+        s.xo = (int)xe;
+        s.pivot = j;
+    }
+    return s;
+}
+
 template <int K> __device__ __forceinline__ int elem(int tid, int i);
 template <> __device__ __forceinline__ int elem<0>(int tid, int i) { return (tid << 4) | i; }
 template <> __device__ __forceinline__ int elem<1>(int tid, int i) {
     return ((tid >> 4) << 8) | (i << 4) | (tid & 15);
 }
 template <> __device__ __forceinline__ int elem<2>(int tid, int i) { return (i << 8) | tid; }
+
+// Products of a block in round-2 layout (e = i << 8 | tid), any pivot.
+template <typename R, bool ZERO>
+__device__ __forceinline__ void block_values_z(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid, int k) {
+    const int o = s.place(tid), w0 = s.place(256), w1 = s.place(512), w2 = s.place(1024), w3 = s.place(2048);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int e = o + ((i & 1) ? w0 : 0) + ((i & 2) ? w1 : 0) + ((i & 4) ? w2 : 0) + ((i & 8) ? w3 : 0);
+        v[i] = pair_value<R, ZERO>(__ldg(s.par + (e ^ s.xo)), __ldg(s.own + e), k);
+    }
+}
+
+template <typename R>
+__device__ __forceinline__ void block_values(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid, int k) {
+    if (s.zero)
+        block_values_z<R, true>(v, s, tid, k);
+    else
+        block_values_z<R, false>(v, s, tid, k);
+}
 
 // Butterflies over register bits j in [0, 4) whose tile bit 4K + j < NB.
 template <int K, int NB, typename R>
@@ -172,6 +313,61 @@ __device__ __forceinline__ void tile_fwht(cx_t<R> (&v)[16], v2_t<R> *bufA, v2_t<
     }
 }
 
+// Unit exponents of a fixed-point tile: its products, after four bits and
+// after eight.
+struct FxUnits {
+    int a, b, c;
+};
+
+// From the bounds (256 log2) of the largest product and of all partial sums of
+// the tile, none above the exponent `most`.
+__device__ __forceinline__ FxUnits fx_units(int2 l, int most) {
+    FxUnits u;
+    u.c = min(fx_exponent(l.y), most);
+    u.b = min(fx_exponent(l.x + (8 << 8)), u.c);
+    u.a = min(fx_exponent(l.x + (4 << 8)), u.b);
+    return u;
+}
+
+__device__ __forceinline__ void fx_rescale(cx_t<fx> (&v)[16], int q) {
+    if (q <= 0) return;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = make_longlong2(fx_shift(v[i].x, q), fx_shift(v[i].y, q));
+}
+
+// 12-bit transform of the fixed-point mode, bits 8-11 first, of which the bits
+// below NB are transformed: round-2 layout at unit u.a in, round-0 layout at
+// u.c out.  One buffer serves both moves (after the CTA-wide one each warp
+// stays in its own part of it); the barrier before it keeps the previous
+// tile's readers ahead.
+template <int NB>
+__device__ __forceinline__ void fx_tile(cx_t<fx> (&v)[16], double2 *buf, int tid, const FxUnits &u) {
+    reg_stages<2, NB, fx>(v);
+    fx_rescale(v, u.b - u.a);
+    __syncthreads();
+    relayout<2, 1, false, fx>(v, buf, tid);
+    reg_stages<1, NB, fx>(v);
+    fx_rescale(v, u.c - u.b);
+    relayout<1, 0, true, fx>(v, buf, tid);
+    reg_stages<0, NB, fx>(v);
+}
+
+// Bounds (256 log2) of the largest product and of the partial sums of block
+// t'_h = tp of shift x, from the blocks' (largest |phi|^2, squared l2 norm): the
+// block pair's geometric mean, or for a pivot inside the block (x < 4096) twice
+// the larger of the two blocks that the halved one comes from (nb: blocks of
+// the state).
+__device__ __forceinline__ int2 fx_bound(const int2 *bn, int nb, uint64_t x, int tp) {
+    if (x < 4096) {  // x = 0 pairs the halves of the state
+        const int2 a = __ldg(bn + (x ? 2 * tp : tp)), b = __ldg(bn + (x ? 2 * tp + 1 : tp + nb / 2));
+        return make_int2(max(a.x, b.x), max(a.y, b.y) + 256);
+    }
+    const int xh = (int)(x >> 12), j = 31 - __clz(xh);
+    const int th = ((tp >> j) << (j + 1)) | (tp & ((1 << j) - 1));
+    const int2 a = __ldg(bn + th), b = __ldg(bn + (th ^ xh));
+    return make_int2((a.x + b.x + 1) >> 1, (a.y + b.y + 1) >> 1);
+}
+
 // Full 12-bit transform, bits 8-11 first: input in round-2 layout (thread
 // tid holds e = i << 8 | tid, so loads of consecutive threads are
 // contiguous), output in round-0 layout.  One CTA-wide move (bufB, to be
@@ -186,110 +382,57 @@ __device__ __forceinline__ void tile_fwht12_rev(cx_t<R> (&v)[16], v2_t<R> *bufA,
     reg_stages<0, 12, R>(v);
 }
 
-// sum_i |F_i|^4 over the thread's 16 entries, in R.
-template <typename R>
-__device__ __forceinline__ R sum_abs4(const cx_t<R> (&v)[16]) {
-    R s = R(0);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        R re, im;
-        Cx<R>::unpack(Cx<R>::mul(v[i], v[i]), re, im);
-        const R m = re + im;
-        s += m * m;
-    }
-    return s;
-}
-
-// sum_i (Re F_i)^4 + (Im F_i)^4 over the thread's 16 entries, in R.
-template <typename R>
-__device__ __forceinline__ R sum_re4_im4(const cx_t<R> (&v)[16]) {
-    cx_t<R> acc = Cx<R>::zero();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const cx_t<R> sq = Cx<R>::mul(v[i], v[i]);
-        acc = Cx<R>::fma(sq, sq, acc);
-    }
-    R a, b;
-    Cx<R>::unpack(acc, a, b);
-    return a + b;
-}
-
-// Order alpha of Eq. (sre): sum_i (|F_i|^2)^alpha over the thread's 16
-// entries (integer alpha >= 2, a product of alpha factors), in R.
-template <typename R>
-__device__ __forceinline__ R sum_abs_pow(const cx_t<R> (&v)[16], int alpha) {
-    R s = R(0);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        R re, im;
-        Cx<R>::unpack(Cx<R>::mul(v[i], v[i]), re, im);
-        const R m = re + im;
-        R p = m;
-        for (int k = 1; k < alpha; ++k) p *= m;
-        s += p;
-    }
-    return s;
-}
-
-// Order alpha, halved shifts: sum_i (Re F_i)^(2 alpha) + (Im F_i)^(2 alpha).
-template <typename R>
-__device__ __forceinline__ R sum_re_im_pow(const cx_t<R> (&v)[16], int alpha) {
-    cx_t<R> acc = Cx<R>::zero();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const cx_t<R> sq = Cx<R>::mul(v[i], v[i]);
-        cx_t<R> p = sq;
-        for (int k = 1; k < alpha; ++k) p = Cx<R>::mul(p, sq);
-        acc = Cx<R>::add(acc, p);
-    }
-    R a, b;
-    Cx<R>::unpack(acc, a, b);
-    return a + b;
-}
-
-// Orders 3 and 4 with the power unrolled at compile time (same products in
-// the same order as the loops above).
+// sum_i (Re F_i)^(2 A) + (Im F_i)^(2 A) over the thread's 16 entries, in FP32
+// or FP64 (fx, in units of 2^k); A = 0: the order alpha known at run time only.
 template <typename R, int A>
-__device__ __forceinline__ R sum_abs_pow_c(const cx_t<R> (&v)[16]) {
-    R s = R(0);
+__device__ __forceinline__ real_t<R> sum_re_im_pow(const cx_t<R> (&v)[16], int alpha) {
+    if constexpr (sizeof(cx_t<R>) == 8) {
+        cx_t<R> acc = Cx<R>::zero();
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        R re, im;
-        Cx<R>::unpack(Cx<R>::mul(v[i], v[i]), re, im);
-        const R m = re + im;
-        R p = m;
+        for (int i = 0; i < 16; ++i) {
+            const cx_t<R> sq = Cx<R>::mul(v[i], v[i]);
+            if constexpr (A == 2) {
+                acc = Cx<R>::fma(sq, sq, acc);
+                continue;
+            }
+            cx_t<R> p = sq;
+            if constexpr (A > 0) {
 #pragma unroll
-        for (int k = 1; k < A; ++k) p *= m;
-        s += p;
+                for (int k = 1; k < A; ++k) p = Cx<R>::mul(p, sq);
+            } else {
+                for (int k = 1; k < alpha; ++k) p = Cx<R>::mul(p, sq);
+            }
+            acc = Cx<R>::add(acc, p);
+        }
+        float a, b;
+        Cx<R>::unpack(acc, a, b);
+        return a + b;
+    } else {
+        double acc = 0.0, acd = 0.0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const double re = fx_abs(v[i].x), im = fx_abs(v[i].y);
+            const double s = re * re, t = im * im;
+            double p = s, q = t;
+            for (int k = 2; k < (A ? A : alpha); ++k) {
+                p *= s;
+                q *= t;
+            }
+            acc = __fma_rn(p, s, acc);
+            acd = __fma_rn(q, t, acd);
+        }
+        return acc + acd;
     }
-    return s;
 }
 
-template <typename R, int A>
-__device__ __forceinline__ R sum_re_im_pow_c(const cx_t<R> (&v)[16]) {
-    cx_t<R> acc = Cx<R>::zero();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const cx_t<R> sq = Cx<R>::mul(v[i], v[i]);
-        cx_t<R> p = sq;
-#pragma unroll
-        for (int k = 1; k < A; ++k) p = Cx<R>::mul(p, sq);
-        acc = Cx<R>::add(acc, p);
-    }
-    R a, b;
-    Cx<R>::unpack(acc, a, b);
-    return a + b;
-}
-
-// The thread's share of the order-alpha sum (HALF: the halved-shift form);
-// order 2 takes the M2 reductions above unchanged.
-template <typename R, bool HALF>
-__device__ __forceinline__ R sum_order(const cx_t<R> (&v)[16], int alpha) {
+// The thread's share of the order-alpha sum of the halved form.
+template <typename R>
+__device__ __forceinline__ real_t<R> sum_order(const cx_t<R> (&v)[16], int alpha) {
     switch (alpha) {
-        case 2: return HALF ? sum_re4_im4<R>(v) : sum_abs4<R>(v);
-        case 3: return HALF ? sum_re_im_pow_c<R, 3>(v) : sum_abs_pow_c<R, 3>(v);
-        case 4: return HALF ? sum_re_im_pow_c<R, 4>(v) : sum_abs_pow_c<R, 4>(v);
-        default: return HALF ? sum_re_im_pow<R>(v, alpha) : sum_abs_pow<R>(v, alpha);
+        case 2: return sum_re_im_pow<R, 2>(v, alpha);
+        case 3: return sum_re_im_pow<R, 3>(v, alpha);
+        case 4: return sum_re_im_pow<R, 4>(v, alpha);
+        default: return sum_re_im_pow<R, 0>(v, alpha);
     }
 }
 
