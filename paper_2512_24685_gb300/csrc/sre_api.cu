@@ -225,7 +225,7 @@ static sre::LargeCfg plan_cfg(sre_plan_t p, int N) {
     // a tuned configuration serves the kernel it was timed on: the FP32 modes'
     // kernels count items and lag differently
     const bool tuned = p->has_tuned[N] && (p->tuned_mode[N] == SRE_MODE_FP32) == (p->mode == SRE_MODE_FP32);
-    sre::LargeCfg c = tuned ? p->tuned[N] : sre::choose_main_cfg(p->dev, p->ws, N, p->mode);
+    sre::LargeCfg c = tuned ? p->tuned[N] : sre::tuning_base_cfg(p->dev, p->ws, N, p->mode, p->user);
     if (p->user.x_batch_log >= 0) c.C_log = p->user.x_batch_log;
     if (p->user.ring_slots >= 0) c.R = p->user.ring_slots;
     if (p->user.lag >= 0) c.D = p->user.lag;

@@ -91,6 +91,9 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half
 // arithmetic mode (the halved shifts, or all shifts where sre_two.cu takes
 // them), and whether a configuration fits a workspace.
 LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode);
+// The configuration that a caller's partial tuning completes: with a ring field
+// of the caller's own, the L2-sized one, whose lag and slots leave room for it.
+LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t);
 bool main_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, sre_mode_t mode);
 
 // Tensor-core two-pass kernel (sre_tc.cu) for the halved shifts of one

@@ -29,6 +29,7 @@
 #include "sre_internal.h"
 #include "sre_large.cuh"
 #include "sre_tile.cuh"
+#include "sre_batched.h"
 #include "sre_one.h"
 #include "sre_two.h"
 
@@ -381,9 +382,40 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half
     return c;
 }
 
+// The tensor-core kernel's ring: eight shifts per chunk, so that one pass-1
+// operand build serves eight, and as many slots as the tuning scratch (192 MB)
+// holds, with pass 2 a third of the ring behind.  One CTA per SM holds a
+// pass-1 item for far longer than the L2-sized rings of choose_large_cfg last,
+// and pass 1 then waits for slots.  fp16_split, 2^31 to 2^33 halved entries,
+// L2-sized ring -> this one: N = 16 5.68 -> 4.75 ms, 17 12.9 -> 7.5, 18 19.7 -> 12.9,
+// 19 18.6 -> 12.7, 20 18.4 -> 13.1.  Six slots at least: a workspace with less
+// scratch takes fewer shifts per chunk, and below that the general rule.
+static LargeCfg choose_tc_cfg(const DeviceInfo &dev, const Workspace &ws, int N) {
+    LargeCfg c = choose_large_cfg(dev, N, 8, 1);
+    const size_t ring = std::min(ws.scratch_bytes, kTuneScratch);
+    for (int C_log = 3; C_log >= 0; --C_log) {
+        const int R = (int)std::min<size_t>(kMaxRing - 1, ring / ((size_t)8 << (N - 1 + C_log)));
+        if (R < 6) continue;
+        c.C_log = C_log;
+        c.R = R;
+        c.D = R / 3;
+        c.G2_log = std::min(5, N - 1 - kTileBits);
+        break;
+    }
+    return c;
+}
+
 LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode) {
     const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
-    return mode == SRE_MODE_FP32 && two_applies(N, eb) ? choose_two_cfg(dev, ws, N) : choose_large_cfg(dev, N, eb, 1);
+    if (mode == SRE_MODE_FP32 && two_applies(N, eb)) return choose_two_cfg(dev, ws, N);
+    if (tc_mode_available(mode) && tc_applies(N, 1, 2, nullptr)) return choose_tc_cfg(dev, ws, N);
+    return choose_large_cfg(dev, N, eb, 1);
+}
+
+LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t) {
+    if (t.x_batch_log >= 0 || t.ring_slots >= 0 || t.lag >= 0)
+        return choose_large_cfg(dev, N, mode == SRE_MODE_FP64 ? 16 : 8, 1);
+    return choose_main_cfg(dev, ws, N, mode);
 }
 
 bool main_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, sre_mode_t mode) {
@@ -732,8 +764,9 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         if (tc && split < x_end) {
             LargeArgs a;
             int grid = 0;
+            const LargeCfg c = cfg_override ? *cfg_override : choose_tc_cfg(dev, ws, N);
             if ((e = make_large_args(&a, ws, dev, psi, N, split, x_end, 1, eb, chunks,
-                                     d_per_x ? d_per_x + (split - x_begin) : nullptr, wait_ns, cfg_override,
+                                     d_per_x ? d_per_x + (split - x_begin) : nullptr, wait_ns, &c,
                                      &grid)) != cudaSuccess)
                 return e;
             a.alpha = alpha;
@@ -916,7 +949,7 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
     if (one_applies(N, eb)) {
         // one partial per shift, all shifts or those below 4096 beside the
         // tensor-core kernel
-        L.cfg_half = tuned_half ? *tuned_half : choose_large_cfg(dev, N, eb, 1);
+        L.cfg_half = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode);
         L.cps_full = tc_kind ? (long long)kTile : 0;
         L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)
                              : 1ll << N;
@@ -929,7 +962,7 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         // tensor-core kernel
         L.cfg_full = choose_two_cfg(dev, ws, N);
         L.cfg_half = mode == SRE_MODE_FP32 && tuned_half ? *tuned_half : L.cfg_full;
-        if (tc_kind) L.cfg_half = tuned_half ? *tuned_half : choose_large_cfg(dev, N, eb, 1);
+        if (tc_kind) L.cfg_half = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode);
         L.cps_full = tc_kind ? two_layout(ws, L.cfg_full, N, 0, kTile).n_chunks : 0;
         L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)
                              : two_layout(ws, L.cfg_half, N, 0, 1ull << N).n_chunks;

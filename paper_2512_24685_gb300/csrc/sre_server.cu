@@ -390,7 +390,7 @@ sre_status_t sre_server_create(const sre_server_cfg_t *cfg, sre_server_t *out) {
 
 sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t) {
     if (!s || !t || N <= sre::kTileBits || N > s->cfg.max_N) return SRE_EINVAL;
-    sre::LargeCfg c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode);
+    sre::LargeCfg c = sre::tuning_base_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode, *t);
     if (t->x_batch_log >= 0) c.C_log = t->x_batch_log;
     if (t->ring_slots >= 0) c.R = t->ring_slots;
     if (t->lag >= 0) c.D = t->lag;
@@ -400,6 +400,13 @@ sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t)
     if (t->pass2_staged >= 0) c.stage2 = t->pass2_staged;
     c.G2_log = std::min(c.G2_log, N - sre::kTileBits - 1);
     c.B1_log = std::min(c.B1_log, N - sre::kTileBits - 1);
+    // a plan's library configuration, whose ring a slot's smaller scratch may
+    // not hold, stands for the slot's own
+    sre::Workspace plan_ws;
+    plan_ws.scratch_bytes = sre::kTuneScratch;
+    const sre::LargeCfg lib = sre::choose_main_cfg(s->dev, plan_ws, N, s->cfg.mode);
+    if (c.C_log == lib.C_log && c.R == lib.R && c.D == lib.D)
+        c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode);
     std::lock_guard<std::mutex> lk(s->mu);
     for (const Slot &sl : s->slots)
         if (!sre::main_cfg_fits(sl.ws, c, N, s->cfg.mode)) return SRE_EINVAL;
