@@ -15,6 +15,7 @@ constexpr int kPerThread = kTile / kThreads;  // 16 entries per thread (4 regist
 constexpr int kNormBlocks = 264;           // fixed grid of the norm reduction
 constexpr int kFinalThreads = 256;
 constexpr size_t kWorkBytes = 1024;               // work-queue counters of a workspace
+constexpr size_t kFlagBytes = 16;                 // flags, status, ticket: behind the counters
 constexpr int kMaxRing = 64;                      // ring slots a tuned configuration may use
 constexpr size_t kTuneScratch = (size_t)192 << 20;  // scratch floor for N > 12 plans (tuned rings)
 constexpr size_t kSlotScratch = (size_t)96 << 20;   // scratch floor for server slots (default rings)
@@ -60,8 +61,9 @@ struct Workspace {
     size_t chunk_cap = 0;
     unsigned *counters = nullptr;  // done1 | done2 | freed, chunk_cap each
     unsigned long long *work = nullptr;  // work-queue counters (full, halved)
-    int *status = nullptr;         // device status word
+    int *status = nullptr;         // device status word (flags + 1)
     Result *result = nullptr;      // device result block
+    Result *host_result = nullptr; // pinned, the result as well: in a call that waits for it
     void *conv = nullptr;          // state converted to the compute type (lazy)
     size_t conv_bytes = 0;
     int *tc_e = nullptr;           // tensor-core path: scale exponent per x >> 12

@@ -134,6 +134,80 @@ cudaError_t enqueue_fx_scales(const void *psi, const void *const *psis, int nsta
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------------- finalize
+
+// Fixed-order FP64 sum of two segments of partials by one warp: lane l adds
+// entries l, l+32, ... of each segment in order, then a fixed shuffle tree.
+// Shared by the single-state and the batch finalize, so a state's M2 is
+// bitwise the same in either.
+__device__ __forceinline__ double warp_sum_segments(const double *p, long long o1, long long n1,
+                                                    long long o2, long long n2) {
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (long long k = lane; k < n1; k += 32) s += __ldcg(p + o1 + k);
+    for (long long k = lane; k < n2; k += 32) s += __ldcg(p + o2 + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;  // valid in lane 0
+}
+
+__device__ __forceinline__ double m2_from(double S, double n2, int N, bool bad) {
+    // M2 = -log2(S / (d n2^4)), in logs so tiny norms do not underflow
+    return bad ? __longlong_as_double(0x7ff8000000000000ll)
+               : -(log2(S) - (double)N - 4.0 * log2(n2));
+}
+
+// Eq. (sre) at integer order alpha: M_alpha = log2(S / (d n2^(2 alpha))) /
+// (1 - alpha); order 2 is m2_from.
+__device__ __forceinline__ double malpha_from(double S, double n2, int N, int alpha, bool bad) {
+    if (alpha == 2) return m2_from(S, n2, N, bad);
+    return bad ? __longlong_as_double(0x7ff8000000000000ll)
+               : (log2(S) - (double)N - 2.0 * alpha * log2(n2)) / (1.0 - alpha);
+}
+
+// One warp: S from the partial segments [o1, o1+n1) and [o2, o2+n2), n2 from
+// the norm partials, M2 and the status (by_norm: the entries are FP32, whose n2
+// is finite unless an entry is not); host, when given, is pinned memory of
+// the caller's that gets the result as well.
+__device__ __forceinline__ void finalize_warp(const double *parts, long long o1, long long n1, long long o2,
+                                              long long n2c, const double *npart, int nn, int N, int st, bool bad, bool by_norm,
+                                              Result *res, Result *host, double *d_m2, int alpha) {
+    const double S = warp_sum_segments(parts, o1, n1, o2, n2c);
+    const double n2 = warp_sum_segments(npart, 0, nn, 0, 0);
+    if ((threadIdx.x & 31) == 0) {
+        if (st == 0 && (bad || (by_norm && !isfinite(n2)))) st = SRE_ENONFINITE;
+        if (st == 0 && !(n2 > 0.0)) st = SRE_EZERO;
+        const double m2 = malpha_from(S, n2, N, alpha, st != 0);
+        res->m2 = m2;
+        res->S = S;
+        res->n2 = n2;
+        res->status = st;
+        if (host) *host = *res;
+        if (d_m2) *d_m2 = m2;
+    }
+}
+
+__global__ void k_finalize(const double *__restrict__ parts, long long o1, long long n1, long long o2,
+                           long long n2c, const double *__restrict__ npart, int nn, int N,
+                           const int *flags, const int *status, Result *res, Result *host, double *d_m2,
+                           int alpha) {
+    finalize_warp(parts, o1, n1, o2, n2c, npart, nn, N, *status, (*flags & kFlagNonFinite) != 0, false, res, host,
+                  d_m2, alpha);
+}
+
+// What the single-state k_small does besides its tiles: the norm of the state
+// that it holds in shared memory (the partials of k_norm, by the same CTAs'
+// worth of entries in the same order) and, in the CTA that ends last, the
+// finalize.  Two kernels of a few microseconds each, and the gaps before
+// them, were most of the device time of a call with N <= 10.
+struct SmallTail {
+    double *npart = nullptr;  // null: a batch, whose norms and sums are formed elsewhere
+    unsigned *ticket = nullptr;
+    Result *res = nullptr, *host = nullptr;
+    double *d_m2 = nullptr;
+};
+static_assert(kNormBlocks * kThreads >= kTile, "one entry per thread of k_norm");
+
 // ------------------------------------------------------- N <= 12: k_small
 
 // Tile g covers flat indices [g*4096, (g+1)*4096) of the (x - x_begin, t')
@@ -146,7 +220,7 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
                                                     long long tiles_per_state,
                                                     uint64_t x_begin, uint64_t x_end,
                                                     long long ntiles,
-                                                    double *__restrict__ part, int alpha) {
+                                                    double *__restrict__ part, int alpha, SmallTail tail) {
     // Single state: psis == nullptr.  Several states of the same N: psis[s] is
     // state s and tiles are numbered state-major.  Tile g's sum goes to
     // part[g] (fixed-order tree inside the tile), so a state's partials do not
@@ -193,6 +267,26 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
         const double s = block_sum(hfac * (double)sum_order<R>(v, alpha), red);
         if (tid == 0) part[g] = s;
     }
+    if (!tail.npart) return;
+    constexpr int kUsed = (d + kThreads - 1) / kThreads;  // norm blocks with entries
+    for (int b = blockIdx.x; b < kUsed; b += gridDim.x) {
+        const int t = b * kThreads + tid;
+        const V e = t < d ? psi_s[pad(t)] : V{0, 0};
+        const double re = (double)e.x, im = (double)e.y;
+        __syncthreads();  // red is free
+        const double s = block_sum(re * re + im * im, red);
+        if (tid == 0) tail.npart[b] = s;
+    }
+    __shared__ bool last;
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(tail.ticket, 1u) + 1u == gridDim.x;
+        __threadfence();
+    }
+    __syncthreads();
+    if (last && tid < 32)
+        finalize_warp(part, 0, ntiles, 0, 0, tail.npart, kUsed, N, 0, false, true, tail.res, tail.host, tail.d_m2,
+                      alpha);
 }
 
 // The same in the fixed-point mode: factors straight from global memory (the
@@ -237,58 +331,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restr
         fx_tile<NB>(v, buf, tid, un);
         const double s = block_sum(half_factor<fx>(alpha, un.c) * sum_order<fx>(v, alpha), red);
         if (tid == 0) part[g] = s;
-    }
-}
-
-// ------------------------------------------------------------- finalize
-
-// Fixed-order FP64 sum of two segments of partials by one warp: lane l adds
-// entries l, l+32, ... of each segment in order, then a fixed shuffle tree.
-// Shared by the single-state and the batch finalize, so a state's M2 is
-// bitwise the same in either.
-__device__ __forceinline__ double warp_sum_segments(const double *p, long long o1, long long n1,
-                                                    long long o2, long long n2) {
-    const int lane = threadIdx.x & 31;
-    double s = 0.0;
-    for (long long k = lane; k < n1; k += 32) s += p[o1 + k];
-    for (long long k = lane; k < n2; k += 32) s += p[o2 + k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    return s;  // valid in lane 0
-}
-
-__device__ __forceinline__ double m2_from(double S, double n2, int N, bool bad) {
-    // M2 = -log2(S / (d n2^4)), in logs so tiny norms do not underflow
-    return bad ? __longlong_as_double(0x7ff8000000000000ll)
-               : -(log2(S) - (double)N - 4.0 * log2(n2));
-}
-
-// Eq. (sre) at integer order alpha: M_alpha = log2(S / (d n2^(2 alpha))) /
-// (1 - alpha); order 2 is m2_from.
-__device__ __forceinline__ double malpha_from(double S, double n2, int N, int alpha, bool bad) {
-    if (alpha == 2) return m2_from(S, n2, N, bad);
-    return bad ? __longlong_as_double(0x7ff8000000000000ll)
-               : (log2(S) - (double)N - 2.0 * alpha * log2(n2)) / (1.0 - alpha);
-}
-
-// One warp: S from the partial segments [o1, o1+n1) and [o2, o2+n2), n2 from
-// the norm partials, M2 and the status.
-__global__ void k_finalize(const double *__restrict__ parts, long long o1, long long n1, long long o2,
-                           long long n2c, const double *__restrict__ npart, int nn, int N,
-                           const int *flags, const int *status, Result *res, double *d_m2,
-                           int alpha) {
-    const double S = warp_sum_segments(parts, o1, n1, o2, n2c);
-    const double n2 = warp_sum_segments(npart, 0, nn, 0, 0);
-    if (threadIdx.x == 0) {
-        int st = *status;
-        if (st == 0 && (*flags & kFlagNonFinite)) st = SRE_ENONFINITE;
-        if (st == 0 && !(n2 > 0.0)) st = SRE_EZERO;
-        const double m2 = malpha_from(S, n2, N, alpha, st != 0);
-        res->m2 = m2;
-        res->S = S;
-        res->n2 = n2;
-        res->status = st;
-        if (d_m2) *d_m2 = m2;
     }
 }
 
@@ -438,14 +480,12 @@ void workspace_free(Workspace *ws) {
     if (ws->ev_begin) cudaEventDestroy(ws->ev_begin);
     if (ws->ev_end) cudaEventDestroy(ws->ev_end);
     cudaFree(ws->npart);
-    cudaFree(ws->flags);
     cudaFree(ws->part);
     cudaFree(ws->scratch);
     cudaFree(ws->item_part);
     cudaFree(ws->chunk_sum);
     cudaFree(ws->counters);
     cudaFree(ws->work);
-    cudaFree(ws->status);
     cudaFree(ws->result);
     cudaFree(ws->conv);
     cudaFree(ws->tc_e);
@@ -470,11 +510,11 @@ cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int
         }                           \
     } while (0)
     SRE_TRY(cudaMalloc(&ws->npart, sizeof(double) * kNormBlocks));
-    SRE_TRY(cudaMalloc(&ws->flags, sizeof(int)));
     ws->part_cap = kTile;  // one partial per tile of an N <= 12 state
     SRE_TRY(cudaMalloc(&ws->part, sizeof(double) * ws->part_cap));
-    SRE_TRY(cudaMalloc(&ws->work, kWorkBytes));
-    SRE_TRY(cudaMalloc(&ws->status, sizeof(int)));
+    SRE_TRY(cudaMalloc(&ws->work, kWorkBytes + kFlagBytes));
+    ws->flags = reinterpret_cast<int *>(ws->work + kWorkBytes / 8);
+    ws->status = ws->flags + 1;
     SRE_TRY(cudaMalloc(&ws->fx_k, sizeof(FxUnits)));
     SRE_TRY(cudaMalloc(&ws->result, sizeof(Result)));
     if (N_max > kTileBits) {
@@ -512,7 +552,7 @@ template <typename R, int NB>
 static cudaError_t launch_small_nb(const void *psi, const void *const *psis, int nstates,
                                    uint64_t x_begin, uint64_t x_end, double *part, int part_cap,
                                    const DeviceInfo &dev, cudaStream_t st, int *nparts,
-                                   int forced_grid, int alpha, const int *fx_k) {
+                                   int forced_grid, int alpha, const int *fx_k, const SmallTail &tail) {
     constexpr bool kFx = sizeof(cx_t<R>) == 16;
     const size_t smem = (size_t)(kFx ? 1 : 3) * kTileSlots * sizeof(v2_t<R>);
     cudaError_t e;
@@ -533,7 +573,7 @@ static cudaError_t launch_small_nb(const void *psi, const void *const *psis, int
                                                      ntiles, part, alpha, reinterpret_cast<const FxUnits *>(fx_k));
     else
         k_small<R, NB><<<grid, kThreads, smem, st>>>(reinterpret_cast<const float2 *>(psi), psis, tps, x_begin, x_end,
-                                                     ntiles, part, alpha);
+                                                     ntiles, part, alpha, tail);
     *nparts = (int)ntiles;
     return cudaGetLastError();
 }
@@ -542,10 +582,10 @@ template <typename R>
 static cudaError_t launch_small(int N, const void *psi, const void *const *psis, int nstates,
                                 uint64_t xb, uint64_t xe, double *part, int part_cap,
                                 const DeviceInfo &dev, cudaStream_t st, int *nparts,
-                                int forced_grid, int alpha, const int *fx_k) {
+                                int forced_grid, int alpha, const int *fx_k, const SmallTail &tail = SmallTail()) {
     switch (N) {
 #define SRE_CASE(n) \
-    case n: return launch_small_nb<R, n - 1>(psi, psis, nstates, xb, xe, part, part_cap, dev, st, nparts, forced_grid, alpha, fx_k);
+    case n: return launch_small_nb<R, n - 1>(psi, psis, nstates, xb, xe, part, part_cap, dev, st, nparts, forced_grid, alpha, fx_k, tail);
         SRE_CASE(1) SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6)
         SRE_CASE(7) SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11) SRE_CASE(12)
 #undef SRE_CASE
@@ -676,6 +716,28 @@ cudaError_t enqueue_copy_sums(const Workspace &ws, double *d_out2, cudaStream_t 
     return cudaGetLastError();
 }
 
+// The workspace's words that start from zero: flags, status and ticket, which
+// follow the work-queue counters (with_work) in one allocation.
+static cudaError_t clear_words(const Workspace &ws, bool with_work, cudaStream_t st) {
+    return with_work ? cudaMemsetAsync(ws.work, 0, kWorkBytes + kFlagBytes, st)
+                     : cudaMemsetAsync(ws.flags, 0, kFlagBytes, st);
+}
+
+// One FP32 state with N <= 12, shifts [xb, xe): one kernel, result and all.
+static cudaError_t enqueue_small(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N, uint64_t xb,
+                                 uint64_t xe, cudaStream_t st, double *d_m2, int alpha) {
+    const cudaError_t e = clear_words(ws, false, st);
+    if (e != cudaSuccess) return e;
+    SmallTail tail;
+    tail.npart = ws.npart;
+    tail.ticket = reinterpret_cast<unsigned *>(ws.flags) + 2;
+    tail.res = ws.result;
+    tail.host = ws.host_result;
+    tail.d_m2 = d_m2;
+    int np = 0;
+    return launch_small<float>(N, psi, nullptr, 1, xb, xe, ws.part, ws.part_cap, dev, st, &np, 0, alpha, nullptr, tail);
+}
+
 template <typename R>
 static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N,
                                 uint64_t x_begin, uint64_t x_end, cudaStream_t st, double *d_m2,
@@ -684,8 +746,16 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
     cudaError_t e;
     constexpr bool kFx = sizeof(cx_t<R>) == 16;
     const uint64_t d = 1ull << N;
-    if ((e = cudaMemsetAsync(ws.flags, 0, sizeof(int), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ws.status, 0, sizeof(int), st)) != cudaSuccess) return e;
+    if constexpr (!kFx)
+        if (N <= kTileBits) {
+            if (ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
+            if ((e = enqueue_small(ws, dev, psi, N, x_begin, x_end, st, d_m2, alpha)) != cudaSuccess) return e;
+            if (ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
+            ws.main_kernel = "k_small";
+            ws.launches += 1;
+            return cudaSuccess;
+        }
+    if ((e = clear_words(ws, N > kTileBits, st)) != cudaSuccess) return e;
     k_norm<<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart, ws.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ws.launches += 2;  // k_norm + k_finalize
@@ -706,7 +776,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         int np = 0;
         if (ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
         if ((e = launch_small<R>(N, psi, nullptr, 1, x_begin, x_end, ws.part, ws.part_cap, dev, st,
-                                 &np, 0, alpha, kFx ? ws.fx_k : nullptr)) != cudaSuccess)
+                                 &np, 0, alpha, ws.fx_k)) != cudaSuccess)
             return e;
         if (ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
         ws.main_kernel = "k_small";
@@ -715,19 +785,21 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         nparts = np;
     } else {
         const int eb = (int)sizeof(v2_t<R>);
-        if ((e = cudaMemsetAsync(ws.counters, 0, sizeof(unsigned) * 3 * ws.chunk_cap, st)) != cudaSuccess)
-            return e;
-        if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;
         // every shift in one launch, or with the tensor-core kernel on the
         // shifts from 4096 up those below it
         const bool tc = tc_kind && tc_applies(N, 1, alpha, psi);
         const uint64_t split = tc ? std::min<uint64_t>(std::max<uint64_t>(x_begin, kTile), x_end) : x_end;
+        const bool single_pass = one_applies(N, eb) || mid_applies(N, eb);
+        // chunk counters: not for a shift per CTA
+        if ((tc || !single_pass) &&
+            (e = cudaMemsetAsync(ws.counters, 0, sizeof(unsigned) * 3 * ws.chunk_cap, st)) != cudaSuccess)
+            return e;
         size_t chunks = 0;
         if (x_begin < split) {
             const bool timed = split == x_end;
             if (timed && ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
             const char *name;
-            if (one_applies(N, eb) || mid_applies(N, eb)) {
+            if (single_pass) {
                 // a shift in one CTA, one partial per shift
                 name = kFx ? "k_mid" : "k_one";
                 chunks = (size_t)(split - x_begin);
@@ -778,7 +850,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         nparts = (long long)chunks;
     }
     k_finalize<<<1, 32, 0, st>>>(parts, 0, seg1, seg1, nparts - seg1, ws.npart, kNormBlocks, N,
-                                 ws.flags, ws.status, ws.result, d_m2, alpha);
+                                 ws.flags, ws.status, ws.result, ws.host_result, d_m2, alpha);
     return cudaGetLastError();
 }
 
@@ -786,33 +858,18 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
 // single-state path's kernels, on scratch that the caller hands in.
 cudaError_t enqueue_m2_fixed(const Workspace &ws, const DeviceInfo &dev, const void *psi, int N, cudaStream_t st,
                              double *d_m2, long long wait_ns) {
-    using R = float;
     cudaError_t e;
     const uint64_t d = 1ull << N;
-    if ((e = cudaMemsetAsync(ws.flags, 0, sizeof(int), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ws.status, 0, sizeof(int), st)) != cudaSuccess) return e;
-    k_norm<<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart, ws.flags);
+    if (N <= kTileBits) return enqueue_small(ws, dev, psi, N, 0, d, st, d_m2, 2);
+    if (!one_applies(N, 8) || d > ws.chunk_cap) return cudaErrorInvalidValue;
+    if ((e = clear_words(ws, true, st)) != cudaSuccess) return e;
+    k_norm<<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const float2 *>(psi), d, ws.npart, ws.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    long long nparts = 0;
-    const double *parts = nullptr;
-    if (N <= kTileBits) {
-        int np = 0;
-        if ((e = launch_small<R>(N, psi, nullptr, 1, 0, d, ws.part, ws.part_cap, dev, st, &np, 0, 2,
-                                 nullptr)) != cudaSuccess)
-            return e;
-        parts = ws.part;
-        nparts = np;
-    } else {
-        if (!one_applies(N, 8) || d > ws.chunk_cap) return cudaErrorInvalidValue;
-        if ((e = cudaMemsetAsync(ws.work, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
-        if ((e = launch_one(N, psi, nullptr, 1, 0, d, 2, ws.chunk_sum, nullptr, ws.work, ws.status, wait_ns, dev,
-                            st)) != cudaSuccess)
-            return e;
-        parts = ws.chunk_sum;
-        nparts = (long long)d;
-    }
-    k_finalize<<<1, 32, 0, st>>>(parts, 0, nparts, nparts, 0, ws.npart, kNormBlocks, N, ws.flags, ws.status,
-                                 ws.result, d_m2, 2);
+    if ((e = launch_one(N, psi, nullptr, 1, 0, d, 2, ws.chunk_sum, nullptr, ws.work + 2, ws.status, wait_ns, dev,
+                        st)) != cudaSuccess)
+        return e;
+    k_finalize<<<1, 32, 0, st>>>(ws.chunk_sum, 0, (long long)d, (long long)d, 0, ws.npart, kNormBlocks, N, ws.flags,
+                                 ws.status, ws.result, nullptr, d_m2, 2);
     return cudaGetLastError();
 }
 

@@ -44,9 +44,7 @@ constexpr size_t kOffChunk = 0;
 constexpr size_t kOffPart = align_up(kOffChunk + sizeof(double) * kChunkCap);
 constexpr size_t kOffNorm = align_up(kOffPart + sizeof(double) * kPartCap);
 constexpr size_t kOffWork = align_up(kOffNorm + sizeof(double) * sre::kNormBlocks);
-constexpr size_t kOffStatus = align_up(kOffWork + sizeof(unsigned long long));
-constexpr size_t kOffFlags = align_up(kOffStatus + sizeof(int));
-constexpr size_t kOffResult = align_up(kOffFlags + sizeof(int));
+constexpr size_t kOffResult = align_up(kOffWork + sre::kWorkBytes + sre::kFlagBytes);
 constexpr size_t kNoAllocBytes = align_up(kOffResult + sizeof(sre::Result));  // about 0.56 MB
 
 }  // namespace
@@ -114,8 +112,8 @@ extern "C" sre_status_t sre_m2_noalloc(const void *d_state, int N, sre_stream_t 
     ws.part_cap = (int)kPartCap;
     ws.npart = reinterpret_cast<double *>(base + kOffNorm);
     ws.work = reinterpret_cast<unsigned long long *>(base + kOffWork);
-    ws.status = reinterpret_cast<int *>(base + kOffStatus);
-    ws.flags = reinterpret_cast<int *>(base + kOffFlags);
+    ws.flags = reinterpret_cast<int *>(base + kOffWork + sre::kWorkBytes);
+    ws.status = ws.flags + 1;
     ws.result = reinterpret_cast<sre::Result *>(base + kOffResult);
 
     const cudaError_t e = sre::enqueue_m2_fixed(ws, g_info[dev], d_state, N, (cudaStream_t)stream, d_m2, 5000000000ll);
