@@ -438,7 +438,7 @@ def run_modes(binding, torch, W, N, head_mode, head, peaks):
         r["pauli_terms_per_s"] = float(d) * d / (r["ms"] * 1e-3)
         r["abs_diff_vs_oracle"] = abs(r["m2"] - ref) if ref is not None else None
         if mode == "fp32":
-            r["alu_roofline_frac"] = (2 * N + 11) * float(d) * (d - 4096) / (kms_m * 1e-3) / alu_peak
+            r["alu_roofline_frac"] = (2 * N + 11) * float(d) * d / (kms_m * 1e-3) / alu_peak
         else:
             flops = tc_mma_flops(N)
             r["mma_flops_executed"] = flops
@@ -451,7 +451,7 @@ def run_modes(binding, torch, W, N, head_mode, head, peaks):
         out[mode]["vs_fp32_kernel_time"] = out[mode]["kernel_ms"] / out["fp32"]["kernel_ms"]
     out["note"] = ("split modes: both passes' Hadamard stages as tcgen05 MMAs (pass 1: 4 register bits, one "
                    "H_128 stage, one accumulator butterfly; pass 2: one H_128 or I x H_{2^h2} stage) on "
-                   "fixed-point hi/lo pieces, FP32 accumulate in TMEM; kernel_ms is the launch of the halved "
+                   "fixed-point hi/lo pieces, FP32 accumulate in TMEM; kernel_ms is the launch of the "
                    "shifts x >= 4096 alone; tensor peak = measured bf16 sustained (burst alongside)")
     return out
 
@@ -551,8 +551,6 @@ def run_tfim(binding, torch, W, cases=((14, 100, 10), (16, 100, 3)), dt=0.2):
 # evaluation.  Valid only for that kernel build and tuning; any other run
 # reports null.
 TRAFFIC = {
-    # FP32 CUDA-core two-pass kernel, its autotuned tuning (read + written on the slice)
-    ("fp32", (0, 47, 23, 3, 3)): 45.449725e9 + 61.593259e9,
     # tensor-core kernel, FP16 pieces, the tunings its autotuner picks
     # (read + written on the slice)
     ("fp16_split", (3, 6, 2, 4, 0)): 45.709644e9 + 59.002857e9,
@@ -690,9 +688,9 @@ def run_gpu(args):
     max_mhz = clocks.get("sm_max_mhz") or peaks.get("sm_max_mhz", 2070.0)
     # FP32 ALU roofline: SMs x 128 FP32 lanes x max SM clock (one add / mul /
     # fma per lane per clock); algorithmic ops (2N + 11) d per Pauli term,
-    # over the terms of the timed launch (the halved shifts x >= 4096; the
-    # plan's profiling events bracket that launch alone)
-    timed_terms = float(d) * (d - 4096) if N > 12 else terms
+    # over the terms of the timed launch (every shift, in the split modes those
+    # from 4096; the plan's profiling events bracket that launch alone)
+    timed_terms = float(d) * (d - 4096) if kname == "k_tc" else terms
     alg_ops = (2 * N + 11) * timed_terms
     kern_s = statistics.mean(kern_ms) / 1000.0
     if args.mode == "fp64":

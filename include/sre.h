@@ -81,13 +81,17 @@ typedef enum {
  * 2^11 for fp16) and the remainder rounded to the 16-bit type as the low
  * piece.  The Hadamard matrix is +-1, so the high piece's sums are exact in
  * the FP32 accumulator and the low piece adds the next 8 (bf16) or 11
- * (fp16) significant bits; the remaining shifts run in FP32.  Value 3 is unused (a tf32 split would need the same two
- * pieces at half the bf16 tensor rate and twice the operand bytes). */
+ * (fp16) significant bits; the remaining shifts run in FP32.  The FP64 mode
+ * forms products and powers in FP64 and runs the butterflies between them in
+ * 64-bit fixed point, on units that bound the whole transform (no rounding in
+ * a butterfly but the rescaling between groups of stages).  Value 3 is unused
+ * (a tf32 split would need the same two pieces at half the bf16 tensor rate
+ * and twice the operand bytes). */
 typedef enum {
     SRE_MODE_FP32 = 0,       /* CUDA-core FP32 butterflies */
     SRE_MODE_BF16_SPLIT = 1, /* tensor-core Hadamard stages, bf16 hi/lo fixed-point split */
     SRE_MODE_FP16_SPLIT = 2, /* tensor-core Hadamard stages, fp16 hi/lo fixed-point split */
-    SRE_MODE_FP64 = 4,       /* CUDA-core FP64 everywhere */
+    SRE_MODE_FP64 = 4,       /* FP64 products and powers, 64-bit fixed-point butterflies */
     SRE_MODE_AUTO = -1       /* the plan's tuned default */
 } sre_mode_t;
 
@@ -120,9 +124,9 @@ SRE_API sre_status_t sre_plan_set_mode(sre_plan_t plan, sre_mode_t mode);
 SRE_API sre_status_t sre_plan_get_mode(sre_plan_t plan, sre_mode_t *mode);
 
 /*
- * Tuning of the two-pass kernel used for N > 12 (one pass transforms the
- * low 12 bits of t per block into an L2-resident ring of scratch, the other
- * the remaining bits).  x_batch_log: log2 of the shifts that share one
+ * Tuning of the two-pass kernels (FP32 N >= 17, FP64 N >= 15, the split
+ * modes' shifts x >= 4096 at 16 <= N <= 20): one pass transforms the low bits
+ * of t per block into a ring of scratch, the other the remaining bits.  x_batch_log: log2 of the shifts that share one
  * pass-1 partner block (0..3); ring_slots: chunks held in the ring (>= 2);
  * lag: how many chunks pass 2 trails pass 1 (1 <= lag < ring_slots);
  * pass2_tiles_log: log2 of the 2^12-entry tiles per pass-2 work item;
@@ -132,11 +136,15 @@ SRE_API sre_status_t sre_plan_get_mode(sre_plan_t plan, sre_mode_t *mode);
  * copy into shared memory (FP32 CUDA-core path, x_batch_log = 0 and a
  * 16-byte aligned state; otherwise, or with 0, per-thread loads);
  * pass2_staged (0/1): pass 2 takes its tiles by 2-D tensor-memory-accelerator
- * copies into shared memory (FP32, 17 <= N <= 21; otherwise, or with 0,
+ * copies into shared memory (FP32, N = 21; otherwise, or with 0,
  * per-thread loads).
  * A value of -1 keeps the library's choice for that field; all -1 restores
- * the defaults.  The scratch ring must fit the plan's allocation
- * (SRE_EINVAL otherwise).  Applies to the halved shifts (x >= 4096).
+ * the defaults.  With one of x_batch_log, ring_slots and lag given, the others
+ * keep those of an L2-sized ring.  The scratch ring must fit the plan's
+ * allocation (SRE_EINVAL otherwise).  FP32 with 17 <= N <= 20 takes x_batch_log
+ * and ring_slots alone (work is handed out as it becomes possible), the
+ * staging fields apply to FP32 with N >= 21, and the sizes that run in one
+ * pass (FP32 N <= 16, FP64 N <= 14) take none.
  */
 typedef struct {
     int x_batch_log;
@@ -155,17 +163,17 @@ SRE_API sre_status_t sre_plan_get_tuning(sre_plan_t plan, int N, sre_tuning_t *t
  * candidate tunings on a bounded slice of shifts of a synthetic state held in
  * the plan, keep the fastest and make it the plan's tuning for that N.
  * SYNCHRONOUS (uses `stream`).  *best receives the chosen tuning and *ms its
- * time on the slice (either may be NULL).  N <= 12 has nothing to tune
- * (SRE_OK, tuning left unchanged).
+ * time on the slice (either may be NULL).  FP32 N <= 15 and FP64 N <= 14 have
+ * nothing to tune (SRE_OK, tuning left unchanged).
  */
 SRE_API sre_status_t sre_plan_autotune(sre_plan_t plan, int N, sre_stream_t stream,
                                        sre_tuning_t *best, double *ms);
 
 /* Profiling support.  When enabled (enable != 0), the plan records two CUDA
  * events on the stream around the main transform launch of each
- * evaluation: for N > 12 the launch of the conjugate-symmetry halved
- * shifts x >= 4096 (k_large, k_mid or k_tc; 99.6 % of the shifts at
- * N = 20), else the single-tile kernel.  sre_plan_last_kernel_ms waits for
+ * evaluation: the launch of every shift (k_small, k_one, k_two, k_mid or
+ * k_large), in the split modes that of the shifts x >= 4096 (k_tc; 99.6 % of
+ * the shifts at N = 20).  sre_plan_last_kernel_ms waits for
  * the second event and returns the elapsed milliseconds of the last
  * evaluation's main launch and its kernel's name (static string).  sre_plan_launch_count returns the number of kernels
  * the plan has launched since it was created (its own kernels only). */
@@ -333,11 +341,11 @@ SRE_API sre_status_t sre_m2_batched(sre_plan_t plan, const void *const *d_states
  *            aligned, 1 <= N <= SRE_NOALLOC_MAX_QUBITS (16); larger N is
  *            rejected with SRE_EINVAL before anything is launched.
  *   d_m2:    device double receiving M2; NaN for a zero / non-finite state,
- *            and NaN as well when a device wait of the two-pass kernel
+ *            and NaN as well when a device wait of the kernel
  *            expires (fixed limit of 5 s): the status the kernel records
  *            stays in the library's own array, out of the caller's reach.
  * Asynchronous on `stream`.  Its only scratch is one fixed module array of
- * about 5.4 MB that every GPU loading the library holds until exit; a call
+ * about 0.56 MB that every GPU loading the library holds until exit; a call
  * made while `stream` is not being captured looks up that array's address
  * (so a call after cudaDeviceReset finds the reloaded array), a call during
  * a capture reuses the address found before, so the first call with a
@@ -350,7 +358,7 @@ SRE_API sre_status_t sre_m2_noalloc(const void *d_state, int N, sre_stream_t str
 
 /*
  * Failure-detection self test: launch one CTA that waits, with the same
- * bounded wait the two-pass kernel uses, on a device counter that nothing
+ * bounded wait the two-pass kernels use, on a device counter that nothing
  * increments.  The wait gives up after wait_ns of GPU time and the call
  * returns the status the kernel recorded (SRE_ETIMEDOUT when the bound
  * works).  SYNCHRONOUS on `stream`; the device context stays usable.
@@ -404,11 +412,12 @@ SRE_API void sre_server_cfg_default(sre_server_cfg_t *cfg);
 SRE_API sre_status_t sre_server_create(const sre_server_cfg_t *cfg, sre_server_t *out);
 
 /*
- * Tuning of the two-pass kernel for requests of N qubits (13 <= N <= the
+ * Tuning of the two-pass kernels for requests of N qubits (13 <= N <= the
  * server's max_N; fields as sre_tuning_t for sre_plan_set_tuning, -1 keeps
- * the library's choice), applied to the halved shifts of every later unit
- * of that N.  The ring must fit each slot's scratch (SRE_EINVAL otherwise;
- * see slot_scratch_bytes).  Thread-safe.
+ * the library's choice), applied to every later unit of that N.  The
+ * ring must fit each slot's scratch (SRE_EINVAL otherwise; see
+ * slot_scratch_bytes); a plan's library choice, which sre_plan_get_tuning
+ * returns, stands for the slot's own.  Thread-safe.
  */
 SRE_API sre_status_t sre_server_set_tuning(sre_server_t srv, int N, const sre_tuning_t *tuning);
 

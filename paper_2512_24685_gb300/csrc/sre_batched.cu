@@ -2,8 +2,8 @@
 //
 // States are grouped in classes of equal N (largest first).  Each class is
 // one persistent launch that walks the concatenated work list of all its
-// states (the single-tile kernel for N <= 12; for N > 12 the two-pass
-// kernel, once for shifts below 4096 and once for the halved shifts).  A norm
+// states: the kernel that the size and mode take alone, and in the split modes
+// for 16 <= N <= 20 one more for the shifts below 4096.  A norm
 // launch covers all states and a finalize launch turns each state's
 // fixed-order partial sums into M2, so every result is bitwise the same as
 // for that state alone in a batch of equal composition.

@@ -13,8 +13,8 @@ BatchedContext *batched_create(const DeviceInfo &dev);
 void batched_destroy(BatchedContext *ctx);
 
 // M2 of `count` states (device pointers, uneven N) into d_m2_out[count].
-// tuned_half[N] (may be null, or hold nulls) gives autotuned two-pass
-// configurations of the halved shifts per N.  d_status_out (device, may be
+// tuned_half[N] (may be null, or hold nulls) gives the two-pass
+// configurations per N.  d_status_out (device, may be
 // null) receives each state's sre_status_t (SRE_ETIMEDOUT for every state
 // of a batch in which a device wait expired).
 cudaError_t batched_run(BatchedContext *ctx, const Workspace &ws, const DeviceInfo &dev,

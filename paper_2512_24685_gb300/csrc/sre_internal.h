@@ -85,13 +85,12 @@ struct DeviceInfo {
 
 cudaError_t query_device(DeviceInfo *info);
 
-// Pick the two-pass configuration for N > 12 (half: conjugate-symmetry halved
-// shifts, x >= 4096).
+// The L2-sized two-pass configuration for N > 12 (half: transforms of 2^(N-1)
+// entries).
 LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half);
 
 // The library's two-pass configuration for the main shift range of an
-// arithmetic mode (the halved shifts, or all shifts where sre_two.cu takes
-// them), and whether a configuration fits a workspace.
+// arithmetic mode (every shift, in the split modes those from 4096), and whether a configuration fits a workspace.
 LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode);
 // The configuration that a caller's partial tuning completes: with a ring field
 // of the caller's own, the L2-sized one, whose lag and slots leave room for it.

@@ -7,7 +7,8 @@
 //
 // Kernels
 //   k_convert   element-type conversion of the state (complex128 <-> complex64)
-//   k_norm      n2 = <psi|psi> in FP64 + NaN/Inf detection (fixed grid)
+//   k_norm      n2 = <psi|psi> in FP64 + NaN/Inf detection (fixed grid); a
+//               single FP32 state with N <= 12 has it from k_small
 //   k_small     N <= 12, FP32: one 2^12-entry tile holds 2^(13-N) whole shifts
 //               (halved form); the state sits in shared memory; static
 //               tile->CTA assignment.  k_small_fx: the same in fixed point

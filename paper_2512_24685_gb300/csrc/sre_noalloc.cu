@@ -11,8 +11,9 @@
 //
 // The array belongs to the module: every GPU that loads the library holds
 // its kNoAllocBytes until the process exits, and every call on a device uses
-// the same array.  The words that must start at zero (status, flags) are cleared on the stream by each call; the rest is overwritten
-// before it is read.  Two calls whose work overlaps on the GPU (different
+// the same array.  The words that must start at zero (counters, status, flags)
+// are cleared on the stream by each call; the rest is overwritten before it
+// is read.  Two calls whose work overlaps on the GPU (different
 // streams, or host threads racing on one stream) therefore race on the
 // array; calls that are ordered on the GPU are safe.
 //
