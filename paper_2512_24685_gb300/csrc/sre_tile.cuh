@@ -133,9 +133,14 @@ __device__ __forceinline__ int fx_log(double m) {
 // Smallest k with 2^(l / 256) <= 2^k.
 __device__ __forceinline__ int fx_exponent(int l) { return l >= kFxNonFinite / 2 ? kFxNonFinite : (l + 255) >> 8; }
 
-// From unit 2^(k1 - 63) to the coarser 2^(k2 - 63), q = k2 - k1, rounded.
-__device__ __forceinline__ long long fx_shift(long long a, int q) {
-    return q <= 0 ? a : q > 62 ? 0 : (a + (1ll << (q - 1))) >> q;
+// From unit 2^(k1 - 63) to the coarser 2^(k2 - 63), q = k2 - k1, rounded half
+// up: the last bit shifted out is added afterwards, since a + 2^(q - 1) leaves 64
+// bits for a near full scale.
+__host__ __device__ __forceinline__ long long fx_shift(long long a, int q) {
+    if (q <= 0) return a;
+    if (q > 62) return 0;
+    const long long t = a >> (q - 1);
+    return (t >> 1) + (t & 1);
 }
 
 // round(p 2^(63 - k)), |p| < 2^k.  The mantissa, 10 bits up, moves right by
