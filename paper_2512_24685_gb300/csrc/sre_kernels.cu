@@ -236,7 +236,6 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
     constexpr int d = 1 << N;
     const int tid = threadIdx.x;
 
-    const double hfac = half_factor<R>(alpha, 0);
     long long cur = -1;
     for (long long g = blockIdx.x; g < ntiles; g += gridDim.x) {
         const long long sidx = psis ? g / tiles_per_state : 0;
@@ -265,7 +264,7 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
         }
         tile_fwht<NB, R>(v, bufA, bufB, tid);
         // block_sum's barriers also protect bufB before the next tile
-        const double s = block_sum(hfac * (double)sum_order<R>(v, alpha), red);
+        const double s = block_sum(half_scale<R>((double)sum_order<R>(v, alpha), alpha, 0), red);
         if (tid == 0) part[g] = s;
     }
     if (!tail.npart) return;
@@ -330,8 +329,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restr
             for (int i = 0; i < 16; ++i) v[i] = value(i, std::false_type());
         }
         fx_tile<NB>(v, buf, tid, un);
-        const double s = block_sum(half_factor<fx>(alpha, un.c) * sum_order<fx>(v, alpha), red);
-        if (tid == 0) part[g] = s;
+        const double s = block_sum(sum_order<fx>(v, alpha), red);
+        if (tid == 0) part[g] = half_scale<fx>(s, alpha, un.c);
     }
 }
 

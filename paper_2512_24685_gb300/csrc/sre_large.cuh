@@ -375,7 +375,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
             const int zb0 = (j & ((1 << ipx_log) - 1)) << a.G2_log;
             const uint64_t x = xc + (uint64_t)xl;
             double acc = 0.0;
-            const double hfac = half_factor<R>(a.alpha, fxk);
             const bool staged2 = kTma && a.stage2;
             if constexpr (kTma) {
                 // One thread waits for the chunk's pass 1 and keeps two TMA
@@ -425,7 +424,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         }
                         const unsigned char *stage = reinterpret_cast<const unsigned char *>(st ? bufC : bufB);
                         const float s = p2_tile<H2>(stage, reinterpret_cast<float2 *>(bufA), pl, a.alpha);
-                        acc += hfac * (double)s;
+                        acc += half_scale<R>((double)s, a.alpha, 0);
                         if (gb + 2 < ntiles) {
                             __syncthreads();  // every thread has read stage st
                             if (tid == 0) {
@@ -461,12 +460,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         if (kFx) __syncthreads();  // one buffer: the previous tile's readers are done
                     }
                     tile_fwht<H2, R>(v, bufA, bB, tid);
-                    acc += hfac * (double)sum_order<R>(v, a.alpha);
+                    if constexpr (kFx)
+                        acc += sum_order<R>(v, a.alpha);
+                    else
+                        acc += half_scale<R>((double)sum_order<R>(v, a.alpha), a.alpha, 0);
                 }
             }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+            if constexpr (kFx) acc = half_scale<R>(acc, a.alpha, fxk);
             // All warps' loads of this item are complete after this barrier:
             // drop the item's scratch lines from L2 without write-back (dead
             // data; the next chunk in this slot rewrites them; the staged path

@@ -66,8 +66,9 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 2 : 1)
             s = sum_order<fx>(w, alpha);
         }
         s += sum_order<fx>(v, alpha);
-        const double tot = block_sum(half_factor<fx>(alpha, k) * s, red);
+        const double units = block_sum(s, red);
         if (tid == 0) {
+            const double tot = half_scale<fx>(units, alpha, k);
             part[g] = tot;
             if (per_x) per_x[g] = tot;
         }

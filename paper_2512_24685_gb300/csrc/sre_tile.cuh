@@ -187,14 +187,16 @@ __device__ __forceinline__ cx_t<R> pair_value(v2_t<R> b, v2_t<R> a, int k) {
         return make_longlong2(fx_from(re, k), fx_from(im, k));
 }
 
-// Factor of a partial sum of (Re W)^(2 alpha) + (Im W)^(2 alpha): 2^(2 alpha)
-// for the halving, and the fixed-point unit 2^k to the same power (NaN for a
-// state without a finite norm, whose fixed-point values mean nothing).
+// A sum of (Re W)^(2 alpha) + (Im W)^(2 alpha) over FP32 values, times 2^(2 alpha)
+// for the halving; over fixed-point values of unit exponent k, times the unit
+// 2^k to the same power as well (NaN for a state without a finite norm, whose
+// fixed-point values mean nothing).  The power alone may leave the range of a
+// double where its product with the sum does not.
 template <typename R>
-__device__ __forceinline__ double half_factor(int alpha, int k) {
-    if constexpr (sizeof(cx_t<R>) == 8) return (double)(1ull << (2 * alpha));
+__device__ __forceinline__ double half_scale(double s, int alpha, int k) {
+    if constexpr (sizeof(cx_t<R>) == 8) return (double)(1ull << (2 * alpha)) * s;
     if (k == kFxNonFinite) return __longlong_as_double(0x7ff8000000000000ll);
-    return scalbn(1.0, 2 * alpha * (1 + k));
+    return scalbn(s, 2 * alpha * (1 + k));
 }
 
 // Where one shift finds the factors of a 4096-entry block of t' (t with the
