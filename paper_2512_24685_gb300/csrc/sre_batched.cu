@@ -67,11 +67,9 @@ struct BatchedContext {
     size_t flags_cap = 0;
     unsigned *counters = nullptr;
     size_t counters_cap = 0;  // 3 * chunk capacity
-    int *tc_e = nullptr;      // split and FP64 modes: per-state scale tables of a class
+    int *tc_e = nullptr;      // split modes: per-state scale tables of a class
     double *tc_bn = nullptr;
     size_t tc_e_cap = 0, tc_bn_cap = 0;
-    int *fx_k = nullptr;      // FP64 mode: three unit exponents per state
-    size_t fx_cap = 0;
     unsigned long long generation = 1;
     std::vector<GraphEntry> graphs;  // most recent last
 };
@@ -101,7 +99,6 @@ void batched_destroy(BatchedContext *ctx) {
     cudaFree(ctx->counters);
     cudaFree(ctx->tc_e);
     cudaFree(ctx->tc_bn);
-    cudaFree(ctx->fx_k);
     delete ctx;
 }
 
@@ -125,15 +122,14 @@ static cudaError_t enqueue_entry(BatchedContext *ctx, const Workspace &ws, const
             off += eb << g.Ns[i];
         }
     }
-    if ((e = enqueue_batch_norm(ws, g.d_ptrs, g.d_Ns, count, ctx->npart, ctx->flags, ctx->fx_k, g.mode, st)) !=
+    if ((e = enqueue_batch_norm(ws, g.d_ptrs, g.d_Ns, count, ctx->npart, ctx->flags, g.mode, st)) !=
         cudaSuccess)
         return e;
     size_t first = 0;
     for (const BatchClass &L : classes) {
         if ((e = enqueue_batch_class(ws, dev, L, g.d_ptrs + first, ctx->parts, ctx->counters, chunk_cap,
                                      g.mode, st, wait_ns, ctx->tc_e, ctx->tc_bn,
-                                     std::min(ctx->tc_e_cap, ctx->tc_bn_cap),
-                                     fp64 ? ctx->fx_k + 3 * first : nullptr)) != cudaSuccess)
+                                     std::min(ctx->tc_e_cap, ctx->tc_bn_cap))) != cudaSuccess)
             return e;
         first += (size_t)L.S;
     }
@@ -210,14 +206,13 @@ cudaError_t batched_run(BatchedContext *ctx, const Workspace &ws, const DeviceIn
     }
 
     // ---- shared buffers (a reallocation invalidates every captured graph)
-    const size_t gen0 = ctx->parts_cap + ctx->npart_cap + ctx->flags_cap + ctx->counters_cap + ctx->fx_cap;
+    const size_t gen0 = ctx->parts_cap + ctx->npart_cap + ctx->flags_cap + ctx->counters_cap;
     if ((e = grow(&ctx->parts, &ctx->parts_cap, parts_total)) != cudaSuccess) return e;
     if ((e = grow(&ctx->npart, &ctx->npart_cap, (size_t)count * kNormBlocks)) != cudaSuccess) return e;
     if ((e = grow(&ctx->flags, &ctx->flags_cap, (size_t)count)) != cudaSuccess) return e;
     if ((e = grow(&ctx->counters, &ctx->counters_cap, 3 * chunk_cap)) != cudaSuccess) return e;
-    if ((e = grow(&ctx->fx_k, &ctx->fx_cap, (size_t)count * 3)) != cudaSuccess) return e;
     chunk_cap = ctx->counters_cap / 3;
-    if (ctx->parts_cap + ctx->npart_cap + ctx->flags_cap + ctx->counters_cap + ctx->fx_cap != gen0) ++ctx->generation;
+    if (ctx->parts_cap + ctx->npart_cap + ctx->flags_cap + ctx->counters_cap != gen0) ++ctx->generation;
 
     // ---- the entry with its own device tables
     if (ctx->graphs.size() >= 8) {
@@ -250,8 +245,7 @@ cudaError_t batched_run(BatchedContext *ctx, const Workspace &ws, const DeviceIn
     {
         size_t tc_need = 0;
         for (const BatchClass &L : classes)
-            if (L.tc_kind || (fp64 && L.N > kTileBits))
-                tc_need = std::max(tc_need, (size_t)L.S << (L.N - kTileBits));
+            if (L.tc_kind) tc_need = std::max(tc_need, (size_t)L.S << (L.N - kTileBits));
         const size_t tc0 = ctx->tc_e_cap + ctx->tc_bn_cap;
         if (tc_need && ((e = grow(&ctx->tc_e, &ctx->tc_e_cap, tc_need)) != cudaSuccess ||
                         (e = grow(&ctx->tc_bn, &ctx->tc_bn_cap, tc_need)) != cudaSuccess)) {

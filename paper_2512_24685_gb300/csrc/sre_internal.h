@@ -67,9 +67,10 @@ struct Workspace {
     void *conv = nullptr;          // state converted to the compute type (lazy)
     size_t conv_bytes = 0;
     int *tc_e = nullptr;           // tensor-core path: scale exponent per x >> 12
-    double *tc_bn = nullptr;       // tensor-core path: l2 norm per 4096-entry block (FP64 mode: its bounds)
+    double *tc_bn = nullptr;       // tensor-core path: l2 norm per 4096-entry block
     int tc_cap = 0;                // entries of tc_e / tc_bn
-    int *fx_k = nullptr;           // FP64 mode, N <= 12: the state's unit exponents (FxUnits)
+    short *fx_exp = nullptr;       // FP64 mode, N > 12: units and bounds of the ring's blocks (FxExp)
+    size_t fx_cap = 0;             // blocks
     // profiling: events recorded around the main transform kernel when set
     cudaEvent_t ev_begin = nullptr, ev_end = nullptr;
     mutable const char *main_kernel = "";
@@ -152,9 +153,9 @@ cudaError_t enqueue_batch_class(const Workspace &ws, const DeviceInfo &dev, cons
                                 const void *const *d_ptrs, double *parts, unsigned *counters,
                                 size_t chunk_cap, sre_mode_t mode, cudaStream_t st,
                                 long long wait_ns, int *tc_e = nullptr, double *tc_bn = nullptr,
-                                size_t tc_cap = 0, const int *fx_k = nullptr);
+                                size_t tc_cap = 0);
 cudaError_t enqueue_batch_norm(const Workspace &ws, const void *const *d_ptrs, const int *d_Ns,
-                               int count, double *npart, int *flags, int *fx_k, sre_mode_t mode,
+                               int count, double *npart, int *flags, sre_mode_t mode,
                                cudaStream_t st);
 cudaError_t enqueue_batch_finalize(const Workspace &ws, const void *seg, const double *parts,
                                    const double *npart, const int *flags, const int *d_Ns,
@@ -170,13 +171,7 @@ cudaError_t enqueue_malpha_from_sums(const double *S, const double *n2, int N, i
 // state).
 bool mid_applies(int N, int elem_bytes);
 cudaError_t launch_mid(int N, const void *psi, const void *const *psis, int nstates, long long sps, uint64_t x_begin,
-                       int alpha, double *part, double *per_x, const int2 *fx_bn, const int *fx_e,
-                       const DeviceInfo &dev, cudaStream_t st);
-// Scale tables of the FP64 mode for N > 12: bounds (fx_bound) per 4096-entry
-// block, and unit exponent per x >> 12, of nstates states (2^(N - 12)
-// entries each).
-cudaError_t enqueue_fx_scales(const void *psi, const void *const *psis, int nstates, int N, int2 *bn, int *e,
-                              cudaStream_t st);
+                       int alpha, double *part, double *per_x, const DeviceInfo &dev, cudaStream_t st);
 
 // Brickwork circuit dynamics (sre_evolve.cu): S complex128 states of N
 // qubits set to |0...0>; one step t of even-bond then odd-bond gates.

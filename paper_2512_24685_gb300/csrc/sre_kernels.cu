@@ -12,7 +12,6 @@
 //   k_small     N <= 12, FP32: one 2^12-entry tile holds 2^(13-N) whole shifts
 //               (halved form); the state sits in shared memory; static
 //               tile->CTA assignment.  k_small_fx: the same in fixed point
-//   k_fx_*      fixed point: unit exponents of a state, block or shift
 //   k_large     fixed point N >= 15, FP32 N >= 21: persistent two-pass kernel
 //               (sre_large.cuh); the sizes between run in sre_mid.cu,
 //               sre_one.cu and sre_two.cu
@@ -69,70 +68,6 @@ __global__ void __launch_bounds__(kThreads) k_norm(const V *__restrict__ psi, ui
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flags, kFlagNonFinite);
     const double b = block_sum(s, red);
     if (threadIdx.x == 0) npart[blockIdx.x] = b;
-}
-
-// Bounds (256 log2) of n entries by one CTA: largest |phi|^2 and squared l2 norm
-// (in thread 0).
-__device__ int2 fx_norm_max(const double2 *__restrict__ p, int n) {
-    __shared__ double red[kThreads / 32], mx[kThreads / 32];
-    double s = 0.0, m = 0.0;
-    for (int t = threadIdx.x; t < n; t += kThreads) {
-        const double2 v = p[t];
-        const double q = v.x * v.x + v.y * v.y;
-        s += q;
-        m = fmax(m, q);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) mx[threadIdx.x >> 5] = m;
-    s = block_sum(s, red);  // its barriers also order mx
-    if (threadIdx.x == 0)
-        for (int w = 1; w < kThreads / 32; ++w) m = fmax(m, mx[w]);
-    return make_int2(fx_log(m), fx_log(s));
-}
-
-// N <= 12, one CTA per state: the unit exponents of the FP64 mode.
-__global__ void __launch_bounds__(kThreads) k_fx_exponent(const double2 *__restrict__ psi, const void *const *psis,
-                                                          const int *__restrict__ Ns, int N,
-                                                          FxUnits *__restrict__ units) {
-    const int n = Ns ? Ns[blockIdx.x] : N;
-    if (n > kTileBits) return;
-    const int2 b = fx_norm_max(psis ? reinterpret_cast<const double2 *>(psis[blockIdx.x]) : psi, 1 << n);
-    if (threadIdx.x == 0) units[blockIdx.x] = fx_units(b, kFxNonFinite);
-}
-
-// N > 12: bounds of every 4096-entry block (blockIdx.y: state).
-__global__ void __launch_bounds__(kThreads) k_fx_block_norms(const double2 *__restrict__ psi,
-                                                             const void *const *psis, int2 *__restrict__ bn) {
-    const double2 *base = psis ? reinterpret_cast<const double2 *>(psis[blockIdx.y]) : psi;
-    const int2 b = fx_norm_max(base + ((size_t)blockIdx.x << kTileBits), kTile);
-    if (threadIdx.x == 0) bn[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = b;
-}
-
-// Unit exponent per x_h = x >> 12: one warp sums the bounds of the shift's blocks.
-__global__ void k_fx_scales(const int2 *__restrict__ bn_all, int nb, int *__restrict__ e_all) {
-    const int xh = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (xh >= nb) return;
-    const int2 *bn = bn_all + (size_t)blockIdx.y * nb;
-    double s = 0.0;
-    for (int tp = lane; tp < nb / 2; tp += 32) {
-        const int l = fx_bound(bn, nb, (uint64_t)xh << kTileBits, tp).y;
-        s += l >= kFxNonFinite / 2 ? __longlong_as_double(0x7ff0000000000000ll) : exp2((double)l / 256.0);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) e_all[(size_t)blockIdx.y * nb + xh] = fx_exponent(fx_log(s));
-}
-
-cudaError_t enqueue_fx_scales(const void *psi, const void *const *psis, int nstates, int N, int2 *bn, int *e,
-                              cudaStream_t st) {
-    const int nb = 1 << (N - kTileBits);
-    k_fx_block_norms<<<dim3(nb, (unsigned)nstates), kThreads, 0, st>>>(reinterpret_cast<const double2 *>(psi), psis,
-                                                                       bn);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    k_fx_scales<<<dim3((nb + 7) / 8, (unsigned)nstates), 256, 0, st>>>(bn, nb, e);
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------- finalize
@@ -256,8 +191,8 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
                 const int xe = x ? (int)x : d >> 1;
                 const int lo = (int)(flat & ((1u << NB) - 1)) & ((1 << (31 - __clz(xe))) - 1);
                 const int t = (((int)(flat & ((1u << NB) - 1)) - lo) << 1) | lo;
-                v[i] = x ? pair_value<R, false>(psi_s[pad(t ^ xe)], psi_s[pad(t)], 0)
-                         : pair_value<R, true>(psi_s[pad(t ^ xe)], psi_s[pad(t)], 0);
+                v[i] = x ? pair_value<R, false>(psi_s[pad(t ^ xe)], psi_s[pad(t)])
+                         : pair_value<R, true>(psi_s[pad(t ^ xe)], psi_s[pad(t)]);
             } else {
                 v[i] = Cx<R>::zero();
             }
@@ -296,18 +231,17 @@ template <int NB>
 __global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restrict__ psi0,
                                                           const void *const *__restrict__ psis,
                                                           long long tiles_per_state, uint64_t x_begin, uint64_t x_end,
-                                                          long long ntiles, double *__restrict__ part, int alpha,
-                                                          const FxUnits *__restrict__ units) {
+                                                          long long ntiles, double *__restrict__ part, int alpha) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2 *buf = reinterpret_cast<double2 *>(smem_raw);
     __shared__ double red[kThreads / 32];
+    __shared__ FxShared sh;
     constexpr int d = 2 << NB;
     const int tid = threadIdx.x;
     for (long long g = blockIdx.x; g < ntiles; g += gridDim.x) {
         const long long sidx = psis ? g / tiles_per_state : 0;
         const long long gl = g - sidx * tiles_per_state;
         const double2 *psi = psis ? reinterpret_cast<const double2 *>(psis[sidx]) : psi0;
-        const FxUnits un = units[sidx];
         cx_t<fx> v[16];
         auto value = [&](int i, auto with_zero) {
             const uint64_t flat = ((uint64_t)gl << kTileBits) | (uint64_t)elem<2>(tid, i);
@@ -317,8 +251,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restr
             const int lo = tt & ((1 << (31 - __clz(xe))) - 1), t = ((tt - lo) << 1) | lo;
             const double2 b = __ldg(psi + (t ^ xe)), a = __ldg(psi + t);
             if constexpr (decltype(with_zero)::value)
-                if (!x) return pair_value<fx, true>(b, a, un.a);
-            return pair_value<fx, false>(b, a, un.a);
+                if (!x) return pair_value<fx, true>(b, a);
+            return pair_value<fx, false>(b, a);
         };
         // the first tile alone holds x = 0
         if (gl == 0 && x_begin == 0) {
@@ -328,9 +262,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restr
 #pragma unroll
             for (int i = 0; i < 16; ++i) v[i] = value(i, std::false_type());
         }
-        fx_tile<NB>(v, buf, tid, un);
+        const FxExp u = fx_tile<NB>(v, buf, tid, sh);
         const double s = block_sum(sum_order<fx>(v, alpha), red);
-        if (tid == 0) part[g] = half_scale<fx>(s, alpha, un.c);
+        if (tid == 0) part[g] = half_scale<fx>(s, alpha, u.c);
     }
 }
 
@@ -490,7 +424,7 @@ void workspace_free(Workspace *ws) {
     cudaFree(ws->conv);
     cudaFree(ws->tc_e);
     cudaFree(ws->tc_bn);
-    cudaFree(ws->fx_k);
+    cudaFree(ws->fx_exp);
     *ws = Workspace();
 }
 
@@ -515,7 +449,6 @@ cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int
     SRE_TRY(cudaMalloc(&ws->work, kWorkBytes + kFlagBytes));
     ws->flags = reinterpret_cast<int *>(ws->work + kWorkBytes / 8);
     ws->status = ws->flags + 1;
-    SRE_TRY(cudaMalloc(&ws->fx_k, sizeof(FxUnits)));
     SRE_TRY(cudaMalloc(&ws->result, sizeof(Result)));
     if (N_max > kTileBits) {
         // sizes for every N up to N_max and both halves of the shift range,
@@ -543,6 +476,11 @@ cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int
         ws->tc_cap = 1 << (N_max - kTileBits);
         SRE_TRY(cudaMalloc(&ws->tc_e, sizeof(int) * ws->tc_cap));
         SRE_TRY(cudaMalloc(&ws->tc_bn, sizeof(double) * ws->tc_cap));
+        if (elem_bytes == 16) {
+            // unit and bound of every block in the ring: R * C * 2^h2 of each
+            ws->fx_cap = item_cap / 8;
+            SRE_TRY(cudaMalloc(&ws->fx_exp, sizeof(short) * 2 * ws->fx_cap));
+        }
     }
 #undef SRE_TRY
     return cudaSuccess;
@@ -552,7 +490,7 @@ template <typename R, int NB>
 static cudaError_t launch_small_nb(const void *psi, const void *const *psis, int nstates,
                                    uint64_t x_begin, uint64_t x_end, double *part, int part_cap,
                                    const DeviceInfo &dev, cudaStream_t st, int *nparts,
-                                   int forced_grid, int alpha, const int *fx_k, const SmallTail &tail) {
+                                   int forced_grid, int alpha, const SmallTail &tail) {
     constexpr bool kFx = sizeof(cx_t<R>) == 16;
     const size_t smem = (size_t)(kFx ? 1 : 3) * kTileSlots * sizeof(v2_t<R>);
     cudaError_t e;
@@ -570,7 +508,7 @@ static cudaError_t launch_small_nb(const void *psi, const void *const *psis, int
     if (grid < 1) return cudaErrorInvalidValue;
     if constexpr (kFx)
         k_small_fx<NB><<<grid, kThreads, smem, st>>>(reinterpret_cast<const double2 *>(psi), psis, tps, x_begin, x_end,
-                                                     ntiles, part, alpha, reinterpret_cast<const FxUnits *>(fx_k));
+                                                     ntiles, part, alpha);
     else
         k_small<R, NB><<<grid, kThreads, smem, st>>>(reinterpret_cast<const float2 *>(psi), psis, tps, x_begin, x_end,
                                                      ntiles, part, alpha, tail);
@@ -582,10 +520,10 @@ template <typename R>
 static cudaError_t launch_small(int N, const void *psi, const void *const *psis, int nstates,
                                 uint64_t xb, uint64_t xe, double *part, int part_cap,
                                 const DeviceInfo &dev, cudaStream_t st, int *nparts,
-                                int forced_grid, int alpha, const int *fx_k, const SmallTail &tail = SmallTail()) {
+                                int forced_grid, int alpha, const SmallTail &tail = SmallTail()) {
     switch (N) {
 #define SRE_CASE(n) \
-    case n: return launch_small_nb<R, n - 1>(psi, psis, nstates, xb, xe, part, part_cap, dev, st, nparts, forced_grid, alpha, fx_k, tail);
+    case n: return launch_small_nb<R, n - 1>(psi, psis, nstates, xb, xe, part, part_cap, dev, st, nparts, forced_grid, alpha, tail);
         SRE_CASE(1) SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6)
         SRE_CASE(7) SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11) SRE_CASE(12)
 #undef SRE_CASE
@@ -672,7 +610,8 @@ static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const Devi
     A.psi = psi;
     A.psis = nullptr;
     A.chunks_per_state = 0;
-    A.fx_bn = reinterpret_cast<const int2 *>(ws.tc_bn);
+    A.fx_exp = ws.fx_exp;
+    A.fx_cap = ws.fx_cap;
     A.tc_e = ws.tc_e;
     A.N = N;
     A.half = half;
@@ -695,7 +634,8 @@ static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const Devi
     A.n_items = A.n_chunks * (long long)(A.P1 + A.P2);
     const size_t need_scratch = (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)elem_bytes << (N - half));
     if (need_scratch > ws.scratch_bytes || chunk_off + (size_t)A.n_chunks > ws.chunk_cap ||
-        (size_t)c.R * A.P2 * 8 > ws.item_part_cap)
+        (size_t)c.R * A.P2 * 8 > ws.item_part_cap ||
+        (elem_bytes == 16 && (size_t)c.R << (c.C_log + A.h2) > ws.fx_cap))
         return cudaErrorInvalidValue;
     A.scratch = ws.scratch;
     A.item_part = ws.item_part;
@@ -735,7 +675,7 @@ static cudaError_t enqueue_small(const Workspace &ws, const DeviceInfo &dev, con
     tail.host = ws.host_result;
     tail.d_m2 = d_m2;
     int np = 0;
-    return launch_small<float>(N, psi, nullptr, 1, xb, xe, ws.part, ws.part_cap, dev, st, &np, 0, alpha, nullptr, tail);
+    return launch_small<float>(N, psi, nullptr, 1, xb, xe, ws.part, ws.part_cap, dev, st, &np, 0, alpha, tail);
 }
 
 template <typename R>
@@ -759,24 +699,13 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
     k_norm<<<kNormBlocks, kThreads, 0, st>>>(reinterpret_cast<const v2_t<R> *>(psi), d, ws.npart, ws.flags);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ws.launches += 2;  // k_norm + k_finalize
-    if constexpr (kFx) {
-        if (N <= kTileBits) {
-            k_fx_exponent<<<1, kThreads, 0, st>>>(reinterpret_cast<const double2 *>(psi), nullptr, nullptr, N,
-                                                  reinterpret_cast<FxUnits *>(ws.fx_k));
-            e = cudaGetLastError();
-        } else {
-            e = enqueue_fx_scales(psi, nullptr, 1, N, reinterpret_cast<int2 *>(ws.tc_bn), ws.tc_e, st);
-        }
-        if (e != cudaSuccess) return e;
-        ws.launches += N <= kTileBits ? 1 : 2;
-    }
     const double *parts = nullptr;
     long long nparts = 0, seg1 = 0;  // [0, seg1) shifts below 4096 beside the tensor-core kernel's [seg1, nparts)
     if (N <= kTileBits) {
         int np = 0;
         if (ws.ev_begin && (e = cudaEventRecord(ws.ev_begin, st)) != cudaSuccess) return e;
         if ((e = launch_small<R>(N, psi, nullptr, 1, x_begin, x_end, ws.part, ws.part_cap, dev, st,
-                                 &np, 0, alpha, ws.fx_k)) != cudaSuccess)
+                                 &np, 0, alpha)) != cudaSuccess)
             return e;
         if (ws.ev_end && (e = cudaEventRecord(ws.ev_end, st)) != cudaSuccess) return e;
         ws.main_kernel = "k_small";
@@ -805,8 +734,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                 chunks = (size_t)(split - x_begin);
                 if (chunks > ws.chunk_cap) return cudaErrorInvalidValue;
                 if constexpr (kFx)
-                    e = launch_mid(N, psi, nullptr, 1, (long long)chunks, x_begin, alpha, ws.chunk_sum, d_per_x,
-                                   reinterpret_cast<const int2 *>(ws.tc_bn), ws.tc_e, dev, st);
+                    e = launch_mid(N, psi, nullptr, 1, (long long)chunks, x_begin, alpha, ws.chunk_sum, d_per_x, dev, st);
                 else
                     e = launch_one(N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, d_per_x, ws.work + 2,
                                    ws.status, wait_ns, dev, st);
@@ -1042,20 +970,15 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
                                          const BatchClass &L, const void *const *d_ptrs,
                                          double *parts, unsigned *counters, size_t chunk_cap,
                                          cudaStream_t st, long long wait_ns, int *tc_e, double *tc_bn,
-                                         size_t tc_cap, const int *fx_k) {
+                                         size_t tc_cap) {
     cudaError_t e;
     const int N = L.N;
     if (N <= kTileBits) {
         int np = 0;
         e = launch_small<R>(N, nullptr, d_ptrs, L.S, 0, 1ull << N, parts + L.parts_off,
-                            (int)L.parts_n, dev, st, &np, L.small_grid, 2, fx_k);
+                            (int)L.parts_n, dev, st, &np, L.small_grid, 2);
         ws.launches += 1;
         return e;
-    }
-    if constexpr (sizeof(cx_t<R>) == 16) {
-        if (!tc_e || !tc_bn || (size_t)L.S << (N - kTileBits) > tc_cap) return cudaErrorInvalidValue;
-        if ((e = enqueue_fx_scales(nullptr, d_ptrs, L.S, N, reinterpret_cast<int2 *>(tc_bn), tc_e, st)) != cudaSuccess) return e;
-        ws.launches += 2;
     }
     size_t off = L.parts_off;
     for (int half = 0; half <= 1; ++half) {
@@ -1090,9 +1013,7 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
         if constexpr (sizeof(cx_t<R>) == 16) {
             if (mid_applies(N, 16)) {
                 // one partial per shift
-                if ((e = launch_mid(N, nullptr, d_ptrs, L.S, cps, 0, 2, parts + off, nullptr,
-                                    reinterpret_cast<const int2 *>(tc_bn), tc_e, dev, st)) !=
-                    cudaSuccess)
+                if ((e = launch_mid(N, nullptr, d_ptrs, L.S, cps, 0, 2, parts + off, nullptr, dev, st)) != cudaSuccess)
                     return e;
                 ws.launches += 1;
                 off += (size_t)cps * L.S;
@@ -1103,7 +1024,8 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
         LargeArgs A;
         A.psi = nullptr;
         A.psis = d_ptrs;
-        A.fx_bn = reinterpret_cast<const int2 *>(tc_bn);
+        A.fx_exp = ws.fx_exp;
+        A.fx_cap = ws.fx_cap;
         A.tc_e = tc_e;
         A.chunks_per_state = cps;
         A.N = N;
@@ -1124,7 +1046,8 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
         A.P1 = 1 << (A.h2 - A.B1_log);
         A.P2 = (1 << c.C_log) << (A.h2 - A.G2_log);
         A.n_items = A.n_chunks * (long long)(A.P1 + A.P2);
-        if ((size_t)A.n_chunks > chunk_cap || (size_t)A.R * A.P2 * 8 > ws.item_part_cap)
+        if ((size_t)A.n_chunks > chunk_cap || (size_t)A.R * A.P2 * 8 > ws.item_part_cap ||
+            (sizeof(cx_t<R>) == 16 && (size_t)A.R << (A.C_log + A.h2) > ws.fx_cap))
             return cudaErrorInvalidValue;
         A.scratch = ws.scratch;
         A.item_part = ws.item_part;
@@ -1153,16 +1076,16 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
 cudaError_t enqueue_batch_class(const Workspace &ws, const DeviceInfo &dev, const BatchClass &L,
                                 const void *const *d_ptrs, double *parts, unsigned *counters,
                                 size_t chunk_cap, sre_mode_t mode, cudaStream_t st,
-                                long long wait_ns, int *tc_e, double *tc_bn, size_t tc_cap, const int *fx_k) {
+                                long long wait_ns, int *tc_e, double *tc_bn, size_t tc_cap) {
     if (mode == SRE_MODE_FP64)
         return enqueue_batch_class_t<fx>(ws, dev, L, d_ptrs, parts, counters, chunk_cap, st, wait_ns, tc_e,
-                                         tc_bn, tc_cap, fx_k);
+                                         tc_bn, tc_cap);
     return enqueue_batch_class_t<float>(ws, dev, L, d_ptrs, parts, counters, chunk_cap, st, wait_ns, tc_e, tc_bn,
-                                        tc_cap, nullptr);
+                                        tc_cap);
 }
 
 cudaError_t enqueue_batch_norm(const Workspace &ws, const void *const *d_ptrs, const int *d_Ns,
-                               int count, double *npart, int *flags, int *fx_k, sre_mode_t mode,
+                               int count, double *npart, int *flags, sre_mode_t mode,
                                cudaStream_t st) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(flags, 0, sizeof(int) * count, st)) != cudaSuccess) return e;
@@ -1172,9 +1095,6 @@ cudaError_t enqueue_batch_norm(const Workspace &ws, const void *const *d_ptrs, c
         k_norm_batch<double><<<grid, kThreads, 0, st>>>(d_ptrs, d_Ns, npart, flags);
     else
         k_norm_batch<float><<<grid, kThreads, 0, st>>>(d_ptrs, d_Ns, npart, flags);
-    ws.launches += 1;
-    if ((e = cudaGetLastError()) != cudaSuccess || mode != SRE_MODE_FP64) return e;
-    k_fx_exponent<<<count, kThreads, 0, st>>>(nullptr, d_ptrs, d_Ns, 0, reinterpret_cast<FxUnits *>(fx_k));
     ws.launches += 1;
     return cudaGetLastError();
 }

@@ -57,8 +57,8 @@ using namespace dev;
 struct LargeArgs {
     CUtensorMap tmap;          // pass-2 staging (encode_p2_tmap / tc map), else unused
     const int *tc_e;           // tensor-core kernel: scale exponent per x >> 12
-    const int2 *fx_bn;         // fixed-point mode: bounds per 4096-entry block (fx_bound; tc_e: unit
-                               // exponent per x >> 12)
+    short *fx_exp;             // fixed-point mode: units of the blocks in the ring, fx_cap entries, and
+    size_t fx_cap;             // their bounds behind them (FxExp)
     const void *psi;           // the state (single-state launch)
     const void *const *psis;   // or: states of one batch class (device array)
     long long chunks_per_state;  // chunks of each state (batch class)
@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
     uint32_t sphase = 0;  // parity of the next completion of each barrier
     uint32_t slost = 0;   // barriers whose completion wait expired
 
+    __shared__ FxShared sh;
     const int tid = threadIdx.x;
     const int lgx = a.N - 1;                      // log2 scratch entries per shift
     const int C = 1 << a.C_log;
@@ -208,21 +209,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
         // batch class: chunk c belongs to state c / chunks_per_state
         long long cl = c;
         const V *psi = psi0;
-        long long sidx = 0;
         if (a.psis) {
-            sidx = c / a.chunks_per_state;
+            const long long sidx = c / a.chunks_per_state;
             cl = c - sidx * a.chunks_per_state;
             psi = reinterpret_cast<const V *>(a.psis[sidx]);
         }
-        // fixed point: block norms of the state and the exponent of the shifts' unit
-        const int2 *bn = nullptr;
-        int fxk = 0;
         const uint64_t xc = a.x0 + ((uint64_t)cl << a.C_log);
-        if constexpr (kFx) {
-            const size_t at = (size_t)sidx << (a.N - kTileBits);
-            bn = a.fx_bn + at;
-            fxk = a.tc_e[at + (xc >> kTileBits)];
-        }
         V *slot_base = scratch + (size_t)slot * ((size_t)C << lgx);
 
         if (pass1) {
@@ -279,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         for (int i = 0; i < 16; ++i) {
                             const V b = par[((i ^ q) << 8) | pl];
                             const V va = own[(i << 8) | tid];
-                            v[i] = pair_value<R, false>(b, va, 0);  // conj(phi_{t^x}) * phi_t
+                            v[i] = pair_value<R, false>(b, va);  // conj(phi_{t^x}) * phi_t
                         }
                         reg_stages<2, 12, R>(v);
 #pragma unroll
@@ -310,12 +302,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         if (x < a.x_begin || x >= a.x_end) continue;
                         cx_t<R> v[16];
                         if constexpr (kFx) {
-                            const FxUnits un = fx_units(fx_bound(bn, 1 << (a.N - kTileBits), x, tp), fxk);
-                            block_values<R>(v, block_pair(psi, a.N, x, tp), tid, un.a);
-                            fx_tile<12>(v, bufB, tid, un);
-                            fx_rescale(v, fxk - un.c);
+                            block_values<R>(v, block_pair(psi, a.N, x, tp), tid);
+                            const FxExp u = fx_tile<12>(v, bufB, tid, sh);
+                            if (tid == 0) {
+                                short *ex = a.fx_exp + ((((size_t)slot << a.C_log) + xl) << H2) + tp;
+                                __stcg(ex, (short)u.c);
+                                __stcg(ex + a.fx_cap, (short)u.s);
+                            }
                         } else {
-                            block_values<R>(v, block_pair(psi, a.N, x, tp), tid, 0);
+                            block_values<R>(v, block_pair(psi, a.N, x, tp), tid);
                             V *bB = (tcount & 1) ? bufC : bufB;
                             ++tcount;
                             tile_fwht12_rev<R>(v, bufA, bB, tid);
@@ -350,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const V b = __ldg(pbx + ((i ^ q) << 8));
-                        v[i] = pair_value<R, false>(b, own[i], 0);  // conj(phi_{t^x}) * phi_t
+                        v[i] = pair_value<R, false>(b, own[i]);  // conj(phi_{t^x}) * phi_t
                     }
                     V *bB = (tcount & 1) ? bufC : bufB;
                     ++tcount;
@@ -375,6 +370,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
             const int zb0 = (j & ((1 << ipx_log) - 1)) << a.G2_log;
             const uint64_t x = xc + (uint64_t)xl;
             double acc = 0.0;
+            int fxk = 0;  // fixed point: the shift's unit
             const bool staged2 = kTma && a.stage2;
             if constexpr (kTma) {
                 // One thread waits for the chunk's pass 1 and keeps two TMA
@@ -443,6 +439,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
             __threadfence();
             if (x >= a.x_begin && x < a.x_end) {
                 const V *xb = slot_base + ((size_t)xl << lgx);
+                const short *ex = kFx ? a.fx_exp + ((((size_t)slot << a.C_log) + xl) << H2) : nullptr;
+                FxUnits<H2> u;
                 for (int gb = 0; gb < (1 << a.G2_log); ++gb) {
                     const int zb = zb0 + gb;
                     cx_t<R> v[16];
@@ -459,11 +457,20 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         ++tcount;
                         if (kFx) __syncthreads();  // one buffer: the previous tile's readers are done
                     }
-                    tile_fwht<H2, R>(v, bufA, bB, tid);
-                    if constexpr (kFx)
+                    if constexpr (kFx) {
+                        const FxAlign<H2> align(ex, tid);
+                        // behind the first tile's loads
+                        if (gb == 0) {
+                            u = fx_units<H2>(ex, ex + a.fx_cap);
+                            fxk = u.k[2];
+                        }
+                        align(v, u.k[0]);
+                        fx_rows<H2>(v, bufB, tid, u);
                         acc += sum_order<R>(v, a.alpha);
-                    else
+                    } else {
+                        tile_fwht<H2, R>(v, bufA, bB, tid);
                         acc += half_scale<R>((double)sum_order<R>(v, a.alpha), a.alpha, 0);
+                    }
                 }
             }
             }

@@ -26,18 +26,25 @@
 // The FP64 mode transforms 64-bit fixed point (struct fx): an FP64 product is
 // rounded to a multiple of 2^(k - 63) and every butterfly is an exact integer
 // addition.  2^k bounds the values that the next four bits make, so nothing
-// overflows; the unit follows their growth, rounded every four bits: 16 and
-// 256 times the largest product of the block pair, then the product of the
-// blocks' l2 norms (Cauchy-Schwarz), above the block the sum of those products
-// over the shift's blocks.  The rounding that this leaves is below that of FP64
-// sums (per-shift sums of N = 13..15 states against 80-bit arithmetic).  The
-// reason is the pipe: GB300 runs 2 FP64 operations per clock and SM, against
-// some 40 64-bit integer additions.  FP64 operations are left for the product
-// (4 per entry) and the powers (4 per entry); both conversions are integer
-// code, since F2I and I2F run at the FP64 rate too.  Measured: all shifts of an
-// N = 16 state 46 ms (FP64 butterflies, full transforms below x = 4096: 178 ms),
-// 60 states of N = 12 10.5 ms with their evolution (61.9 ms); the FP64 pipe is
-// busy 65 % of the time.
+// overflows; the unit follows their growth, rounded every four bits.  The bounds
+// come from the tile's products themselves: the largest one, times 16 and 256,
+// and the sums of their absolute parts, which no partial sum exceeds.  (Bounds
+// from the norms of the factors are far too wide where their large entries do
+// not meet: for a state close to a basis state a shift of high weight lost all
+// its digits.)  Above the tile each block carries its own unit and bound into
+// the transform over the blocks (FxExp).  Per-shift sums against 80-bit
+// arithmetic, N = 8..20, Haar, product, near-basis, stabilizer and decaying
+// states: at most 8e-16 from the exact ones, FP64 butterflies at most 1.1e-15,
+// the same or smaller on average for each kind of state.  The reason for fixed
+// point is the pipe: GB300 runs 2 FP64 operations per clock and SM, against some
+// 40 64-bit integer additions.  FP64 operations are left for the product (4 per
+// entry) and the powers (4 per entry); both conversions are integer code, since
+// F2I and I2F run at the FP64 rate too, and so are the bounds.  Measured: all
+// shifts of an N = 16 state 47.4 ms (FP64 butterflies, full transforms below x =
+// 4096: 178 ms; units from the factors' norms, known before the products: 46.0
+// ms), 60 states of N = 12 11.3 ms with their evolution (61.9 ms; 10.5 ms); the
+// FP64 pipe is busy 62 to 71 % of the time, and waits while the products of a
+// tile are converted.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -121,17 +128,9 @@ __device__ __forceinline__ cx_t<R> conj_mul(R br, R bi, R ar, R ai) {
     return Cx<R>::pack(br * ar + bi * ai, br * ai - bi * ar);
 }
 
-// Marks a state whose norm is not a finite number.
-constexpr int kFxNonFinite = 0x3fffffff;
-
-// Bounds travel as 256 log2, rounded up, so that the transform kernels derive
-// units without FP64 operations: bound < 2^(l / 256).
-__device__ __forceinline__ int fx_log(double m) {
-    if (!isfinite(m)) return kFxNonFinite;
-    return m > 0.0 ? (int)ceil(256.0 * log2(m)) + 1 : -(1 << 20);
-}
-// Smallest k with 2^(l / 256) <= 2^k.
-__device__ __forceinline__ int fx_exponent(int l) { return l >= kFxNonFinite / 2 ? kFxNonFinite : (l + 255) >> 8; }
+// Marks a tile with a product that is not a finite number (exponents of finite
+// ones lie within +-1100).
+constexpr int kFxNonFinite = 0x7fff;
 
 // From unit 2^(k1 - 63) to the coarser 2^(k2 - 63), q = k2 - k1, rounded half
 // up: the last bit shifted out is added afterwards, since a + 2^(q - 1) leaves 64
@@ -142,10 +141,14 @@ __host__ __device__ __forceinline__ long long fx_shift(long long a, int q) {
     const long long t = a >> (q - 1);
     return (t >> 1) + (t & 1);
 }
+// The same for 0 < q <= 8 and |a| <= 2^63 - 2^10, which all partial sums of a
+// tile keep (a product has 53 bits).
+__host__ __device__ __forceinline__ long long fx_shift_few(long long a, int q) { return (a + (1ll << (q - 1))) >> q; }
 
-// round(p 2^(63 - k)), |p| < 2^k.  The mantissa, 10 bits up, moves right by
-// what its exponent lacks to the top; half of the last place is added first.
-__device__ __forceinline__ long long fx_from(double p, int k) {
+// round(p 2^(63 - k)), |p| < 2^k; the magnitude's high word, `down` places down,
+// is added to sum.  The mantissa, 10 bits up, moves right by what its exponent
+// lacks to the top; half of the last place is added first.
+__device__ __forceinline__ long long fx_from(double p, int k, int down, unsigned &sum) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(p);
     const int e = (int)(b >> 52) & 2047;
     // shift left by e - 1075 + 63 - k in all, 10 of them already done
@@ -153,6 +156,7 @@ __device__ __forceinline__ long long fx_from(double p, int k) {
     const unsigned long long m =
         (((b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull)) << 10) + ((1ull << (q & 63)) >> 1);
     const long long r = (unsigned)q < 64 ? (long long)(m >> (q & 63)) : 0;  // zero, or below half a unit
+    sum += (unsigned)(r >> 32) >> down;
     return (long long)b < 0 ? -r : r;
 }
 
@@ -168,9 +172,9 @@ __device__ __forceinline__ double fx_abs(long long a) {
 
 // g_x(t) = conj(phi_{t^x}) phi_t from the factors b = phi_{t^x}, a = phi_t, or
 // for x = 0 (ZERO) W's input ((g0 + g1) / 2, (g0 - g1) / 2) from the two halves
-// of g_0.  k: the fixed-point unit's exponent (fx only).
+// of g_0.  fx: the bits of the FP64 values, which fx_tile converts.
 template <typename R, bool ZERO>
-__device__ __forceinline__ cx_t<R> pair_value(v2_t<R> b, v2_t<R> a, int k) {
+__device__ __forceinline__ cx_t<R> pair_value(v2_t<R> b, v2_t<R> a) {
     using T = real_t<R>;
     T re, im;
     if constexpr (ZERO) {
@@ -184,7 +188,7 @@ __device__ __forceinline__ cx_t<R> pair_value(v2_t<R> b, v2_t<R> a, int k) {
     if constexpr (sizeof(cx_t<R>) == 8)
         return Cx<R>::pack(re, im);
     else
-        return make_longlong2(fx_from(re, k), fx_from(im, k));
+        return Cx<fx>::from(make_double2(re, im));
 }
 
 // A sum of (Re W)^(2 alpha) + (Im W)^(2 alpha) over FP32 values, times 2^(2 alpha)
@@ -243,21 +247,21 @@ template <> __device__ __forceinline__ int elem<2>(int tid, int i) { return (i <
 
 // Products of a block in round-2 layout (e = i << 8 | tid), any pivot.
 template <typename R, bool ZERO>
-__device__ __forceinline__ void block_values_z(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid, int k) {
+__device__ __forceinline__ void block_values_z(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid) {
     const int o = s.place(tid), w0 = s.place(256), w1 = s.place(512), w2 = s.place(1024), w3 = s.place(2048);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int e = o + ((i & 1) ? w0 : 0) + ((i & 2) ? w1 : 0) + ((i & 4) ? w2 : 0) + ((i & 8) ? w3 : 0);
-        v[i] = pair_value<R, ZERO>(__ldg(s.par + (e ^ s.xo)), __ldg(s.own + e), k);
+        v[i] = pair_value<R, ZERO>(__ldg(s.par + (e ^ s.xo)), __ldg(s.own + e));
     }
 }
 
 template <typename R>
-__device__ __forceinline__ void block_values(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid, int k) {
+__device__ __forceinline__ void block_values(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid) {
     if (s.zero)
-        block_values_z<R, true>(v, s, tid, k);
+        block_values_z<R, true>(v, s, tid);
     else
-        block_values_z<R, false>(v, s, tid, k);
+        block_values_z<R, false>(v, s, tid);
 }
 
 // Butterflies over register bits j in [0, 4) whose tile bit 4K + j < NB.
@@ -320,59 +324,171 @@ __device__ __forceinline__ void tile_fwht(cx_t<R> (&v)[16], v2_t<R> *bufA, v2_t<
     }
 }
 
-// Unit exponents of a fixed-point tile: its products, after four bits and
-// after eight.
-struct FxUnits {
-    int a, b, c;
+// Shared words of a CTA's fixed-point tile, per warp: exponent field of the
+// largest product, sums of the absolute real and imaginary parts.
+struct __align__(16) FxShared {
+    int e[8];
+    uint2 sums[8];
 };
 
-// From the bounds (256 log2) of the largest product and of all partial sums of
-// the tile, none above the exponent `most`.
-__device__ __forceinline__ FxUnits fx_units(int2 l, int most) {
-    FxUnits u;
-    u.c = min(fx_exponent(l.y), most);
-    u.b = min(fx_exponent(l.x + (8 << 8)), u.c);
-    u.a = min(fx_exponent(l.x + (4 << 8)), u.b);
-    return u;
-}
+// A transformed tile: values are multiples of 2^(c - 63) below 2^c, and no sum
+// of +-products of the tile reaches 2^s.
+struct FxExp {
+    int c, s;
+};
 
 __device__ __forceinline__ void fx_rescale(cx_t<fx> (&v)[16], int q) {
     if (q <= 0) return;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = make_longlong2(fx_shift(v[i].x, q), fx_shift(v[i].y, q));
+    for (int i = 0; i < 16; ++i) v[i] = make_longlong2(fx_shift_few(v[i].x, q), fx_shift_few(v[i].y, q));
 }
 
 // 12-bit transform of the fixed-point mode, bits 8-11 first, of which the bits
-// below NB are transformed: round-2 layout at unit u.a in, round-0 layout at
-// u.c out.  One buffer serves both moves (after the CTA-wide one each warp
-// stays in its own part of it); the barrier before it keeps the previous
-// tile's readers ahead.
+// below NB are transformed: products (the bits of FP64 values) in round-2 layout
+// in, round-0 layout out.  The first group of stages runs in units of each
+// warp's own, so that the bounds of the tile meet at the barrier of the
+// CTA-wide move: after it register i holds what warp i / 2 wrote.  One buffer
+// serves both moves (after the CTA-wide one each warp stays in its own part of
+// it); the barrier before it keeps the previous tile's readers ahead.
 template <int NB>
-__device__ __forceinline__ void fx_tile(cx_t<fx> (&v)[16], double2 *buf, int tid, const FxUnits &u) {
+__device__ __forceinline__ FxExp fx_tile(cx_t<fx> (&v)[16], double2 *buf, int tid, FxShared &sh) {
+    // stages of each group
+    constexpr int GA = NB > 8 ? NB - 8 : 0, GB = NB > 8 ? 4 : NB > 4 ? NB - 4 : 0, GC = NB > 4 ? 4 : NB;
+    const int lane = tid & 31, warp = tid >> 5;
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+        m = max(m, max((unsigned)(v[i].x >> 32) & 0x7fffffffu, (unsigned)(v[i].y >> 32) & 0x7fffffffu));
+    const int e = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);  // the warp's products: below 2^(e - 1022)
+    // sums of |re| and |im|, each entry rounded up to 2^(e - 1022 - 27): 16
+    // entries make 2^31 + 16 at most, then 2^(e - 1022 - 22) for the warp
+    unsigned sr = 16, si = 16;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        v[i].x = fx_from(__longlong_as_double(v[i].x), e - 1022 + GA, 4 - GA, sr);
+        v[i].y = fx_from(__longlong_as_double(v[i].y), e - 1022 + GA, 4 - GA, si);
+    }
+    sr = __reduce_add_sync(0xffffffffu, (sr >> 5) + 1);
+    si = __reduce_add_sync(0xffffffffu, (si >> 5) + 1);
     reg_stages<2, NB, fx>(v);
-    fx_rescale(v, u.b - u.a);
     __syncthreads();
+    if (lane == 0) {
+        sh.e[warp] = e;
+        sh.sums[warp] = make_uint2(sr, si);
+    }
     relayout<2, 1, false, fx>(v, buf, tid);
+    // the tile's largest exponent, and its sums in units of 2^(most - 1022 - 19),
+    // with one unit more: the rescaling below moves a sum by less (2^8 units
+    // of the coarsest, 2^(c - 63))
+    const int ew = sh.e[lane & 7], most = __reduce_max_sync(0xffffffffu, ew);
+    const uint2 t = sh.sums[lane & 7];
+    const int d = min(most - ew + 3, 31);
+    sr = __reduce_add_sync(0xffffffffu, lane < 8 ? (t.x >> d) + 1 : 0) + 1;
+    si = __reduce_add_sync(0xffffffffu, lane < 8 ? (t.y >> d) + 1 : 0) + 1;
+    FxExp u;
+    u.s = most - 1022 - 19 + 32 - __clz(max(sr, si));
+    const int ka = most - 1022 + GA, kb = min(max(u.s, ka), ka + GB);
+    u.c = min(max(u.s, kb), kb + GC);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const int q = kb - (sh.e[w] - 1022 + GA);
+        if (q > 8) {
+#pragma unroll
+            for (int i = 2 * w; i < 2 * w + 2; ++i) v[i] = make_longlong2(fx_shift(v[i].x, q), fx_shift(v[i].y, q));
+        } else if (q > 0) {
+#pragma unroll
+            for (int i = 2 * w; i < 2 * w + 2; ++i)
+                v[i] = make_longlong2(fx_shift_few(v[i].x, q), fx_shift_few(v[i].y, q));
+        }
+    }
     reg_stages<1, NB, fx>(v);
-    fx_rescale(v, u.c - u.b);
+    fx_rescale(v, u.c - kb);
     relayout<1, 0, true, fx>(v, buf, tid);
     reg_stages<0, NB, fx>(v);
+    if (most == 2047) u.c = u.s = kFxNonFinite;
+    return u;
 }
 
-// Bounds (256 log2) of the largest product and of the partial sums of block
-// t'_h = tp of shift x, from the blocks' (largest |phi|^2, squared l2 norm): the
-// block pair's geometric mean, or for a pivot inside the block (x < 4096) twice
-// the larger of the two blocks that the halved one comes from (nb: blocks of
-// the state).
-__device__ __forceinline__ int2 fx_bound(const int2 *bn, int nb, uint64_t x, int tp) {
-    if (x < 4096) {  // x = 0 pairs the halves of the state
-        const int2 a = __ldg(bn + (x ? 2 * tp : tp)), b = __ldg(bn + (x ? 2 * tp + 1 : tp + nb / 2));
-        return make_int2(max(a.x, b.x), max(a.y, b.y) + 256);
+// Units of the transform over a shift's 2^H2 blocks: k[0] for its first four
+// bits, k[1] and k[2] for the next ones; the last also for its results.
+template <int H2>
+struct FxUnits {
+    static constexpr int G0 = H2 < 4 ? H2 : 4, G1 = H2 < 4 ? 0 : H2 < 8 ? H2 - 4 : 4, G2 = H2 < 8 ? 0 : H2 - 8;
+    int k[3];
+};
+
+// From the largest unit cm of the blocks and a bound 2^s of their sum.
+template <int H2>
+__device__ __forceinline__ FxUnits<H2> fx_units(int cm, int s) {
+    using U = FxUnits<H2>;
+    U u;
+    u.k[0] = min(max(s, cm), cm + U::G0);
+    u.k[1] = min(max(s, u.k[0]), u.k[0] + U::G1);
+    u.k[2] = min(max(s, u.k[1]), u.k[1] + U::G2);
+    if (cm == kFxNonFinite) u.k[2] = kFxNonFinite;
+    return u;
+}
+
+// The same from the blocks' exponents in global memory, by a warp.  Bounds are
+// added as multiples of 2^(largest - 20), rounded up: 2^11 blocks fit 32 bits.
+template <int H2>
+__device__ __forceinline__ FxUnits<H2> fx_units(const short *c, const short *s) {
+    constexpr int n = 1 << H2;
+    const int lane = threadIdx.x & 31;
+    int cm = -0x8000, sm = -0x8000;
+#pragma unroll 1
+    for (int t = lane; t < n; t += 32) {
+        cm = max(cm, (int)__ldcg(c + t));
+        sm = max(sm, (int)__ldcg(s + t));
     }
-    const int xh = (int)(x >> 12), j = 31 - __clz(xh);
-    const int th = ((tp >> j) << (j + 1)) | (tp & ((1 << j) - 1));
-    const int2 a = __ldg(bn + th), b = __ldg(bn + (th ^ xh));
-    return make_int2((a.x + b.x + 1) >> 1, (a.y + b.y + 1) >> 1);
+    cm = __reduce_max_sync(0xffffffffu, cm);
+    sm = __reduce_max_sync(0xffffffffu, sm);
+    unsigned sum = 0;
+#pragma unroll 1
+    for (int t = lane; t < n; t += 32) sum += (1u << 20) >> min(sm - (int)__ldcg(s + t), 20);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    return fx_units<H2>(cm, sm - 20 + 32 - __clz(sum - 1));
+}
+
+// This thread's entries (round-0 layout, block = entry index mod 2^H2) from
+// their blocks' units, c, to the unit k.
+template <int H2>
+struct FxAlign {
+    static constexpr int n = H2 < 4 ? 1 << H2 : 16;
+    __align__(16) short q[n];
+    __device__ __forceinline__ FxAlign(const short *c, int tid) {
+        const short *p = c + ((tid << 4) & ((1 << H2) - 1));
+        if constexpr (n == 4) {
+            *reinterpret_cast<int2 *>(q) = __ldcg(reinterpret_cast<const int2 *>(p));
+        } else {
+#pragma unroll
+            for (int j = 0; j < n; j += 8)
+                *reinterpret_cast<int4 *>(q + j) = __ldcg(reinterpret_cast<const int4 *>(p + j));
+        }
+    }
+    __device__ __forceinline__ void operator()(cx_t<fx> (&v)[16], int k) const {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int d = k - q[i & (n - 1)];
+            v[i] = make_longlong2(fx_shift(v[i].x, d), fx_shift(v[i].y, d));
+        }
+    }
+};
+
+// Transform over the 2^H2 blocks, round-0 layout in, units u.
+template <int H2>
+__device__ __forceinline__ void fx_rows(cx_t<fx> (&v)[16], double2 *buf, int tid, const FxUnits<H2> &u) {
+    reg_stages<0, H2, fx>(v);
+    if constexpr (H2 > 4) {
+        fx_rescale(v, u.k[1] - u.k[0]);
+        relayout<0, 1, true, fx>(v, buf, tid);
+        reg_stages<1, H2, fx>(v);
+    }
+    if constexpr (H2 > 8) {
+        fx_rescale(v, u.k[2] - u.k[1]);
+        relayout<1, 2, false, fx>(v, buf, tid);
+        reg_stages<2, H2, fx>(v);
+    }
 }
 
 // Full 12-bit transform, bits 8-11 first: input in round-2 layout (thread

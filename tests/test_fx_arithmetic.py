@@ -13,8 +13,9 @@ SOURCE = r"""
 #include "sre_tile.cuh"
 int main() {
     long long a;
-    int q;
-    while (scanf("%lld %d", &a, &q) == 2) printf("%lld\n", sre::dev::fx_shift(a, q));
+    int q, few;
+    while (scanf("%lld %d %d", &a, &q, &few) == 3)
+        printf("%lld\n", few ? sre::dev::fx_shift_few(a, q) : sre::dev::fx_shift(a, q));
     return 0;
 }
 """
@@ -30,8 +31,8 @@ def shifted(tmp_path_factory):
     subprocess.run([build.nvcc(), "-std=c++17", "-O2", *build.ARCH, "-I", build.CSRC, str(src), "-o", str(exe)],
                    check=True)
 
-    def run(pairs):
-        text = "".join(f"{a} {q}\n" for a, q in pairs)
+    def run(pairs, few=0):
+        text = "".join(f"{a} {q} {few}\n" for a, q in pairs)
         return list(map(int, subprocess.run([str(exe)], input=text, capture_output=True, text=True,
                                             check=True).stdout.split()))
 
@@ -44,3 +45,9 @@ def test_shift_rounds_half_up_over_the_whole_range(shifted):
     pairs = [(a, q) for a in values for q in range(-2, 70)]
     want = [a if q <= 0 else 0 if q > 62 else (a + (1 << (q - 1))) >> q for a, q in pairs]
     assert shifted(pairs) == want
+
+
+def test_short_shift_rounds_alike_below_the_top(shifted):
+    top = (1 << 63) - (1 << 10)
+    pairs = [(s * v, q) for s in (1, -1) for v in (0, 1, 7, 128, 99991, 1 << 50, top - 1, top) for q in range(1, 9)]
+    assert shifted(pairs, 1) == shifted(pairs)
