@@ -414,10 +414,11 @@ SRE_API sre_status_t sre_server_create(const sre_server_cfg_t *cfg, sre_server_t
 /*
  * Tuning of the two-pass kernels for requests of N qubits (13 <= N <= the
  * server's max_N; fields as sre_tuning_t for sre_plan_set_tuning, -1 keeps
- * the library's choice), applied to every later unit of that N.  The
- * ring must fit each slot's scratch (SRE_EINVAL otherwise; see
- * slot_scratch_bytes); a plan's library choice, which sre_plan_get_tuning
- * returns, stands for the slot's own.  Thread-safe.
+ * the library's choice), applied to every later unit that runs alone (N > 16;
+ * smaller requests share launches in the library's configuration).  The ring
+ * must fit each slot's scratch (SRE_EINVAL otherwise; see slot_scratch_bytes);
+ * where it does not, a plan's whole library choice, which
+ * sre_plan_get_tuning returns, stands for the slot's own.  Thread-safe.
  */
 SRE_API sre_status_t sre_server_set_tuning(sre_server_t srv, int N, const sre_tuning_t *tuning);
 

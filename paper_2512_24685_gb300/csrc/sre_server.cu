@@ -400,13 +400,16 @@ sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t)
     if (t->pass2_staged >= 0) c.stage2 = t->pass2_staged;
     c.G2_log = std::min(c.G2_log, N - sre::kTileBits - 1);
     c.B1_log = std::min(c.B1_log, N - sre::kTileBits - 1);
-    // a plan's library configuration, whose ring a slot's smaller scratch may
-    // not hold, stands for the slot's own
-    sre::Workspace plan_ws;
-    plan_ws.scratch_bytes = sre::kTuneScratch;
-    const sre::LargeCfg lib = sre::choose_main_cfg(s->dev, plan_ws, N, s->cfg.mode);
-    if (c.C_log == lib.C_log && c.R == lib.R && c.D == lib.D)
-        c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode);
+    // a plan's library configuration whose ring the slots' smaller scratch does
+    // not hold stands for the slots' own; whatever fits is taken as it is
+    if (!sre::main_cfg_fits(s->slots[0].ws, c, N, s->cfg.mode)) {
+        sre::Workspace plan_ws;
+        plan_ws.scratch_bytes = sre::kTuneScratch;
+        const sre::LargeCfg lib = sre::choose_main_cfg(s->dev, plan_ws, N, s->cfg.mode);
+        if (c.C_log == lib.C_log && c.R == lib.R && c.D == lib.D && c.G2_log == lib.G2_log &&
+            c.B1_log == lib.B1_log && c.stage1 == lib.stage1 && c.stage2 == lib.stage2)
+            c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode);
+    }
     std::lock_guard<std::mutex> lk(s->mu);
     for (const Slot &sl : s->slots)
         if (!sre::main_cfg_fits(sl.ws, c, N, s->cfg.mode)) return SRE_EINVAL;
