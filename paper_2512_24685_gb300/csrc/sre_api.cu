@@ -248,7 +248,7 @@ static sre_status_t enqueue_plan(sre_plan_t p, const void *d_state, int N, uint6
     sre::LargeCfg *cp = nullptr;
     if (N > sre::kTileBits) {
         c = plan_cfg(p, N);
-        if (!sre::main_cfg_fits(p->ws, c, N, p->mode)) return SRE_EINVAL;
+        if (!sre::large_cfg_fits(p->ws, c, N, 1)) return SRE_EINVAL;
         cp = &c;
     }
     return enqueue_plan_cfg(p, d_state, N, xb, xe, st, d_m2, d_per_x, cp, alpha);
@@ -327,26 +327,12 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
             if (o.C_log == c.C_log && o.G2_log == c.G2_log && o.B1_log == c.B1_log && o.D == c.D &&
                 o.R == c.R && o.stage1 == c.stage1 && o.stage2 == c.stage2)
                 return;
-        if (sre::main_cfg_fits(p->ws, c, N, p->mode)) cands.push_back(c);
+        if (sre::large_cfg_fits(p->ws, c, N, 1)) cands.push_back(c);
     };
-    // the FP32 kernel of sre_two.cu has no item sizes or copy paths to vary:
-    // shifts per item and ring alone
-    const bool two = p->mode == SRE_MODE_FP32 && sre::two_applies(N, eb);
-    // N = 16 in FP32 runs in a single pass: nothing to vary, its time alone
-    const bool one = p->mode == SRE_MODE_FP32 && sre::one_applies(N, eb);
-    if (one) add(base);
-    for (int C_log = 0; two && C_log <= 3; ++C_log) {
-        sre::LargeCfg c = base;
-        c.C_log = C_log;
-        const size_t chunk = ((size_t)eb << (N - 1)) << C_log;
-        const int fit = (int)std::min<size_t>(p->ws.scratch_bytes / chunk, sre::kMaxRing);
-        for (int R : {fit, fit * 3 / 4, fit / 2, fit / 4, base.R}) {
-            c.R = R;
-            c.D = R - 1;
-            add(c);
-        }
-    }
-    for (int C_log = 0; !two && !one && C_log <= 3; ++C_log)
+    // FP32 kernels that take no tuning (sre_one.cu, sre_two.cu): the time alone
+    const bool fixed = p->mode == SRE_MODE_FP32 && (sre::one_applies(N, eb) || sre::two_applies(N, eb));
+    if (fixed) add(base);
+    for (int C_log = 0; !fixed && C_log <= 3; ++C_log)
         for (int g = 0; g <= 3; ++g)
             for (int b = 2; b <= 3; ++b)
                 for (int dm = 0; dm <= (tc ? 6 : 3); ++dm) {

@@ -96,7 +96,6 @@ LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_
 // The configuration that a caller's partial tuning completes: with a ring field
 // of the caller's own, the L2-sized one, whose lag and slots leave room for it.
 LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t);
-bool main_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, sre_mode_t mode);
 
 // Tensor-core two-pass kernel (sre_tc.cu) for the halved shifts of one
 // state: tc_kind 1 = BF16 hi/lo pieces, 2 = FP16 hi/lo pieces.  tc_applies

@@ -383,7 +383,6 @@ static LargeCfg choose_tc_cfg(const DeviceInfo &dev, const Workspace &ws, int N)
 
 LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode) {
     const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
-    if (mode == SRE_MODE_FP32 && two_applies(N, eb)) return choose_two_cfg(dev, ws, N);
     if (tc_mode_available(mode) && tc_applies(N, 1, 2, nullptr)) return choose_tc_cfg(dev, ws, N);
     return choose_large_cfg(dev, N, eb, 1);
 }
@@ -392,11 +391,6 @@ LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_
     if (t.x_batch_log >= 0 || t.ring_slots >= 0 || t.lag >= 0)
         return choose_large_cfg(dev, N, mode == SRE_MODE_FP64 ? 16 : 8, 1);
     return choose_main_cfg(dev, ws, N, mode);
-}
-
-bool main_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, sre_mode_t mode) {
-    return mode == SRE_MODE_FP32 && two_applies(N, ws.elem_bytes) ? two_cfg_fits(ws, c, N)
-                                                                   : large_cfg_fits(ws, c, N, 1);
 }
 
 size_t workspace_scratch_bytes(const DeviceInfo &dev, int N_max, int elem_bytes, sre_mode_t mode) {
@@ -740,7 +734,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                                    ws.status, wait_ns, dev, st);
             } else if (two_applies(N, eb)) {
                 name = "k_two";
-                const LargeCfg c = !tc_kind && cfg_override ? *cfg_override : choose_two_cfg(dev, ws, N);
+                const LargeCfg c = choose_two_cfg(dev, ws, N);
                 e = launch_two(ws, c, N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, ws.counters,
                                ws.chunk_cap, ws.chunk_cap, ws.work + 2, d_per_x, wait_ns, st);
                 chunks = (size_t)two_layout(ws, c, N, x_begin, split).n_chunks;
@@ -946,7 +940,7 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         // every shift in one launch, or the shifts below 4096 beside the
         // tensor-core kernel
         L.cfg_full = choose_two_cfg(dev, ws, N);
-        L.cfg_half = mode == SRE_MODE_FP32 && tuned_half ? *tuned_half : L.cfg_full;
+        L.cfg_half = L.cfg_full;
         if (tc_kind) L.cfg_half = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode);
         L.cps_full = tc_kind ? two_layout(ws, L.cfg_full, N, 0, kTile).n_chunks : 0;
         L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)

@@ -463,6 +463,9 @@ int two_u_log(int N) { return std::max(0, 4 - two_h2(N)); }
 
 bool two_applies(int N, int elem_bytes) { return elem_bytes == 8 && N >= 17 && N <= 20; }
 
+// The kernel takes no tuning of the caller's: the fields were found for kernels
+// with other items (a ring of chunks and a lag between the passes), and read as
+// its own they cost up to 45 % (N = 20, one shift per item: no factors shared).
 // Four shifts per item share one fill of the factors; the ring takes the
 // workspace's tuning scratch (192 MB), less where the workspace has less.  With
 // a ring that fits L2 the CTAs run out of slots: a chunk lives for two item
@@ -478,22 +481,18 @@ LargeCfg choose_two_cfg(const DeviceInfo &dev, const Workspace &ws, int N) {
     while (c.C_log > 0 && ws.scratch_bytes >> c.C_log < (size_t)64 << (N - 1)) --c.C_log;  // 8 slots at least
     const size_t chunk = (size_t)8 << (c.C_log + two_u_log(N) + N - 1);
     c.R = (int)std::max<size_t>(2, std::min<size_t>(kMaxRing, std::min(ws.scratch_bytes, kTuneScratch) / chunk));
-    c.D = c.R - 1;  // not used: items are handed out as they become possible
+    c.D = 1;  // not used: items are handed out as they become possible
     return c;
 }
 
 namespace {
+// Does the configuration fit the workspace (ring of scratch, item partials)?
 bool two_fits(const Workspace &ws, const LargeCfg &c, int N, int U_log) {
     const size_t ring = (size_t)c.R << (c.C_log + U_log + N - 1 + 3);
     const size_t parts = (size_t)c.R << (c.C_log + U_log + two_h2(N) + 3);
     return ring <= ws.scratch_bytes && parts <= ws.item_part_cap;
 }
 }  // namespace
-
-bool two_cfg_fits(const Workspace &ws, const LargeCfg &c, int N) {
-    return c.C_log >= 0 && c.C_log <= 3 && c.R >= 2 && c.R <= kMaxRing && c.D >= 1 && c.D < c.R &&
-           two_fits(ws, c, N, 0);
-}
 
 TwoLayout two_layout(const Workspace &ws, const LargeCfg &c, int N, uint64_t xb, uint64_t xe) {
     TwoLayout L;
@@ -513,7 +512,7 @@ cudaError_t launch_two(const Workspace &ws, const LargeCfg &c, int N, const void
                        int nstates, uint64_t xb, uint64_t xe, int alpha, double *chunk_sum, unsigned *counters,
                        size_t counter_stride, size_t counter_cap, unsigned long long *work, double *per_x,
                        long long wait_ns, cudaStream_t st) {
-    if (!two_cfg_fits(ws, c, N)) return cudaErrorInvalidValue;
+    if (!two_fits(ws, c, N, 0)) return cudaErrorInvalidValue;
     const TwoLayout L = two_layout(ws, c, N, xb, xe);
     TwoArgs a;
     a.psi = reinterpret_cast<const float2 *>(psi);

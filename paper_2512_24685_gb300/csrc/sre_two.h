@@ -14,8 +14,6 @@ struct TwoLayout {
 
 bool two_applies(int N, int elem_bytes);
 LargeCfg choose_two_cfg(const DeviceInfo &dev, const Workspace &ws, int N);
-// Does the configuration fit the workspace (ring of scratch, item partials)?
-bool two_cfg_fits(const Workspace &ws, const LargeCfg &c, int N);
 // Chunks of one state over the shifts [xb, xe).
 TwoLayout two_layout(const Workspace &ws, const LargeCfg &c, int N, uint64_t xb, uint64_t xe);
 // Enqueue the sums over [xb, xe) of one state (psi) or of nstates states of a

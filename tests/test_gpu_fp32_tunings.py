@@ -1,0 +1,35 @@
+"""Tunings of the FP32 two-pass kernels that were saved for other kernels.  N =
+17..19 take none: a saved one changes neither the order of the sums (bit for
+bit) nor the share of the work that is done twice."""
+import pytest
+
+from paper_2512_24685_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sre():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2512_24685_gb300 import binding
+    binding.load_library()
+    return binding
+
+
+@pytest.mark.parametrize("N,tuning", [(17, (2, 55, 27, 3, 0, 1, 1)), (17, (0, 9, 4, 1, 1, 0, 0)),
+                                      (18, (3, 23, 11, 3, 0, 1, 1)), (19, (0, 40, 20, 3, 1, 1, 1))])
+def test_saved_tunings_leave_the_kernel_as_it_is(sre, N, tuning):
+    import numpy as np
+    import torch
+    psi = torch.from_numpy(W.haar_state(N, 9 + N, np.complex64)).cuda()
+    with sre.Plan(N, "c64") as p:
+        for b, e in ((5, 5 + 40001), (8192, 8192 + 300)):
+            want = p.sum4_range(psi, b, e).tolist()
+            p.set_tuning(*tuning)
+            got = p.sum4_range(psi, b, e).tolist()
+            p.set_tuning(-1, -1, -1, -1, -1)
+            assert got == want
+        p.set_tuning(3, 64, 5)  # a ring beyond the plan's scratch is refused as ever
+        with pytest.raises(sre.SreError):
+            p.sum4_range(psi, 0, 8)
