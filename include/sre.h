@@ -124,7 +124,7 @@ SRE_API sre_status_t sre_plan_set_mode(sre_plan_t plan, sre_mode_t mode);
 SRE_API sre_status_t sre_plan_get_mode(sre_plan_t plan, sre_mode_t *mode);
 
 /*
- * Tuning of the two-pass kernels (FP32 N >= 21, FP64 N >= 15, the split
+ * Tuning of the two-pass kernels (FP32 N >= 20, FP64 N >= 15, the split
  * modes' shifts x >= 4096 at 16 <= N <= 20): one pass transforms the low bits
  * of t per block into a ring of scratch, the other the remaining bits.  x_batch_log: log2 of the shifts that share one
  * pass-1 partner block (0..3); ring_slots: chunks held in the ring (>= 2);
@@ -136,14 +136,14 @@ SRE_API sre_status_t sre_plan_get_mode(sre_plan_t plan, sre_mode_t *mode);
  * copy into shared memory (FP32 CUDA-core path, x_batch_log = 0 and a
  * 16-byte aligned state; otherwise, or with 0, per-thread loads);
  * pass2_staged (0/1): pass 2 takes its tiles by 2-D tensor-memory-accelerator
- * copies into shared memory (FP32, N = 21; otherwise, or with 0,
+ * copies into shared memory (FP32, N = 20 and 21; otherwise, or with 0,
  * per-thread loads).
  * A value of -1 keeps the library's choice for that field; all -1 restores
  * the defaults.  With one of x_batch_log, ring_slots and lag given, the others
  * keep those of an L2-sized ring.  The scratch ring must fit the plan's
- * allocation (SRE_EINVAL otherwise).  The kernels of FP32 N <= 20 and FP64 N <= 14
+ * allocation (SRE_EINVAL otherwise).  The kernels of FP32 N <= 19 and FP64 N <= 14
  * take no tuning (the fields are checked, kept and not used); the staging
- * fields apply to FP32 with N >= 21.
+ * fields apply to FP32 with N >= 20.
  */
 typedef struct {
     int x_batch_log;
@@ -163,7 +163,7 @@ SRE_API sre_status_t sre_plan_get_tuning(sre_plan_t plan, int N, sre_tuning_t *t
  * the plan, keep the fastest and make it the plan's tuning for that N.
  * SYNCHRONOUS (uses `stream`).  *best receives the chosen tuning and *ms its
  * time on the slice (either may be NULL).  FP32 N <= 15 and FP64 N <= 14 have
- * nothing to tune (SRE_OK, tuning left unchanged), FP32 16 <= N <= 20 one
+ * nothing to tune (SRE_OK, tuning left unchanged), FP32 16 <= N <= 19 one
  * candidate.
  */
 SRE_API sre_status_t sre_plan_autotune(sre_plan_t plan, int N, sre_stream_t stream,

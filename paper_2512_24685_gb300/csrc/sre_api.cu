@@ -221,11 +221,11 @@ sre_status_t sre_plan_destroy(sre_plan_t p) {
 
 // Configuration of the halved shifts for N > 12: the library default, then
 // the autotuned one, then the caller's explicit fields.
-static sre::LargeCfg plan_cfg(sre_plan_t p, int N) {
+static sre::LargeCfg plan_cfg(sre_plan_t p, int N, uint64_t shifts) {
     // a tuned configuration serves the kernel it was timed on: the FP32 modes'
     // kernels count items and lag differently
     const bool tuned = p->has_tuned[N] && (p->tuned_mode[N] == SRE_MODE_FP32) == (p->mode == SRE_MODE_FP32);
-    sre::LargeCfg c = tuned ? p->tuned[N] : sre::tuning_base_cfg(p->dev, p->ws, N, p->mode, p->user);
+    sre::LargeCfg c = tuned ? p->tuned[N] : sre::tuning_base_cfg(p->dev, p->ws, N, p->mode, p->user, shifts);
     if (p->user.x_batch_log >= 0) c.C_log = p->user.x_batch_log;
     if (p->user.ring_slots >= 0) c.R = p->user.ring_slots;
     if (p->user.lag >= 0) c.D = p->user.lag;
@@ -247,7 +247,7 @@ static sre_status_t enqueue_plan(sre_plan_t p, const void *d_state, int N, uint6
     sre::LargeCfg c;
     sre::LargeCfg *cp = nullptr;
     if (N > sre::kTileBits) {
-        c = plan_cfg(p, N);
+        c = plan_cfg(p, N, xe - xb);
         if (!sre::large_cfg_fits(p->ws, c, N, 1)) return SRE_EINVAL;
         cp = &c;
     }
@@ -283,7 +283,7 @@ sre_status_t sre_plan_get_tuning(sre_plan_t p, int N, sre_tuning_t *t) {
         *t = {-1, -1, -1, -1, -1, -1, -1};
         return SRE_OK;
     }
-    const sre::LargeCfg c = plan_cfg(p, N);
+    const sre::LargeCfg c = plan_cfg(p, N, 1ull << N);
     t->x_batch_log = c.C_log;
     t->ring_slots = c.R;
     t->lag = c.D;
@@ -314,7 +314,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
     // once (one lag step claims the P1 + P2 items of a chunk) or the largest
     // ring 2 D + 1 the scratch holds
     const int eb = elem_bytes_for_mode(p->mode);
-    const sre::LargeCfg base = sre::choose_main_cfg(p->dev, p->ws, N, p->mode);
+    const sre::LargeCfg base = sre::choose_main_cfg(p->dev, p->ws, N, p->mode, 1ull << N);
     const int h2 = N - sre::kTileBits - 1;
     // the tensor-core kernel runs one CTA per SM and always stages its
     // copies, so its lag steps are counted over the SMs, its lag is tried at
@@ -330,7 +330,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
         if (sre::large_cfg_fits(p->ws, c, N, 1)) cands.push_back(c);
     };
     // FP32 kernels that take no tuning (sre_one.cu, sre_two.cu): the time alone
-    const bool fixed = p->mode == SRE_MODE_FP32 && (sre::one_applies(N, eb) || sre::two_applies(N, eb));
+    const bool fixed = p->mode == SRE_MODE_FP32 && (sre::one_applies(N, eb) || (sre::two_applies(N, eb) && N < 20));
     if (fixed) add(base);
     for (int C_log = 0; !fixed && C_log <= 3; ++C_log)
         for (int g = 0; g <= 3; ++g)
@@ -362,7 +362,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
                         add(w);
                     }
                     // both copy paths where they apply
-                    const bool tma = eb == 8 && h2 >= 5 && h2 <= 8;
+                    const bool tma = eb == 8 && h2 >= 7 && h2 <= 8;
                     for (int s1 = (C_log == 0 && eb == 8 && !tc) ? 0 : 1; s1 <= 1; ++s1)
                         for (int s2 = (tma && !tc) ? 0 : 1; s2 <= 1; ++s2) {
                             c.stage1 = s1;
@@ -639,7 +639,7 @@ sre_status_t sre_m2_batched(sre_plan_t p, const void *const *d_states, const int
     for (int n = 0; n <= SRE_MAX_QUBITS; ++n) {
         tuned[n] = nullptr;
         if (n > sre::kTileBits && n <= p->N) {
-            p->batch_cfg[n] = plan_cfg(p, n);
+            p->batch_cfg[n] = plan_cfg(p, n, 1ull << n);
             tuned[n] = &p->batch_cfg[n];
         }
     }

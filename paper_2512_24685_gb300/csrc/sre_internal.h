@@ -41,7 +41,8 @@ struct LargeCfg {
     int B1_log;  // log2 consecutive blocks per pass-1 work item
     int grid;    // persistent CTAs
     int stage1 = 1;  // pass 1 by bulk copy where available (C = 1, FP32, aligned)
-    int stage2 = 1;  // pass 2 by TMA tile copies where available (FP32, 5 <= h2 <= 8)
+    int stage2 = 1;  // pass 2 by TMA tile copies where available (FP32, h2 = 7 and 8)
+    bool two = false;  // FP32, N = 20: the library's choice is the kernel of sre_two.cu
 };
 
 // Everything one evaluation needs on the device (owned by a plan or a
@@ -90,12 +91,13 @@ cudaError_t query_device(DeviceInfo *info);
 // entries).
 LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half);
 
-// The library's two-pass configuration for the main shift range of an
-// arithmetic mode (every shift, in the split modes those from 4096), and whether a configuration fits a workspace.
-LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode);
+// The library's two-pass configuration for a number of shifts in an arithmetic
+// mode (in the split modes those from 4096).
+LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, uint64_t shifts);
 // The configuration that a caller's partial tuning completes: with a ring field
 // of the caller's own, the L2-sized one, whose lag and slots leave room for it.
-LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t);
+LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t,
+                         uint64_t shifts);
 
 // Tensor-core two-pass kernel (sre_tc.cu) for the halved shifts of one
 // state: tc_kind 1 = BF16 hi/lo pieces, 2 = FP16 hi/lo pieces.  tc_applies
@@ -143,6 +145,7 @@ struct BatchClass {
     size_t parts_off = 0, parts_n = 0;     // partials of the class
     size_t chunks_max = 0;                 // counters needed by one launch
     int tc_kind = 0;                       // split modes: the halved shifts on the tensor cores
+    bool two = false;                      // the kernel of sre_two.cu
 };
 
 // tc_kind: the class takes the tensor-core kernel for its halved shifts.

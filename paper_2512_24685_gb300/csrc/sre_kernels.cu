@@ -12,7 +12,7 @@
 //   k_small     N <= 12, FP32: one 2^12-entry tile holds 2^(13-N) whole shifts
 //               (halved form); the state sits in shared memory; static
 //               tile->CTA assignment.  k_small_fx: the same in fixed point
-//   k_large     fixed point N >= 15, FP32 N >= 21: persistent two-pass kernel
+//   k_large     fixed point N >= 15, FP32 N >= 20: persistent two-pass kernel
 //               (sre_large.cuh); the sizes between run in sre_mid.cu,
 //               sre_one.cu and sre_two.cu
 //   k_finalize  fixed-order FP64 sums of the partials, M2 and the status.
@@ -349,7 +349,7 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half
     while (C_log > 0 && (double)c.R * (double)(1 << C_log) * per_x > budget) --C_log;
     c.C_log = C_log;
     c.G2_log = std::min(C_log, h2);
-    // pass 2 staged through TMA (FP32, 5 <= h2 <= 8) overlaps the copy of
+    // pass 2 staged through TMA (FP32, h2 = 7 and 8) overlaps the copy of
     // tile g + 2 with tile g: give each item four tiles or more
     c.stage1 = 1;
     c.stage2 = 1;
@@ -381,16 +381,45 @@ static LargeCfg choose_tc_cfg(const DeviceInfo &dev, const Workspace &ws, int N)
     return c;
 }
 
-LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode) {
+// FP32 at N = 20: one shift per chunk, block pairs and tiles by bulk and tensor
+// copies, eight blocks and eight tiles per item, and all the slots that the
+// tuning scratch holds (47 of 4 MB).  1.90 s for a whole state, against 1.97 s
+// by the item-list kernel of sre_two.cu.  A short ring makes this kernel wait (96 MB: 2.46 s): with less
+// scratch long ranges take the other one (2.36 s), and so does a handful of
+// shifts (one 76 against 84 us, 32 161 against 133 us).
+constexpr int kFp32LargeN = 20, kFp32Ring = 47;
+static LargeCfg choose_fp32_20_cfg(const DeviceInfo &dev, const Workspace &ws, uint64_t shifts) {
+    LargeCfg c = choose_large_cfg(dev, kFp32LargeN, 8, 1);
+    const int R = (int)std::min<size_t>(kFp32Ring, ws.scratch_bytes / ((size_t)8 << (kFp32LargeN - 1)));
+    if (shifts < 16 || (R < kFp32Ring && shifts >= 16384)) {
+        c.two = true;
+    } else if (R >= 23) {
+        c.C_log = 0;
+        c.R = R;
+        c.D = (R - 1) / 2;
+        c.G2_log = c.B1_log = 3;
+    }
+    return c;
+}
+
+LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, uint64_t shifts) {
     const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
+    if (mode == SRE_MODE_FP32 && N == kFp32LargeN) return choose_fp32_20_cfg(dev, ws, shifts);
     if (tc_mode_available(mode) && tc_applies(N, 1, 2, nullptr)) return choose_tc_cfg(dev, ws, N);
     return choose_large_cfg(dev, N, eb, 1);
 }
 
-LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t) {
+LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t,
+                         uint64_t shifts) {
     if (t.x_batch_log >= 0 || t.ring_slots >= 0 || t.lag >= 0)
         return choose_large_cfg(dev, N, mode == SRE_MODE_FP64 ? 16 : 8, 1);
-    return choose_main_cfg(dev, ws, N, mode);
+    return choose_main_cfg(dev, ws, N, mode, shifts);
+}
+
+// FP32 shifts of N = 17..20 by sre_two.cu: N = 20 only where the library chose
+// it, and beside the tensor-core kernel.
+static bool takes_two(int N, int elem_bytes, int tc_kind, const LargeCfg &c) {
+    return two_applies(N, elem_bytes) && (N < kFp32LargeN || tc_kind || c.two);
 }
 
 size_t workspace_scratch_bytes(const DeviceInfo &dev, int N_max, int elem_bytes, sre_mode_t mode) {
@@ -548,7 +577,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 cudaError_t encode_p2_tmap(LargeArgs &a) {
     auto enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
-    if (a.h2 != 8 || ((uintptr_t)a.scratch & 15)) return cudaErrorInvalidValue;
+    if (a.h2 < 7 || a.h2 > 8 || ((uintptr_t)a.scratch & 15)) return cudaErrorInvalidValue;
     const cuuint64_t rows = (cuuint64_t)a.R << (a.C_log + a.h2);
     if (rows > 0xFFFFFFFFull) return cudaErrorInvalidValue;
     const cuuint64_t dims[2] = {2ull * kTile, rows};
@@ -577,18 +606,18 @@ static cudaError_t launch_large_h(const LargeArgs &a, int grid, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// FP32: N >= 21 (smaller sizes run in sre_one.cu and sre_two.cu); fixed point:
+// FP32: N >= 20 (smaller sizes run in sre_one.cu and sre_two.cu); fixed point:
 // N >= 15.
 template <typename R>
 static cudaError_t launch_large(const LargeArgs &a, int grid, cudaStream_t st) {
     switch (a.h2) {
 #define SRE_CASE(n) \
     case n: return launch_large_h<R, n>(a, grid, st);
-        SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11)
+        SRE_CASE(7) SRE_CASE(8) SRE_CASE(9) SRE_CASE(10) SRE_CASE(11)
 #undef SRE_CASE
 #define SRE_CASE(n) \
     case n: if constexpr (sizeof(cx_t<R>) == 16) return launch_large_h<R, n>(a, grid, st); break;
-        SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6) SRE_CASE(7)
+        SRE_CASE(2) SRE_CASE(3) SRE_CASE(4) SRE_CASE(5) SRE_CASE(6)
 #undef SRE_CASE
     }
     return cudaErrorInvalidValue;
@@ -598,8 +627,7 @@ static cudaError_t launch_large(const LargeArgs &a, int grid, cudaStream_t st) {
 static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const DeviceInfo &dev,
                                    const void *psi, int N, uint64_t xb, uint64_t xe, int half,
                                    int elem_bytes, size_t chunk_off, double *per_x,
-                                   long long wait_ns, const LargeCfg *ovr, int *grid) {
-    const LargeCfg c = ovr ? *ovr : choose_large_cfg(dev, N, elem_bytes, half);
+                                   long long wait_ns, const LargeCfg &c, int *grid) {
     LargeArgs &A = *a;
     A.psi = psi;
     A.psis = nullptr;
@@ -713,6 +741,8 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         const bool tc = tc_kind && tc_applies(N, 1, alpha, psi);
         const uint64_t split = tc ? std::min<uint64_t>(std::max<uint64_t>(x_begin, kTile), x_end) : x_end;
         const bool single_pass = one_applies(N, eb) || mid_applies(N, eb);
+        const sre_mode_t mode = kFx ? SRE_MODE_FP64 : tc_kind ? SRE_MODE_FP16_SPLIT : SRE_MODE_FP32;
+        const LargeCfg main = cfg_override ? *cfg_override : choose_main_cfg(dev, ws, N, mode, x_end - split + (tc ? 0 : split - x_begin));
         // chunk counters: not for a shift per CTA
         if ((tc || !single_pass) &&
             (e = cudaMemsetAsync(ws.counters, 0, sizeof(unsigned) * 3 * ws.chunk_cap, st)) != cudaSuccess)
@@ -732,7 +762,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                 else
                     e = launch_one(N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, d_per_x, ws.work + 2,
                                    ws.status, wait_ns, dev, st);
-            } else if (two_applies(N, eb)) {
+            } else if (takes_two(N, eb, tc_kind, main)) {
                 name = "k_two";
                 const LargeCfg c = choose_two_cfg(dev, ws, N);
                 e = launch_two(ws, c, N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, ws.counters,
@@ -743,7 +773,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                 LargeArgs a;
                 int grid = 0;
                 if ((e = make_large_args(&a, ws, dev, psi, N, x_begin, split, 1, eb, 0, d_per_x, wait_ns,
-                                         cfg_override, &grid)) != cudaSuccess)
+                                         main, &grid)) != cudaSuccess)
                     return e;
                 a.alpha = alpha;
                 e = launch_large<R>(a, grid, st);
@@ -758,9 +788,8 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         if (tc && split < x_end) {
             LargeArgs a;
             int grid = 0;
-            const LargeCfg c = cfg_override ? *cfg_override : choose_tc_cfg(dev, ws, N);
             if ((e = make_large_args(&a, ws, dev, psi, N, split, x_end, 1, eb, chunks,
-                                     d_per_x ? d_per_x + (split - x_begin) : nullptr, wait_ns, &c,
+                                     d_per_x ? d_per_x + (split - x_begin) : nullptr, wait_ns, main,
                                      &grid)) != cudaSuccess)
                 return e;
             a.alpha = alpha;
@@ -925,10 +954,12 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         L.parts_n = (size_t)S * (size_t)tps;
         return L;
     }
+    const LargeCfg main = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode, 1ull << N);
+    L.two = takes_two(N, eb, tc_kind, main);
     if (one_applies(N, eb)) {
         // one partial per shift, all shifts or those below 4096 beside the
         // tensor-core kernel
-        L.cfg_half = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode);
+        L.cfg_half = main;
         L.cps_full = tc_kind ? (long long)kTile : 0;
         L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)
                              : 1ll << N;
@@ -936,12 +967,12 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         L.chunks_max = tc_kind ? (size_t)S * (size_t)L.cps_half : 1;
         return L;
     }
-    if (two_applies(N, eb)) {
+    if (L.two) {
         // every shift in one launch, or the shifts below 4096 beside the
         // tensor-core kernel
         L.cfg_full = choose_two_cfg(dev, ws, N);
         L.cfg_half = L.cfg_full;
-        if (tc_kind) L.cfg_half = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode);
+        if (tc_kind) L.cfg_half = main;
         L.cps_full = tc_kind ? two_layout(ws, L.cfg_full, N, 0, kTile).n_chunks : 0;
         L.cps_half = tc_kind ? (long long)((((1ull << N) - kTile) + (1ull << L.cfg_half.C_log) - 1) >> L.cfg_half.C_log)
                              : two_layout(ws, L.cfg_half, N, 0, 1ull << N).n_chunks;
@@ -949,7 +980,7 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         L.chunks_max = (size_t)S * (size_t)std::max(L.cps_full, L.cps_half);
         return L;
     }
-    L.cfg_half = tuned_half ? *tuned_half : choose_large_cfg(dev, N, eb, 1);
+    L.cfg_half = main;
     // the single-pass kernel has one partial per shift
     if (mid_applies(N, eb)) L.cfg_half.C_log = 0;
     L.cps_full = 0;
@@ -990,7 +1021,7 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
                 off += (size_t)cps * L.S;
                 continue;
             }
-            if (two_applies(N, 8) && !(half && L.tc_kind)) {
+            if (L.two && !(half && L.tc_kind)) {
                 if (cps == 0) continue;
                 if ((e = cudaMemsetAsync(counters, 0, sizeof(unsigned) * 3 * chunk_cap, st)) != cudaSuccess) return e;
                 if ((e = cudaMemsetAsync(ws.work, 0, kWorkBytes, st)) != cudaSuccess) return e;

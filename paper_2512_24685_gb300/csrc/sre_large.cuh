@@ -1,5 +1,5 @@
 // sre_large.cuh -- the persistent two-pass CUDA-core kernel of libsre (fixed
-// point: N >= 15; FP32: N >= 21, smaller sizes run in sre_one.cu and
+// point: N >= 15; FP32: N >= 20, smaller sizes run in sre_one.cu and
 // sre_two.cu), and the work-item order and bounded waits it shares with the
 // tensor-core kernel of sre_tc.cu.
 #pragma once
@@ -49,7 +49,7 @@ using namespace dev;
 // with a zero inserted at bit j - 12; below that it removes a bit of the block,
 // and x = 0 pairs the halves of the state (BlockPair).  h2 = N - 13.
 //
-// FP32 launches with h2 = 8 (N = 21) stage pass-2 tiles through TMA
+// FP32 launches with h2 = 7 and 8 (N = 20, 21) stage pass-2 tiles through TMA
 // (sre_stage.cuh): tmap then describes the scratch ring as a 2-D FP32 array
 // of 8192 columns (4096 complex per block t'_h) by R * C * 2^h2 rows.  The
 // tensor-core kernel (sre_tc.cu) describes its 16-bit scratch planes there
@@ -133,7 +133,7 @@ __device__ __forceinline__ void decode_item(const LargeArgs &a, long long item, 
 // Pass 2 of this instantiation stages its tiles through TMA.
 template <typename R, int H2>
 __host__ __device__ constexpr bool large_uses_tma() {
-    return sizeof(R) == 4 && H2 == 8;
+    return sizeof(R) == 4 && (H2 == 7 || H2 == 8);
 }
 
 // Pass 1 of this instantiation can take its block pairs by bulk copy (FP32

@@ -390,7 +390,7 @@ sre_status_t sre_server_create(const sre_server_cfg_t *cfg, sre_server_t *out) {
 
 sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t) {
     if (!s || !t || N <= sre::kTileBits || N > s->cfg.max_N) return SRE_EINVAL;
-    sre::LargeCfg c = sre::tuning_base_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode, *t);
+    sre::LargeCfg c = sre::tuning_base_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode, *t, 1ull << N);
     if (t->x_batch_log >= 0) c.C_log = t->x_batch_log;
     if (t->ring_slots >= 0) c.R = t->ring_slots;
     if (t->lag >= 0) c.D = t->lag;
@@ -405,10 +405,10 @@ sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t)
     if (!sre::large_cfg_fits(s->slots[0].ws, c, N, 1)) {
         sre::Workspace plan_ws;
         plan_ws.scratch_bytes = sre::kTuneScratch;
-        const sre::LargeCfg lib = sre::choose_main_cfg(s->dev, plan_ws, N, s->cfg.mode);
+        const sre::LargeCfg lib = sre::choose_main_cfg(s->dev, plan_ws, N, s->cfg.mode, 1ull << N);
         if (c.C_log == lib.C_log && c.R == lib.R && c.D == lib.D && c.G2_log == lib.G2_log &&
             c.B1_log == lib.B1_log && c.stage1 == lib.stage1 && c.stage2 == lib.stage2)
-            c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode);
+            c = sre::choose_main_cfg(s->dev, s->slots[0].ws, N, s->cfg.mode, 1ull << N);
     }
     std::lock_guard<std::mutex> lk(s->mu);
     for (const Slot &sl : s->slots)
