@@ -1,19 +1,21 @@
-// sre_two.cu -- FP32 two-pass kernel for 17 <= N <= 20, all shifts in the
-// halved form (sre_wht32.cuh).
+// sre_two.cu -- FP32 two-pass kernel for 17 <= N <= 19, all shifts in the
+// halved form (sre_wht32.cuh); at N = 20 for the shifts below 4096 beside the
+// tensor-core kernel, a handful of shifts, and slots with a short ring.
 //
 // Pass 1 (one item: a block of 8192 entries for the 2^C_log shifts that share
 // its factors) forms the products, transforms the 13 block bits and writes
 // the block to a slot of a scratch ring as one row; pass 2 (one item: a set of
 // columns of the rows) transforms the N - 14 row bits in registers and sums
-// the powers.  The factors of a block are loaded once per item into tensor
-// memory: the item's shifts differ only in block bits that index registers, so
+// the powers.  In long ranges the factors of a block are loaded once per item into
+// tensor memory: the item's shifts differ only in block bits that index registers, so
 // each thread finds its own and its partner factors for all of them in its own
 // tensor-memory columns, the partner's by an XOR of the column address, and
 // the loads leave the L1 pipe.
 //
-// Shifts are grouped in chunks: 2^C_log shifts 2^(13 - C_log) apart times 2^U_log
-// consecutive ones (U_log > 0 where few blocks make a shift, so that a chunk
-// has 16 items per pass or more).  A chunk owns one ring slot from its first
+// Shifts are grouped in chunks: 2^C_log shifts per item, 2^(13 - C_log) apart where
+// they share factors (long ranges), else consecutive ones, times 2^U_log items
+// per block (U_log > 0 where few blocks make a shift, so that a chunk has 16 items
+// per pass or more).  A chunk owns one ring slot from its first
 // pass-1 item to its last pass-2 item.
 //
 // What bounds it: about 31 SM cycles per 32 entries of the halved transform at
@@ -60,6 +62,12 @@ struct TwoArgs {
     int *status;
     long long wait_ns;
 };
+
+// Spacing (log2) of an item's shifts, and of a chunk's shifts in other items.
+template <bool SHARE>
+__device__ __forceinline__ int two_spacing(const TwoArgs &a) { return SHARE ? kBlockBits - a.C_log : 0; }
+template <bool SHARE>
+__device__ __forceinline__ int two_item_spacing(const TwoArgs &a) { return SHARE ? 0 : a.C_log; }
 
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
@@ -264,7 +272,7 @@ struct TwoDone {
     uint64_t xc;  // the chunk's first shift
 };
 
-template <int H2>
+template <int H2, bool SHARE>
 __device__ __noinline__ void two_publish(const TwoArgs &a, TwoDone *d) {
     const int lane = threadIdx.x & 31, C = 1 << a.C_log, S_log = a.C_log + a.U_log, P_log = H2 + a.U_log;
     const long long c = d->t.c;
@@ -294,7 +302,8 @@ __device__ __noinline__ void two_publish(const TwoArgs &a, TwoDone *d) {
             double sx = 0.0;
             for (int m = lane; m < (kParts << H2); m += 32) sx += __ldcg(ip + m);
             sx = hfac * warp_sum(sx);
-            const uint64_t x = d->xc + (uint64_t)(q >> a.C_log) + ((uint64_t)(q & (C - 1)) << (kBlockBits - a.C_log));
+            const uint64_t x = d->xc + ((uint64_t)(q >> a.C_log) << two_item_spacing<SHARE>(a)) +
+                               ((uint64_t)(q & (C - 1)) << two_spacing<SHARE>(a));
             if (lane == 0 && a.per_x && x >= a.x_begin && x < a.x_end) a.per_x[x - a.x_begin] = sx;
             cs += sx;
         }
@@ -315,7 +324,7 @@ __device__ __noinline__ void two_publish(const TwoArgs &a, TwoDone *d) {
     __syncwarp();
 }
 
-template <int H2>
+template <int H2, bool SHARE>
 __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_constant__ TwoArgs a) {
     extern __shared__ __align__(1024) unsigned char buf[];
     __shared__ TwoItem s_next;
@@ -326,7 +335,7 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
     const int C = 1 << a.C_log, S_log = a.C_log + a.U_log;
     const int P_log = H2 + a.U_log;  // items per chunk and pass
 
-    if (warp == 0) tc_alloc(&s_tmem, 2 * kFactorCols);
+    if (SHARE && warp == 0) tc_alloc(&s_tmem, 2 * kFactorCols);
     TwoClaim claim;  // thread 0
     if (tid == 0) {
         s_done.t.c = -1;
@@ -336,7 +345,7 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
     __syncthreads();
     tc_fence_after();
     // this warp's 32 lanes; warps w and w + 4 share them
-    const uint32_t tmem = s_tmem + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * kFactorCols;
+    const uint32_t tmem = SHARE ? s_tmem + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * kFactorCols : 0;
     while (s_next.c >= 0) {
         const long long c = s_next.c;
         const int r = s_next.r, slot = s_next.slot;
@@ -348,29 +357,34 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
             cl = c - sidx * a.chunks_per_state;
             psi = reinterpret_cast<const float2 *>(a.psis[sidx]);
         }
-        // chunk cl: shifts xc + (k << (13 - C_log)) + u, k < 2^C_log, u < 2^U_log
+        // chunk cl: shifts k < 2^C_log of items u < 2^U_log, from xc
         const int cw_log = a.W_log - S_log, u = r >> H2, b = r & ((1 << H2) - 1);
         const uint64_t xc = a.x0 + ((uint64_t)(cl >> cw_log) << a.W_log) +
                             ((uint64_t)(cl & ((1ll << cw_log) - 1)) << a.U_log);
-        const uint64_t x0 = xc + (uint64_t)u;
+        const uint64_t x0 = xc + ((uint64_t)u << two_item_spacing<SHARE>(a));
         // the item's first scratch row block
         float2 *base = a.scratch + ((((((size_t)slot << a.U_log) + (size_t)u) << a.C_log)) << (H2 + kBlockBits));
         if (pass1) {
             bool filled = false;
             for (int k = 0; k < C; ++k) {
-                const uint64_t x = x0 + ((uint64_t)k << (kBlockBits - a.C_log));
+                const uint64_t x = x0 + ((uint64_t)k << two_spacing<SHARE>(a));
                 const bool claiming = tid == 0 && k + 1 == C;
                 if (claiming) two_step(a, claim, P_log);
                 __syncwarp();
                 if (x < a.x_begin || x >= a.x_end) continue;
                 // from x = 8192 up the item's shifts share the pivot and differ
-                // in register bits alone: one fill serves them all
-                const bool shared = x >= (1u << kBlockBits);
-                if (!shared || !filled) w32_fill(tmem, pair_src(psi, a.N, shared ? x0 : x, b), tid);
-                filled = shared;
-                if (warp == kPubWarp) two_publish<H2>(a, &s_done);
+                // in register bits alone: one fill serves them all.  A shift
+                // that shares nothing takes its factors straight to registers
                 c64_t v[32];
-                w32_products(v, tmem, shared ? (uint32_t)k << (3 - a.C_log) : 0u);
+                if (SHARE && x >= (1u << kBlockBits)) {
+                    if (!filled) w32_fill(tmem, pair_src(psi, a.N, x0, b), tid);
+                    filled = true;
+                    if (warp == kPubWarp) two_publish<H2, SHARE>(a, &s_done);
+                    w32_products(v, tmem, (uint32_t)k << (3 - a.C_log));
+                } else {
+                    if (warp == kPubWarp) two_publish<H2, SHARE>(a, &s_done);
+                    w32_direct<0, 32>(v, pair_src(psi, a.N, x, b), tid);
+                }
                 if (claiming) two_step(a, claim, P_log);
                 __syncwarp();
                 w32_block(v, buf, tid);
@@ -389,7 +403,7 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
         } else {
             const int wc = (b * Cols::kParts + warp) * Cols::kWarpCols;
             for (int k = 0; k < C; ++k) {
-                const uint64_t x = x0 + ((uint64_t)k << (kBlockBits - a.C_log));
+                const uint64_t x = x0 + ((uint64_t)k << two_spacing<SHARE>(a));
                 const bool claiming = tid == 0 && k + 1 == C;
                 if (claiming) two_step(a, claim, P_log);
                 __syncwarp();
@@ -399,7 +413,7 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
                     s = two_columns<H2>(cols + lane * Cols::V, a.alpha);
                     if (claiming) two_step(a, claim, P_log);
                     __syncwarp();
-                    if (warp == kPubWarp) two_publish<H2>(a, &s_done);
+                    if (warp == kPubWarp) two_publish<H2, SHARE>(a, &s_done);
                     s = warp_sum(s);
                     if (claiming) two_step(a, claim, P_log);
                     __syncwarp();
@@ -419,7 +433,7 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
                 }
             }
         }
-        if (warp == kPubWarp) two_publish<H2>(a, &s_done);  // an item without work has not come by it
+        if (warp == kPubWarp) two_publish<H2, SHARE>(a, &s_done);  // an item without work has not come by it
         __syncthreads();
         if (warp == kPubWarp && lane == 0) {
             s_done.t.c = c;
@@ -429,7 +443,7 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
         if (tid == 0) s_next = two_take(a, claim, P_log);
         __syncthreads();
         if (s_next.c == -1) {
-            if (warp == kPubWarp) two_publish<H2>(a, &s_done);
+            if (warp == kPubWarp) two_publish<H2, SHARE>(a, &s_done);
             TwoItem t;
             if (tid == 0) {
                 t = two_claim(a, claim, P_log);
@@ -440,16 +454,16 @@ __global__ void __launch_bounds__(kBlockThreads, kTwoCtas) k_two(const __grid_co
             __syncthreads();
         }
     }
-    if (warp == kPubWarp) two_publish<H2>(a, &s_done);
+    if (warp == kPubWarp) two_publish<H2, SHARE>(a, &s_done);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tc_dealloc(s_tmem, 2 * kFactorCols);
+    if (SHARE && warp == 0) tc_dealloc(s_tmem, 2 * kFactorCols);
 }
 
 template <int H2>
-cudaError_t launch_two_h(const TwoArgs &a, int grid, cudaStream_t st) {
-    auto kern = k_two<H2>;
+cudaError_t launch_two_h(const TwoArgs &a, bool share, int grid, cudaStream_t st) {
+    auto kern = share ? k_two<H2, true> : k_two<H2, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMoveBytes);
     if (e != cudaSuccess) return e;
     kern<<<grid, kBlockThreads, kMoveBytes, st>>>(a);
@@ -498,10 +512,16 @@ TwoLayout two_layout(const Workspace &ws, const LargeCfg &c, int N, uint64_t xb,
     TwoLayout L;
     L.U_log = two_u_log(N);
     while (L.U_log > 0 && !two_fits(ws, c, N, L.U_log)) --L.U_log;
-    // short ranges take consecutive shifts: windows of 8192 would be mostly empty
-    L.C_log = xe - xb >= 16384 ? c.C_log : 0;
+    // Windows of 8192 shifts whose items share factors; a shorter range would
+    // leave most of a window empty and takes consecutive shifts, which share no
+    // factors but a claim and a publication per item (N = 17, us for 2048 and
+    // 8192 shifts: 575 and 2054; one shift per item: 769 and 2940; the general
+    // kernel: 677 and 2551), fewer of them where the items run out.
+    const uint64_t n = xe - xb;
+    L.share = n >= 16384 && c.C_log > 0;
+    L.C_log = n >= 1024 ? c.C_log : n >= 256 ? std::min(c.C_log, 1) : 0;
     L.R = c.R << (c.C_log - L.C_log);
-    L.W_log = L.C_log ? kBlockBits : L.U_log;
+    L.W_log = L.share ? kBlockBits : L.C_log + L.U_log;
     L.x0 = xb & ~((1ull << L.W_log) - 1);
     const uint64_t windows = (xe - L.x0 + (1ull << L.W_log) - 1) >> L.W_log;
     L.n_chunks = (long long)(windows << (L.W_log - L.C_log - L.U_log));
@@ -542,10 +562,10 @@ cudaError_t launch_two(const Workspace &ws, const LargeCfg &c, int N, const void
     a.wait_ns = wait_ns;
     const int grid = (int)std::max<long long>(1, std::min<long long>(c.grid, n_items));
     switch (two_h2(N)) {
-        case 3: return launch_two_h<3>(a, grid, st);
-        case 4: return launch_two_h<4>(a, grid, st);
-        case 5: return launch_two_h<5>(a, grid, st);
-        case 6: return launch_two_h<6>(a, grid, st);
+        case 3: return launch_two_h<3>(a, L.share, grid, st);
+        case 4: return launch_two_h<4>(a, L.share, grid, st);
+        case 5: return launch_two_h<5>(a, L.share, grid, st);
+        case 6: return launch_two_h<6>(a, L.share, grid, st);
     }
     return cudaErrorInvalidValue;
 }

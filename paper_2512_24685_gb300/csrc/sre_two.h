@@ -8,6 +8,7 @@ namespace sre {
 
 struct TwoLayout {
     int C_log, U_log, W_log, R;
+    bool share;  // an item's shifts share factors (sre_two.cu)
     uint64_t x0;
     long long n_chunks;  // per state
 };
