@@ -143,6 +143,9 @@ struct SmallTail {
     double *d_m2 = nullptr;
 };
 static_assert(kNormBlocks * kThreads >= kTile, "one entry per thread of k_norm");
+// Norm partials with entries; a launch has a CTA for each, however short its
+// range: one CTA that forms all sixteen of N = 12 takes 10 us more.
+constexpr int small_norm_blocks(int N) { return ((1 << N) + kThreads - 1) / kThreads; }
 
 // ------------------------------------------------------- N <= 12: k_small
 
@@ -203,10 +206,11 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
         if (tid == 0) part[g] = s;
     }
     if (!tail.npart) return;
-    constexpr int kUsed = (d + kThreads - 1) / kThreads;  // norm blocks with entries
+    constexpr int kUsed = small_norm_blocks(N);
     for (int b = blockIdx.x; b < kUsed; b += gridDim.x) {
         const int t = b * kThreads + tid;
-        const V e = t < d ? psi_s[pad(t)] : V{0, 0};
+        // a CTA without a tile has no copy of the state
+        const V e = t >= d ? V{0, 0} : cur < 0 ? psi[t] : psi_s[pad(t)];
         const double re = (double)e.x, im = (double)e.y;
         __syncthreads();  // red is free
         const double s = block_sum(re * re + im * im, red);
@@ -526,9 +530,9 @@ static cudaError_t launch_small_nb(const void *psi, const void *const *psis, int
     const long long tps = (long long)((flat + kTile - 1) >> kTileBits);
     const long long ntiles = tps * nstates;
     if (ntiles > part_cap) return cudaErrorInvalidValue;
-    const int grid = forced_grid > 0 ? forced_grid
-                                     : (int)std::min<long long>(ntiles, (long long)dev.sms * 2);
+    int grid = forced_grid > 0 ? forced_grid : (int)std::min<long long>(ntiles, (long long)dev.sms * 2);
     if (grid < 1) return cudaErrorInvalidValue;
+    if (tail.npart) grid = std::max(grid, small_norm_blocks(NB + 1));
     if constexpr (kFx)
         k_small_fx<NB><<<grid, kThreads, smem, st>>>(reinterpret_cast<const double2 *>(psi), psis, tps, x_begin, x_end,
                                                      ntiles, part, alpha);

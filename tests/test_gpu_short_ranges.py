@@ -45,3 +45,28 @@ def test_orders_in_short_ranges(sre, alpha):
         _, px = p.sum_pow_range(psi, alpha, 8185, 8185 + 300, per_x=True)
         _, py = p.sum_pow_range(psi, alpha, 8185, 8185 + 20, per_x=True)
     assert torch.equal(px[:20], py)
+
+
+def _us(call, reps=200):
+    import torch
+    best = float("inf")
+    for _ in range(6):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(reps):
+            call()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / reps * 1e3)
+    return best
+
+
+def test_one_shift_of_a_small_state_costs_no_more_than_many(sre):
+    """The norm of a state in one tile is spread over CTAs however short the
+    range is (by the range's only CTA: 35 us against 21).  30 % between runs."""
+    import torch
+    psi = torch.from_numpy(W.haar_state(12, 3, np.complex64)).cuda()
+    with sre.Plan(12, "c64") as p:
+        n2 = [p.sum4_range(psi, b, e)[1].item() for b, e in ((0, 4096), (5, 6), (4000, 4003), (0, 70))]
+        assert len(set(n2)) == 1
+        assert _us(lambda: p.sum4_range(psi, 5, 6)) <= 1.3 * _us(lambda: p.sum4_range(psi, 0, 64))
