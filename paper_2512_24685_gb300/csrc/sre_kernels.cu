@@ -409,7 +409,10 @@ static LargeCfg choose_fp32_20_cfg(const DeviceInfo &dev, const Workspace &ws, u
 LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, uint64_t shifts) {
     const int eb = mode == SRE_MODE_FP64 ? 16 : 8;
     if (mode == SRE_MODE_FP32 && N == kFp32LargeN) return choose_fp32_20_cfg(dev, ws, shifts);
-    if (tc_mode_available(mode) && tc_applies(N, 1, 2, nullptr)) return choose_tc_cfg(dev, ws, N);
+    // fewer than 64 shifts leave most SMs without an item of the large chunks:
+    // one shift of N = 18 takes 87 us in small ones, 108 in large ones; 48 shifts
+    // 105 and 121, 128 shifts 154 and 144
+    if (tc_mode_available(mode) && tc_applies(N, 1, 2, nullptr) && shifts >= 64) return choose_tc_cfg(dev, ws, N);
     return choose_large_cfg(dev, N, eb, 1);
 }
 

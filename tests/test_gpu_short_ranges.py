@@ -70,3 +70,16 @@ def test_one_shift_of_a_small_state_costs_no_more_than_many(sre):
         n2 = [p.sum4_range(psi, b, e)[1].item() for b, e in ((0, 4096), (5, 6), (4000, 4003), (0, 70))]
         assert len(set(n2)) == 1
         assert _us(lambda: p.sum4_range(psi, 5, 6)) <= 1.3 * _us(lambda: p.sum4_range(psi, 0, 64))
+
+
+def test_a_handful_of_shifts_in_a_split_mode_takes_small_items(sre):
+    """One shift of N = 18 beside the same with an L2-sized ring of small chunks,
+    which a caller can ask for (in chunks of eight shifts 24 % slower).  10 %
+    between runs."""
+    import torch
+    psi = torch.from_numpy(W.haar_state(18, 3, np.complex64)).cuda()
+    x = (1 << 17) + 1
+    with sre.Plan(18, "c64", "fp16_split") as p:
+        library = _us(lambda: p.sum4_range(psi, x, x + 1))
+        p.set_tuning(1, 23, 11, 3, 0)
+        assert library <= 1.1 * _us(lambda: p.sum4_range(psi, x, x + 1))
