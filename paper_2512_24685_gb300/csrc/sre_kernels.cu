@@ -196,13 +196,14 @@ __global__ void __launch_bounds__(kThreads) k_small(const v2_t<R> *__restrict__ 
                 const int t = (((int)(flat & ((1u << NB) - 1)) - lo) << 1) | lo;
                 v[i] = x ? pair_value<R, false>(psi_s[pad(t ^ xe)], psi_s[pad(t)])
                          : pair_value<R, true>(psi_s[pad(t ^ xe)], psi_s[pad(t)]);
+                v[i] = Cx<R>::add(v[i], v[i]);  // fp32_doubled
             } else {
                 v[i] = Cx<R>::zero();
             }
         }
         tile_fwht<NB, R>(v, bufA, bufB, tid);
         // block_sum's barriers also protect bufB before the next tile
-        const double s = block_sum(half_scale<R>((double)sum_order<R>(v, alpha), alpha, 0), red);
+        const double s = block_sum((double)sum_order<R>(v, alpha), red);
         if (tid == 0) part[g] = s;
     }
     if (!tail.npart) return;
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_small_fx(const double2 *__restr
         }
         const FxExp u = fx_tile<NB>(v, buf, tid, sh);
         const double s = block_sum(sum_order<fx>(v, alpha), red);
-        if (tid == 0) part[g] = half_scale<fx>(s, alpha, u.c);
+        if (tid == 0) part[g] = fx_scale(s, alpha, u.c);
     }
 }
 

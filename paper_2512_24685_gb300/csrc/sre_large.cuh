@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         }
                         const unsigned char *stage = reinterpret_cast<const unsigned char *>(st ? bufC : bufB);
                         const float s = p2_tile<H2>(stage, reinterpret_cast<float2 *>(bufA), pl, a.alpha);
-                        acc += half_scale<R>((double)s, a.alpha, 0);
+                        acc += (double)s;
                         if (gb + 2 < ntiles) {
                             __syncthreads();  // every thread has read stage st
                             if (tid == 0) {
@@ -469,14 +469,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                         acc += sum_order<R>(v, a.alpha);
                     } else {
                         tile_fwht<H2, R>(v, bufA, bB, tid);
-                        acc += half_scale<R>((double)sum_order<R>(v, a.alpha), a.alpha, 0);
+                        acc += (double)sum_order<R>(v, a.alpha);
                     }
                 }
             }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-            if constexpr (kFx) acc = half_scale<R>(acc, a.alpha, fxk);
+            acc = kFx ? fx_scale(acc, a.alpha, fxk) : fp32_scale(fp32_doubled(x), a.alpha) * acc;
             // All warps' loads of this item are complete after this barrier:
             // drop the item's scratch lines from L2 without write-back (dead
             // data; the next chunk in this slot rewrites them; the staged path

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 2 : 1)
         s += sum_order<fx>(v, alpha);
         const double units = block_sum(s, red);
         if (tid == 0) {
-            const double tot = half_scale<fx>(units, alpha, k);
+            const double tot = fx_scale(units, alpha, k);
             part[g] = tot;
             if (per_x) per_x[g] = tot;
         }

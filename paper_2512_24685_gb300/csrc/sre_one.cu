@@ -48,6 +48,10 @@ struct One {
     static constexpr int kTmemBlocks = kBlocks == 1 ? 0 : kBlocks == 2 ? 1 : 2;
     static constexpr bool kHalfMove = kBlocks == 4;
     static constexpr size_t kSmem = kHalfMove ? kMoveBytes / 2 + 8192 * sizeof(float2) : kMoveBytes;
+    // Doubled products below x = 4096 (fp32_doubled).  N = 16 doubles all shifts'
+    // results instead, at orders above 4 alone: the branch in each of its four
+    // transforms costs 3 % (4.64 -> 4.78 ms).
+    static constexpr bool kTwice = N < 16;
     static constexpr uint32_t kCols = 64 * kTmemBlocks;  // tensor-memory columns of a warp
 };
 
@@ -148,7 +152,6 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
         // this warp's 32 lanes; warps w and w + 4 share them
         tmem = s_tmem + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * O::kCols;
     }
-    const double hfac = (double)(1ull << (2 * alpha));
     for (uint32_t n = 0;; ++n) {
         one_wait(smem_u32(&s_claim), n & 1, status, wait_ns);
         const long long g = s_tile[n & 1];
@@ -177,7 +180,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
         } else {
 #pragma unroll
             for (int tp = 0; tp < O::kBlocks; ++tp) {
-                w32_direct<0, 32>(v, pair_src(psi, N, x0, tp), tid);
+                w32_direct<0, 32, O::kTwice>(v, pair_src(psi, N, x0, tp), tid);
                 w32_block<kBlockBits, O::kHalfMove>(v, smem, tid);
                 if (tp + 1 < O::kBlocks) {
                     if (tp < O::kTmemBlocks) {
@@ -197,7 +200,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
                     case 2: s = one_blocks<N, 2>(v, tmem, park, tid, alpha); break;
                     case 3: s = one_blocks<N, 3>(v, tmem, park, tid, alpha); break;
                     case 4: s = one_blocks<N, 4>(v, tmem, park, tid, alpha); break;
-                    default: s = one_blocks<N, 0>(v, tmem, park, tid, alpha);
+                    default: s = one_blocks<N, O::kTwice ? 0 : -1>(v, tmem, park, tid, alpha);
                 }
             }
         }
@@ -214,7 +217,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
             constexpr int kWarps = 8 / O::kShifts;
             double t = 0.0;
             for (int w = 0; w < kWarps; ++w) t += red[kWarps * tid + w];
-            t *= hfac;
+            t *= fp32_scale(O::kTwice ? fp32_doubled(x0 + (uint64_t)tid) : alpha > 4, alpha);
             const uint64_t at = x0 - x_begin + (uint64_t)tid;
             part[(uint64_t)sidx * (x_end - x_begin) + at] = t;
             if (per_x) per_x[at] = t;

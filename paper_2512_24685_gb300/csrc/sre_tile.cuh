@@ -191,14 +191,22 @@ __device__ __forceinline__ cx_t<R> pair_value(v2_t<R> b, v2_t<R> a) {
         return Cx<fx>::from(make_double2(re, im));
 }
 
-// A sum of (Re W)^(2 alpha) + (Im W)^(2 alpha) over FP32 values, times 2^(2 alpha)
-// for the halving; over fixed-point values of unit exponent k, times the unit
-// 2^k to the same power as well (NaN for a state without a finite norm, whose
-// fixed-point values mean nothing).  The power alone may leave the range of a
-// double where its product with the sum does not.
-template <typename R>
-__device__ __forceinline__ double half_scale(double s, int alpha, int k) {
-    if constexpr (sizeof(cx_t<R>) == 8) return (double)(1ull << (2 * alpha)) * s;
+// FP32: shifts below 4096 run on doubled products, so that their transforms are
+// A, not W = A / 2.  The doubling is exact; the powers of W leave the range of
+// FP32 where those of A do not (order 14 at N = 12: all digits of a sum of
+// shifts).  From 4096 up, where states have twice the entries and more, it is W.
+__device__ __forceinline__ bool fp32_doubled(uint64_t x) { return x < 4096; }
+// Factor of an FP32 sum of powers: 1 for A, 2^(2 alpha) for W.
+__device__ __forceinline__ double fp32_scale(bool doubled, int alpha) {
+    return doubled ? 1.0 : (double)(1ull << (2 * alpha));
+}
+
+// A sum of (Re W)^(2 alpha) + (Im W)^(2 alpha) over fixed-point values of unit
+// exponent k, times 2^(2 alpha) for the halving and the unit 2^k to the same
+// power (NaN for a state without a finite norm, whose fixed-point values mean
+// nothing).  The power alone may leave the range of a double where its product
+// with the sum does not.
+__device__ __forceinline__ double fx_scale(double s, int alpha, int k) {
     if (k == kFxNonFinite) return __longlong_as_double(0x7ff8000000000000ll);
     return scalbn(s, 2 * alpha * (1 + k));
 }
@@ -245,7 +253,8 @@ template <> __device__ __forceinline__ int elem<1>(int tid, int i) {
 }
 template <> __device__ __forceinline__ int elem<2>(int tid, int i) { return (i << 8) | tid; }
 
-// Products of a block in round-2 layout (e = i << 8 | tid), any pivot.
+// Products of a block in round-2 layout (e = i << 8 | tid), any pivot; FP32 ones
+// doubled where the pivot lies inside the block (fp32_doubled).
 template <typename R, bool ZERO>
 __device__ __forceinline__ void block_values_z(cx_t<R> (&v)[16], const BlockPair<v2_t<R>> &s, int tid) {
     const int o = s.place(tid), w0 = s.place(256), w1 = s.place(512), w2 = s.place(1024), w3 = s.place(2048);
@@ -253,6 +262,7 @@ __device__ __forceinline__ void block_values_z(cx_t<R> (&v)[16], const BlockPair
     for (int i = 0; i < 16; ++i) {
         const int e = o + ((i & 1) ? w0 : 0) + ((i & 2) ? w1 : 0) + ((i & 4) ? w2 : 0) + ((i & 8) ? w3 : 0);
         v[i] = pair_value<R, ZERO>(__ldg(s.par + (e ^ s.xo)), __ldg(s.own + e));
+        if constexpr (sizeof(cx_t<R>) == 8) v[i] = Cx<R>::add(v[i], v[i]);
     }
 }
 

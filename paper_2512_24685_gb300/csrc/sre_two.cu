@@ -295,15 +295,14 @@ __device__ __noinline__ void two_publish(const TwoArgs &a, TwoDone *d) {
         // last item of the chunk: per-shift and chunk sums in fixed order
         fence_gpu();
         constexpr int kParts = TwoCols<H2>::kParts;
-        const double hfac = (double)(1ull << (2 * a.alpha));
         double cs = 0.0;
         for (int q = 0; q < (1 << S_log); ++q) {
             const double *ip = a.item_part + (((((size_t)d->t.slot << S_log) + q) << H2) * kParts);
             double sx = 0.0;
             for (int m = lane; m < (kParts << H2); m += 32) sx += __ldcg(ip + m);
-            sx = hfac * warp_sum(sx);
             const uint64_t x = d->xc + ((uint64_t)(q >> a.C_log) << two_item_spacing<SHARE>(a)) +
                                ((uint64_t)(q & (C - 1)) << two_spacing<SHARE>(a));
+            sx = fp32_scale(fp32_doubled(x), a.alpha) * warp_sum(sx);
             if (lane == 0 && a.per_x && x >= a.x_begin && x < a.x_end) a.per_x[x - a.x_begin] = sx;
             cs += sx;
         }

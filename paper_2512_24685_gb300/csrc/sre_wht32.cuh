@@ -157,13 +157,15 @@ __device__ __forceinline__ void w32_block(c64_t (&v)[32], unsigned char *buf, in
 struct PairSrc {
     const unsigned char *own, *par;
     uint32_t xo;
-    int pivot;  // kBlockBits: the pivot lies above the block
-    bool zero;  // x = 0
+    int pivot;   // kBlockBits: the pivot lies above the block
+    bool zero;   // x = 0
+    bool twice;  // fp32_doubled
 };
 
 __device__ __forceinline__ PairSrc pair_src(const float2 *psi, int N, uint64_t x, int tp) {
     PairSrc s;
     s.zero = x == 0;
+    s.twice = fp32_doubled(x);
     const uint64_t xe = s.zero ? 1ull << (N - 1) : x;  // x = 0 pairs the two halves
     const int j = 63 - __clzll((long long)xe);
     if (j >= kBlockBits) {
@@ -211,9 +213,15 @@ __device__ __forceinline__ float2 w32_zero_value(float2 a, float2 b) {
     return make_float2(0.5f * (g0 + g1), 0.5f * (g0 - g1));
 }
 
-// Products of the entries with register index [F, F + COUNT) (and the thread's
-// bits), by loads of both factors.
 template <int F, int COUNT>
+__device__ __forceinline__ void w32_double(c64_t (&v)[32]) {
+#pragma unroll
+    for (int i = F; i < F + COUNT; ++i) v[i] = Cx<float>::add(v[i], v[i]);
+}
+
+// Products of the entries with register index [F, F + COUNT) (and the thread's
+// bits), by loads of both factors, doubled where the shift asks for it (TWICE).
+template <int F, int COUNT, bool TWICE = true>
 __device__ __forceinline__ void w32_direct(c64_t (&v)[32], const PairSrc &s, int tid) {
     const int tau = (int)local_copy((uint32_t)tid);
     const uint32_t o = w32_place(s, w32_thr(tau));
@@ -235,6 +243,7 @@ __device__ __forceinline__ void w32_direct(c64_t (&v)[32], const PairSrc &s, int
             v[F + i] = conj_mul<float>(b.x, b.y, a.x, a.y);  // conj(phi_{t^x}) * phi_t
         }
     }
+    if (TWICE && s.twice) w32_double<F, COUNT>(v);
 }
 
 __device__ __forceinline__ void tmem_put4(uint32_t addr, const c64_t *v) {
@@ -247,8 +256,9 @@ __device__ __forceinline__ void tmem_put4(uint32_t addr, const c64_t *v) {
     tc_st8(addr, r);
 }
 
-// Load a shift's own and partner factors of one block into this thread's
-// tensor-memory columns (own entry i at columns 2i, partner at 64 + 2i).
+// Load the own and partner factors of one block, for a shift with the pivot above
+// it, into this thread's tensor-memory columns (own entry i at columns 2i, partner
+// at 64 + 2i).
 __device__ __forceinline__ void w32_fill(uint32_t tmem, const PairSrc &s, int tid) {
     const int tau = (int)local_copy((uint32_t)tid);
     const uint32_t o = w32_place(s, w32_thr(tau));
@@ -265,19 +275,11 @@ __device__ __forceinline__ void w32_fill(uint32_t tmem, const PairSrc &s, int ti
     c64_t a[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) a[i] = Cx<float>::from(__ldg(reinterpret_cast<const float2 *>(s.own + entry(i))));
-    if (s.zero) {
-        // x = 0: the value itself as own factor, partner 1
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            a[i] = Cx<float>::from(w32_zero_value(
-                Cx<float>::to(a[i]), __ldg(reinterpret_cast<const float2 *>(s.par + entry(i)))));
-    }
 #pragma unroll
     for (int i = 0; i < 32; i += 4) tmem_put4(tmem + 2 * i, a + i);
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-        a[i] = Cx<float>::from(s.zero ? make_float2(1.f, 0.f)
-                                      : __ldg(reinterpret_cast<const float2 *>(s.par + (entry(i) ^ s.xo))));
+        a[i] = Cx<float>::from(__ldg(reinterpret_cast<const float2 *>(s.par + (entry(i) ^ s.xo))));
 #pragma unroll
     for (int i = 0; i < 32; i += 4) tmem_put4(tmem + 64 + 2 * i, a + i);
     tc_wait_st();
@@ -306,9 +308,10 @@ __device__ __forceinline__ void w32_products(c64_t (&v)[32], uint32_t tmem, uint
 // ----------------------------------------------------------------- powers
 
 // acc + the 2 alpha-th powers of the real and imaginary parts of x, in FP32;
-// A = alpha, or 0 for an order known at run time only.
+// A = alpha, or 0 for an order known at run time only, -1 for one of 2 x.
 template <int A>
 __device__ __forceinline__ c64_t w32_acc(c64_t acc, c64_t x, int alpha) {
+    if constexpr (A < 0) x = Cx<float>::add(x, x);
     const c64_t sq = Cx<float>::mul(x, x);
     if constexpr (A == 2) return Cx<float>::fma(sq, sq, acc);
     c64_t p = sq;
