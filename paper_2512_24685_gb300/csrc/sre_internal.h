@@ -42,7 +42,6 @@ struct LargeCfg {
     int grid;    // persistent CTAs
     int stage1 = 1;  // pass 1 by bulk copy where available (C = 1, FP32, aligned)
     int stage2 = 1;  // pass 2 by TMA tile copies where available (FP32, h2 = 7 and 8)
-    bool two = false;  // FP32, N = 20: the library's choice is the kernel of sre_two.cu
 };
 
 // Everything one evaluation needs on the device (owned by a plan or a

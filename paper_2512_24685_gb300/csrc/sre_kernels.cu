@@ -388,21 +388,22 @@ static LargeCfg choose_tc_cfg(const DeviceInfo &dev, const Workspace &ws, int N)
 
 // FP32 at N = 20: one shift per chunk, block pairs and tiles by bulk and tensor
 // copies, eight blocks and eight tiles per item, and all the slots that the
-// tuning scratch holds (47 of 4 MB).  1.90 s for a whole state, against 1.97 s
-// by the item-list kernel of sre_two.cu.  A short ring makes this kernel wait (96 MB: 2.46 s): with less
-// scratch long ranges take the other one (2.36 s), and so does a handful of
-// shifts (one 76 against 84 us, 32 161 against 133 us).
+// tuning scratch holds (47 of 4 MB).  1.90 s for a whole state, against 1.98 s
+// by the item-list kernel of sre_two.cu.  A short ring makes it wait: a server's
+// slots (96 MB) take 2.46 s, 8192 shifts 19.1 ms in place of 14.9 (the item-list
+// kernel with that ring 2.36 s and 22.2 ms).  Below 23 slots the general rule.
+// Fewer than 16 shifts take smaller items, or most SMs have none (one shift 56
+// against 68 us, 16 shifts 90 in either).
 constexpr int kFp32LargeN = 20, kFp32Ring = 47;
 static LargeCfg choose_fp32_20_cfg(const DeviceInfo &dev, const Workspace &ws, uint64_t shifts) {
     LargeCfg c = choose_large_cfg(dev, kFp32LargeN, 8, 1);
     const int R = (int)std::min<size_t>(kFp32Ring, ws.scratch_bytes / ((size_t)8 << (kFp32LargeN - 1)));
-    if (shifts < 16 || (R < kFp32Ring && shifts >= 16384)) {
-        c.two = true;
-    } else if (R >= 23) {
+    if (R >= 23) {
         c.C_log = 0;
         c.R = R;
         c.D = (R - 1) / 2;
-        c.G2_log = c.B1_log = 3;
+        c.G2_log = shifts < 16 ? 2 : 3;
+        c.B1_log = shifts < 16 ? 0 : 3;
     }
     return c;
 }
@@ -424,10 +425,9 @@ LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_
     return choose_main_cfg(dev, ws, N, mode, shifts);
 }
 
-// FP32 shifts of N = 17..20 by sre_two.cu: N = 20 only where the library chose
-// it, and beside the tensor-core kernel.
-static bool takes_two(int N, int elem_bytes, int tc_kind, const LargeCfg &c) {
-    return two_applies(N, elem_bytes) && (N < kFp32LargeN || tc_kind || c.two);
+// FP32 shifts by sre_two.cu: at N = 20 only beside the tensor-core kernel.
+static bool takes_two(int N, int elem_bytes, int tc_kind) {
+    return two_applies(N, elem_bytes) && (N < kFp32LargeN || tc_kind);
 }
 
 size_t workspace_scratch_bytes(const DeviceInfo &dev, int N_max, int elem_bytes, sre_mode_t mode) {
@@ -770,7 +770,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                 else
                     e = launch_one(N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, d_per_x, ws.work + 2,
                                    ws.status, wait_ns, dev, st);
-            } else if (takes_two(N, eb, tc_kind, main)) {
+            } else if (takes_two(N, eb, tc_kind)) {
                 name = "k_two";
                 const LargeCfg c = choose_two_cfg(dev, ws, N);
                 e = launch_two(ws, c, N, psi, nullptr, 1, x_begin, split, alpha, ws.chunk_sum, ws.counters,
@@ -963,7 +963,7 @@ BatchClass batch_class_layout(const DeviceInfo &dev, const Workspace &ws, int N,
         return L;
     }
     const LargeCfg main = tuned_half ? *tuned_half : choose_main_cfg(dev, ws, N, mode, 1ull << N);
-    L.two = takes_two(N, eb, tc_kind, main);
+    L.two = takes_two(N, eb, tc_kind);
     if (one_applies(N, eb)) {
         // one partial per shift, all shifts or those below 4096 beside the
         // tensor-core kernel

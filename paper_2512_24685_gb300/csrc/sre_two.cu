@@ -1,6 +1,6 @@
 // sre_two.cu -- FP32 two-pass kernel for 17 <= N <= 19, all shifts in the
 // halved form (sre_wht32.cuh); at N = 20 for the shifts below 4096 beside the
-// tensor-core kernel, a handful of shifts, and slots with a short ring.
+// tensor-core kernel.
 //
 // Pass 1 (one item: a block of 8192 entries for the 2^C_log shifts that share
 // its factors) forms the products, transforms the 13 block bits and writes

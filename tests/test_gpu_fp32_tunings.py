@@ -59,3 +59,21 @@ def test_twenty_qubits_take_the_tuned_kernel(sre):
         library = ms(p)
         p.set_tuning(0, 47, 23, 3, 3, 1, 1)
         assert ms(p) <= 1.1 * library
+
+
+def test_twenty_qubits_alike_for_every_range_and_server(sre):
+    """N = 20: a shift's sum does not depend on the length of its range, nor M2 on
+    whether a plan or a server with a shorter ring forms it (range sums add the
+    same doubles in another order: n 2^-52)."""
+    import numpy as np
+    import torch
+    host = W.haar_state(20, 29, np.complex64)
+    psi = torch.from_numpy(host).cuda()
+    with sre.Plan(20, "c64") as p:
+        _, px = p.sum4_range(psi, 4090, 4090 + 200, per_x=True)
+        for a, n in ((4090, 1), (4095, 3), (4200, 15), (4100, 64)):
+            _, py = p.sum4_range(psi, a, a + n, per_x=True)
+            assert torch.allclose(px[a - 4090:a - 4090 + n], py, rtol=2.0 ** -48, atol=0)
+        want = p.m2(psi)
+    with sre.Server(max_inflight=1, max_N=20) as srv:
+        assert abs(srv.wait(srv.submit(host), 120000) - want) <= 2.0 ** (20 - 52)
