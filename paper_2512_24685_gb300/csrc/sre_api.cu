@@ -248,7 +248,7 @@ static sre_status_t enqueue_plan(sre_plan_t p, const void *d_state, int N, uint6
     sre::LargeCfg *cp = nullptr;
     if (N > sre::kTileBits) {
         c = plan_cfg(p, N, xe - xb);
-        if (!sre::large_cfg_fits(p->ws, c, N, 1)) return SRE_EINVAL;
+        if (!sre::large_cfg_fits(p->ws, c, N)) return SRE_EINVAL;
         cp = &c;
     }
     return enqueue_plan_cfg(p, d_state, N, xb, xe, st, d_m2, d_per_x, cp, alpha);
@@ -319,7 +319,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
     // the tensor-core kernel runs one CTA per SM and always stages its
     // copies, so its lag steps are counted over the SMs, its lag is tried at
     // every step count, and the copy-path fields are not varied
-    const bool tc = sre::tc_mode_available(p->mode) && sre::tc_applies(N, 1, 2, p->tune_state);
+    const bool tc = sre::tc_mode_available(p->mode) && sre::tc_applies(N, 2, p->tune_state);
     const int grid_eff = tc ? std::min(base.grid, p->dev.sms) : base.grid;
     std::vector<sre::LargeCfg> cands;
     auto add = [&](const sre::LargeCfg &c) {
@@ -327,7 +327,7 @@ sre_status_t sre_plan_autotune(sre_plan_t p, int N, sre_stream_t stream, sre_tun
             if (o.C_log == c.C_log && o.G2_log == c.G2_log && o.B1_log == c.B1_log && o.D == c.D &&
                 o.R == c.R && o.stage1 == c.stage1 && o.stage2 == c.stage2)
                 return;
-        if (sre::large_cfg_fits(p->ws, c, N, 1)) cands.push_back(c);
+        if (sre::large_cfg_fits(p->ws, c, N)) cands.push_back(c);
     };
     // FP32 kernels that take no tuning (sre_one.cu, sre_two.cu): the time alone
     const bool fixed = p->mode == SRE_MODE_FP32 && (sre::one_applies(N, eb) || (sre::two_applies(N, eb) && N < 20));

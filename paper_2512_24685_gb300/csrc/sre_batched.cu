@@ -169,7 +169,7 @@ cudaError_t batched_run(BatchedContext *ctx, const Workspace &ws, const DeviceIn
         // (16 <= N <= 20) and whose states are all 16-byte aligned takes it
         // (converted copies are aligned)
         int tc_kind = 0;
-        if (tc_mode_available(mode) && N > kTileBits && tc_applies(N, 1, 2, nullptr)) {
+        if (tc_mode_available(mode) && N > kTileBits && tc_applies(N, 2, nullptr)) {
             bool aligned = true;
             for (int q = k; q < j; ++q) aligned &= dtype != SRE_C64 || ((uintptr_t)d_states[order[q]] & 15) == 0;
             if (aligned) tc_kind = mode == SRE_MODE_BF16_SPLIT ? 1 : 2;

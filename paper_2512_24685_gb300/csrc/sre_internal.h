@@ -13,7 +13,6 @@ constexpr int kTile = 1 << kTileBits;
 constexpr int kThreads = 256;              // threads per tile CTA
 constexpr int kPerThread = kTile / kThreads;  // 16 entries per thread (4 register bits)
 constexpr int kNormBlocks = 264;           // fixed grid of the norm reduction
-constexpr int kFinalThreads = 256;
 constexpr size_t kWorkBytes = 1024;               // work-queue counters of a workspace
 constexpr size_t kFlagBytes = 16;                 // flags, status, ticket: behind the counters
 constexpr int kMaxRing = 64;                      // ring slots a tuned configuration may use
@@ -86,9 +85,8 @@ struct DeviceInfo {
 
 cudaError_t query_device(DeviceInfo *info);
 
-// The L2-sized two-pass configuration for N > 12 (half: transforms of 2^(N-1)
-// entries).
-LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half);
+// The L2-sized two-pass configuration for N > 12.
+LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes);
 
 // The library's two-pass configuration for a number of shifts in an arithmetic
 // mode (in the split modes those from 4096).
@@ -100,11 +98,11 @@ LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_
 
 // Tensor-core two-pass kernel (sre_tc.cu) for the halved shifts of one
 // state: tc_kind 1 = BF16 hi/lo pieces, 2 = FP16 hi/lo pieces.  tc_applies
-// says whether it covers (N, half, Renyi order, state alignment); the launch
+// says whether it covers (N, Renyi order, state alignment); the launch
 // first computes the per-shift fixed-point scales of the state into
 // ws.tc_bn / ws.tc_e.
 struct LargeArgs;
-bool tc_applies(int N, int half, int alpha, const void *psi);
+bool tc_applies(int N, int alpha, const void *psi);
 // Tensor-core launch of the halved shifts of one state (a.psi) or of the
 // states of a batch class (a.psis, a.chunks_per_state); the per-state scale
 // tables go to e_buf / bn_buf (buf_cap entries) when given, else to ws.
@@ -113,13 +111,10 @@ cudaError_t launch_large_tc(const LargeArgs &a, const Workspace &ws, const Devic
                             size_t buf_cap = 0);
 
 // Does a (possibly tuned) configuration fit the workspace allocation?
-bool large_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, int half);
+bool large_cfg_fits(const Workspace &ws, const LargeCfg &c, int N);
 
 // Fill a state buffer with deterministic pseudo-random amplitudes (timing).
 cudaError_t enqueue_fill_synthetic(void *buf, int N, sre_dtype_t dtype, cudaStream_t st);
-
-// Bytes of workspace needed for states up to N_max with element size.
-size_t workspace_scratch_bytes(const DeviceInfo &dev, int N_max, int elem_bytes, sre_mode_t mode);
 
 cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int elem_bytes,
                             sre_mode_t mode, size_t scratch_floor = kTuneScratch);

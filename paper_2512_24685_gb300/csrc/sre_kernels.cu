@@ -324,11 +324,11 @@ cudaError_t enqueue_fill_synthetic(void *buf, int N, sre_dtype_t dtype, cudaStre
     return cudaGetLastError();
 }
 
-bool large_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, int half) {
+bool large_cfg_fits(const Workspace &ws, const LargeCfg &c, int N) {
     if (c.C_log < 0 || c.C_log > 3 || c.R < 2 || c.R > kMaxRing || c.D < 1 || c.D >= c.R) return false;
-    const int h2 = N - kTileBits - half;
+    const int h2 = N - kTileBits - 1;
     if (c.G2_log < 0 || c.G2_log > h2 || c.B1_log < 0 || c.B1_log > h2) return false;
-    const size_t ring = (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)ws.elem_bytes << (N - half));
+    const size_t ring = (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)ws.elem_bytes << (N - 1));
     const size_t P2 = ((size_t)1 << c.C_log) << (h2 - c.G2_log);
     return ring <= ws.scratch_bytes && (size_t)c.R * P2 * 8 <= ws.item_part_cap;
 }
@@ -338,12 +338,12 @@ bool large_cfg_fits(const Workspace &ws, const LargeCfg &c, int N, int half) {
 // lags D = that + 1 chunks behind and the ring holds R = 2 D + 1 chunks:
 // pass-2 items then find their chunk finished and pass-1 items find their
 // slot free.  The chunk size C (shifts sharing one pass-1 partner block) is
-// the largest power of two up to 8 whose ring R * C * elem * 2^(N - half)
+// the largest power of two up to 8 whose ring R * C * elem * 2^(N - 1)
 // stays within 60% of L2, so the inter-pass traffic stays on chip.
-LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half) {
+LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes) {
     LargeCfg c;
-    const int h2 = N - kTileBits - half;
-    const double per_x = (double)elem_bytes * (double)(1ull << (N - half));
+    const int h2 = N - kTileBits - 1;
+    const double per_x = (double)elem_bytes * (double)(1ull << (N - 1));
     const double budget = std::max(24.0 * (1 << 20), 0.6 * (double)dev.l2_bytes);
     c.grid = std::max(1, dev.sms * 2);
     const int P1 = 1 << h2;
@@ -372,7 +372,7 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes, int half
 // 19 18.6 -> 12.7, 20 18.4 -> 13.1.  Six slots at least: a workspace with less
 // scratch takes fewer shifts per chunk, and below that the general rule.
 static LargeCfg choose_tc_cfg(const DeviceInfo &dev, const Workspace &ws, int N) {
-    LargeCfg c = choose_large_cfg(dev, N, 8, 1);
+    LargeCfg c = choose_large_cfg(dev, N, 8);
     const size_t ring = std::min(ws.scratch_bytes, kTuneScratch);
     for (int C_log = 3; C_log >= 0; --C_log) {
         const int R = (int)std::min<size_t>(kMaxRing - 1, ring / ((size_t)8 << (N - 1 + C_log)));
@@ -396,7 +396,7 @@ static LargeCfg choose_tc_cfg(const DeviceInfo &dev, const Workspace &ws, int N)
 // against 68 us, 16 shifts 90 in either).
 constexpr int kFp32LargeN = 20, kFp32Ring = 47;
 static LargeCfg choose_fp32_20_cfg(const DeviceInfo &dev, const Workspace &ws, uint64_t shifts) {
-    LargeCfg c = choose_large_cfg(dev, kFp32LargeN, 8, 1);
+    LargeCfg c = choose_large_cfg(dev, kFp32LargeN, 8);
     const int R = (int)std::min<size_t>(kFp32Ring, ws.scratch_bytes / ((size_t)8 << (kFp32LargeN - 1)));
     if (R >= 23) {
         c.C_log = 0;
@@ -414,31 +414,20 @@ LargeCfg choose_main_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_
     // fewer than 64 shifts leave most SMs without an item of the large chunks:
     // one shift of N = 18 takes 87 us in small ones, 108 in large ones; 48 shifts
     // 105 and 121, 128 shifts 154 and 144
-    if (tc_mode_available(mode) && tc_applies(N, 1, 2, nullptr) && shifts >= 64) return choose_tc_cfg(dev, ws, N);
-    return choose_large_cfg(dev, N, eb, 1);
+    if (tc_mode_available(mode) && tc_applies(N, 2, nullptr) && shifts >= 64) return choose_tc_cfg(dev, ws, N);
+    return choose_large_cfg(dev, N, eb);
 }
 
 LargeCfg tuning_base_cfg(const DeviceInfo &dev, const Workspace &ws, int N, sre_mode_t mode, const sre_tuning_t &t,
                          uint64_t shifts) {
     if (t.x_batch_log >= 0 || t.ring_slots >= 0 || t.lag >= 0)
-        return choose_large_cfg(dev, N, mode == SRE_MODE_FP64 ? 16 : 8, 1);
+        return choose_large_cfg(dev, N, mode == SRE_MODE_FP64 ? 16 : 8);
     return choose_main_cfg(dev, ws, N, mode, shifts);
 }
 
 // FP32 shifts by sre_two.cu: at N = 20 only beside the tensor-core kernel.
 static bool takes_two(int N, int elem_bytes, int tc_kind) {
     return two_applies(N, elem_bytes) && (N < kFp32LargeN || tc_kind);
-}
-
-size_t workspace_scratch_bytes(const DeviceInfo &dev, int N_max, int elem_bytes, sre_mode_t mode) {
-    (void)mode;
-    if (N_max <= kTileBits) return 0;
-    size_t b = 0;
-    for (int half = 0; half <= 1; ++half) {
-        const LargeCfg c = choose_large_cfg(dev, N_max, elem_bytes, half);
-        b = std::max(b, (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)elem_bytes << (N_max - half)));
-    }
-    return b;
 }
 
 void workspace_free(Workspace *ws) {
@@ -482,20 +471,16 @@ cudaError_t workspace_alloc(Workspace *ws, const DeviceInfo &dev, int N_max, int
     ws->status = ws->flags + 1;
     SRE_TRY(cudaMalloc(&ws->result, sizeof(Result)));
     if (N_max > kTileBits) {
-        // sizes for every N up to N_max and both halves of the shift range,
-        // with room for tuned configurations: chunks of a single shift, up to
+        // sizes for every N up to N_max, and with the ring of one qubit more
+        // room for tuned configurations: chunks of a single shift, up to
         // kMaxRing ring slots, a scratch ring of at least scratch_floor bytes
-        size_t scratch = scratch_floor, item_cap = 0, chunk_cap = 0;
-        for (int n = kTileBits + 1; n <= N_max; ++n) {
-            for (int half = 0; half <= 1; ++half) {
-                const LargeCfg c = choose_large_cfg(dev, n, elem_bytes, half);
-                const int h2 = n - kTileBits - half;
-                scratch = std::max(scratch, (size_t)c.R * ((size_t)1 << c.C_log) *
-                                                ((size_t)elem_bytes << (n - half)));
-                // R * P2 per-warp partials (8 warps, P2 <= 8 * 2^h2)
-                item_cap = std::max(item_cap, (size_t)std::max(c.R, kMaxRing) * ((size_t)8 << h2) * 8);
-            }
-            chunk_cap = std::max(chunk_cap, ((size_t)1 << n) + 4);
+        size_t scratch = scratch_floor, item_cap = 0;
+        const size_t chunk_cap = ((size_t)1 << N_max) + 4;
+        for (int n = kTileBits + 1; n <= N_max + 1; ++n) {
+            const LargeCfg c = choose_large_cfg(dev, n, elem_bytes);
+            scratch = std::max(scratch, (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)elem_bytes << (n - 1)));
+            // R * P2 per-warp partials (8 warps, P2 <= 8 * 2^h2)
+            item_cap = std::max(item_cap, (size_t)std::max(c.R, kMaxRing) * ((size_t)8 << (n - kTileBits - 1)) * 8);
         }
         ws->scratch_bytes = scratch;
         ws->item_part_cap = item_cap;
@@ -631,9 +616,9 @@ static cudaError_t launch_large(const LargeArgs &a, int grid, cudaStream_t st) {
     return cudaErrorInvalidValue;
 }
 
-// Fill LargeArgs for the shift range [xb, xe) (all of it halved or not).
+// Fill LargeArgs for the shift range [xb, xe).
 static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const DeviceInfo &dev,
-                                   const void *psi, int N, uint64_t xb, uint64_t xe, int half,
+                                   const void *psi, int N, uint64_t xb, uint64_t xe,
                                    int elem_bytes, size_t chunk_off, double *per_x,
                                    long long wait_ns, const LargeCfg &c, int *grid) {
     LargeArgs &A = *a;
@@ -644,8 +629,7 @@ static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const Devi
     A.fx_cap = ws.fx_cap;
     A.tc_e = ws.tc_e;
     A.N = N;
-    A.half = half;
-    A.h2 = N - kTileBits - half;
+    A.h2 = N - kTileBits - 1;
     A.x_begin = xb;
     A.x_end = xe;
     A.C_log = c.C_log;
@@ -662,7 +646,7 @@ static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const Devi
     A.P1 = 1 << (A.h2 - A.B1_log);
     A.P2 = (1 << c.C_log) << (A.h2 - A.G2_log);
     A.n_items = A.n_chunks * (long long)(A.P1 + A.P2);
-    const size_t need_scratch = (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)elem_bytes << (N - half));
+    const size_t need_scratch = (size_t)c.R * ((size_t)1 << c.C_log) * ((size_t)elem_bytes << (N - 1));
     if (need_scratch > ws.scratch_bytes || chunk_off + (size_t)A.n_chunks > ws.chunk_cap ||
         (size_t)c.R * A.P2 * 8 > ws.item_part_cap ||
         (elem_bytes == 16 && (size_t)c.R << (c.C_log + A.h2) > ws.fx_cap))
@@ -673,7 +657,7 @@ static cudaError_t make_large_args(LargeArgs *a, const Workspace &ws, const Devi
     A.done1 = ws.counters + chunk_off;
     A.done2 = ws.counters + ws.chunk_cap + chunk_off;
     A.freed = ws.counters + 2 * ws.chunk_cap + chunk_off;
-    A.work = ws.work + (half ? 1 : 0);
+    A.work = ws.work + 1;
     A.per_x = per_x;
     A.status = ws.status;
     A.wait_ns = wait_ns;
@@ -746,7 +730,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         const int eb = (int)sizeof(v2_t<R>);
         // every shift in one launch, or with the tensor-core kernel on the
         // shifts from 4096 up those below it
-        const bool tc = tc_kind && tc_applies(N, 1, alpha, psi);
+        const bool tc = tc_kind && tc_applies(N, alpha, psi);
         const uint64_t split = tc ? std::min<uint64_t>(std::max<uint64_t>(x_begin, kTile), x_end) : x_end;
         const bool single_pass = one_applies(N, eb) || mid_applies(N, eb);
         const sre_mode_t mode = kFx ? SRE_MODE_FP64 : tc_kind ? SRE_MODE_FP16_SPLIT : SRE_MODE_FP32;
@@ -780,7 +764,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
                 name = "k_large";
                 LargeArgs a;
                 int grid = 0;
-                if ((e = make_large_args(&a, ws, dev, psi, N, x_begin, split, 1, eb, 0, d_per_x, wait_ns,
+                if ((e = make_large_args(&a, ws, dev, psi, N, x_begin, split, eb, 0, d_per_x, wait_ns,
                                          main, &grid)) != cudaSuccess)
                     return e;
                 a.alpha = alpha;
@@ -796,7 +780,7 @@ static cudaError_t enqueue_m2_t(const Workspace &ws, const DeviceInfo &dev, cons
         if (tc && split < x_end) {
             LargeArgs a;
             int grid = 0;
-            if ((e = make_large_args(&a, ws, dev, psi, N, split, x_end, 1, eb, chunks,
+            if ((e = make_large_args(&a, ws, dev, psi, N, split, x_end, eb, chunks,
                                      d_per_x ? d_per_x + (split - x_begin) : nullptr, wait_ns, main,
                                      &grid)) != cudaSuccess)
                 return e;
@@ -1053,7 +1037,7 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
                 continue;
             }
         }
-        if (!large_cfg_fits(ws, c, N, half)) return cudaErrorInvalidValue;
+        if (!large_cfg_fits(ws, c, N)) return cudaErrorInvalidValue;
         LargeArgs A;
         A.psi = nullptr;
         A.psis = d_ptrs;
@@ -1062,8 +1046,7 @@ static cudaError_t enqueue_batch_class_t(const Workspace &ws, const DeviceInfo &
         A.tc_e = tc_e;
         A.chunks_per_state = cps;
         A.N = N;
-        A.half = half;
-        A.h2 = N - kTileBits - half;
+        A.h2 = N - kTileBits - 1;
         A.x_begin = xb;
         A.x_end = xe;
         A.x0 = xb;  // kTile and 0 are chunk-aligned

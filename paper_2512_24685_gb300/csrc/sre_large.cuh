@@ -63,7 +63,6 @@ struct LargeArgs {
     const void *const *psis;   // or: states of one batch class (device array)
     long long chunks_per_state;  // chunks of each state (batch class)
     int N, h2;                 // h2: pass-2 transform bits (N - 12, or N - 13 halved)
-    int half;
     uint64_t x_begin, x_end;   // evaluated shift range
     uint64_t x0;               // x_begin rounded down to a chunk boundary
     int C_log, R, D, G2_log, B1_log;
@@ -72,7 +71,7 @@ struct LargeArgs {
     long long n_chunks;
     int P1, P2;                // items per chunk in pass 1 / pass 2
     long long n_items;
-    void *scratch;             // R * C * 2^(N - half) complex
+    void *scratch;             // R * C * 2^(N - 1) complex
     double *item_part;         // R * P2
     double *chunk_sum;         // n_chunks
     unsigned *done1, *done2, *freed;  // n_chunks each

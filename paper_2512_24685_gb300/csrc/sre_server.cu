@@ -402,7 +402,7 @@ sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t)
     c.B1_log = std::min(c.B1_log, N - sre::kTileBits - 1);
     // a plan's library configuration whose ring the slots' smaller scratch does
     // not hold stands for the slots' own; whatever fits is taken as it is
-    if (!sre::large_cfg_fits(s->slots[0].ws, c, N, 1)) {
+    if (!sre::large_cfg_fits(s->slots[0].ws, c, N)) {
         sre::Workspace plan_ws;
         plan_ws.scratch_bytes = sre::kTuneScratch;
         const sre::LargeCfg lib = sre::choose_main_cfg(s->dev, plan_ws, N, s->cfg.mode, 1ull << N);
@@ -412,7 +412,7 @@ sre_status_t sre_server_set_tuning(sre_server_t s, int N, const sre_tuning_t *t)
     }
     std::lock_guard<std::mutex> lk(s->mu);
     for (const Slot &sl : s->slots)
-        if (!sre::large_cfg_fits(sl.ws, c, N, 1)) return SRE_EINVAL;
+        if (!sre::large_cfg_fits(sl.ws, c, N)) return SRE_EINVAL;
     s->tuned[N] = c;
     s->has_tuned[N] = true;
     return SRE_OK;

@@ -1,5 +1,6 @@
 // sre_stage.cuh -- pass-2 tiles of the two-pass kernel staged through the
-// Tensor Memory Accelerator (FP32, 5 <= H2 <= 8).
+// Tensor Memory Accelerator (FP32; for 5 <= H2 <= 8, used with H2 = 7 and 8, the
+// sizes N = 20 and 21).
 //
 // A pass-2 tile of one shift is the 2^H2 x 2^(12 - H2) block of inter-pass
 // scratch formed by rows t'_h (the H2 transform bits still to do, one row per

@@ -880,14 +880,14 @@ cudaError_t launch_tc(const LargeArgs &a, int grid, cudaStream_t st) {
 
 }  // namespace
 
-bool tc_applies(int N, int half, int alpha, const void *psi) {
+bool tc_applies(int N, int alpha, const void *psi) {
     const int h2 = N - kTileBits - 1;
-    return half && alpha == 2 && h2 >= kTcMinH2 && h2 <= kTcMaxH2 && ((uintptr_t)psi & 15) == 0;
+    return alpha == 2 && h2 >= kTcMinH2 && h2 <= kTcMaxH2 && ((uintptr_t)psi & 15) == 0;
 }
 
 cudaError_t launch_large_tc(const LargeArgs &a, const Workspace &ws, const DeviceInfo &dev, int grid,
                             cudaStream_t st, int tc_kind, int *e_buf, double *bn_buf, size_t buf_cap) {
-    if (!a.half || a.alpha != 2) return cudaErrorInvalidValue;
+    if (a.alpha != 2) return cudaErrorInvalidValue;
     const int nb = 1 << (a.N - kTileBits);
     // states of the launch: one, or the states of a batch class
     const long long S = a.psis ? a.n_chunks / a.chunks_per_state : 1;
