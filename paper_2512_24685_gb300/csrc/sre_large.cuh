@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_large(const __grid_constant__ L
                             u = fx_units<H2>(ex, ex + a.fx_cap);
                             fxk = u.k[2];
                         }
-                        align(v, u.k[0]);
+                        align(v, u);
                         fx_rows<H2>(v, bufB, tid, u);
                         acc += sum_order<R>(v, a.alpha);
                     } else {

@@ -53,16 +53,23 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 2 : 1)
         double s = 0.0;
         int k = u[0].c;
         if constexpr (NB == 2) {
-            k = fx_units<1>(max(u[0].c, u[1].c), max(u[0].s, u[1].s) + 1).k[2];
+            k = fx_units<1>(0, max(u[0].c, u[1].c), max(u[0].s, u[1].s) + 1).k[2];
+            const int q0 = k - u[0].c, q1 = k - u[1].c;
             cx_t<fx> w[16];
+            auto join = [&](auto shift) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const cx_t<fx> p = Cx<fx>::from(park[(i << 8) | tid]);
-                const cx_t<fx> a = make_longlong2(fx_shift(p.x, k - u[0].c), fx_shift(p.y, k - u[0].c));
-                const cx_t<fx> b = make_longlong2(fx_shift(v[i].x, k - u[1].c), fx_shift(v[i].y, k - u[1].c));
-                w[i] = Cx<fx>::sub(a, b);
-                v[i] = Cx<fx>::add(a, b);
-            }
+                for (int i = 0; i < 16; ++i) {
+                    const cx_t<fx> p = Cx<fx>::from(park[(i << 8) | tid]);
+                    const cx_t<fx> a = make_longlong2(shift(p.x, q0), shift(p.y, q0));
+                    const cx_t<fx> b = make_longlong2(shift(v[i].x, q1), shift(v[i].y, q1));
+                    w[i] = Cx<fx>::sub(a, b);
+                    v[i] = Cx<fx>::add(a, b);
+                }
+            };
+            if (max(q0, q1) <= 8)
+                join([](long long a, int q) { return fx_shift_few(a, q); });
+            else
+                join([](long long a, int q) { return fx_shift(a, q); });
             s = sum_order<fx>(w, alpha);
         }
         s += sum_order<fx>(v, alpha);

@@ -33,14 +33,13 @@
 // not meet: for a state close to a basis state a shift of high weight lost all
 // its digits.)  Above the tile each block carries its own unit and bound into
 // the transform over the blocks (FxExp).  Per-shift sums against 80-bit
-// arithmetic, N = 8..20, Haar, product, near-basis, stabilizer and decaying
-// states: at most 8e-16 from the exact ones, FP64 butterflies at most 1.1e-15,
-// the same or smaller on average for each kind of state.  The reason for fixed
+// arithmetic, N = 6..16, Haar, product, near-basis, stabilizer and decaying
+// states: at most 7e-16 off, as with FP64 butterflies.  The reason for fixed
 // point is the pipe: GB300 runs 2 FP64 operations per clock and SM, against some
 // 40 64-bit integer additions.  FP64 operations are left for the product (4 per
 // entry) and the powers (4 per entry); both conversions are integer code, since
 // F2I and I2F run at the FP64 rate too, and so are the bounds.  Measured: all
-// shifts of an N = 16 state 47.4 ms (FP64 butterflies, full transforms below x =
+// shifts of an N = 16 state 47.5 ms (FP64 butterflies, full transforms below x =
 // 4096: 178 ms; units from the factors' norms, known before the products: 46.0
 // ms), 60 states of N = 12 11.3 ms with their evolution (61.9 ms; 10.5 ms); the
 // FP64 pipe is busy 62 to 71 % of the time, and waits while the products of a
@@ -141,9 +140,9 @@ __host__ __device__ __forceinline__ long long fx_shift(long long a, int q) {
     const long long t = a >> (q - 1);
     return (t >> 1) + (t & 1);
 }
-// The same for 0 < q <= 8 and |a| <= 2^63 - 2^10, which all partial sums of a
+// The same for 0 <= q <= 8 and |a| <= 2^63 - 2^10, which all partial sums of a
 // tile keep (a product has 53 bits).
-__host__ __device__ __forceinline__ long long fx_shift_few(long long a, int q) { return (a + (1ll << (q - 1))) >> q; }
+__host__ __device__ __forceinline__ long long fx_shift_few(long long a, int q) { return (a + ((1ll << q) >> 1)) >> q; }
 
 // round(p 2^(63 - k)), |p| < 2^k; the magnitude's high word, `down` places down,
 // is added to sum.  The mantissa, 10 bits up, moves right by what its exponent
@@ -420,18 +419,20 @@ __device__ __forceinline__ FxExp fx_tile(cx_t<fx> (&v)[16], double2 *buf, int ti
 }
 
 // Units of the transform over a shift's 2^H2 blocks: k[0] for its first four
-// bits, k[1] and k[2] for the next ones; the last also for its results.
+// bits, k[1] and k[2] for the next ones; the last also for its results.  low: the
+// smallest of the blocks' own.
 template <int H2>
 struct FxUnits {
     static constexpr int G0 = H2 < 4 ? H2 : 4, G1 = H2 < 4 ? 0 : H2 < 8 ? H2 - 4 : 4, G2 = H2 < 8 ? 0 : H2 - 8;
-    int k[3];
+    int k[3], low;
 };
 
-// From the largest unit cm of the blocks and a bound 2^s of their sum.
+// From the smallest and largest unit of the blocks and a bound 2^s of their sum.
 template <int H2>
-__device__ __forceinline__ FxUnits<H2> fx_units(int cm, int s) {
+__device__ __forceinline__ FxUnits<H2> fx_units(int low, int cm, int s) {
     using U = FxUnits<H2>;
     U u;
+    u.low = low;
     u.k[0] = min(max(s, cm), cm + U::G0);
     u.k[1] = min(max(s, u.k[0]), u.k[0] + U::G1);
     u.k[2] = min(max(s, u.k[1]), u.k[1] + U::G2);
@@ -445,19 +446,22 @@ template <int H2>
 __device__ __forceinline__ FxUnits<H2> fx_units(const short *c, const short *s) {
     constexpr int n = 1 << H2;
     const int lane = threadIdx.x & 31;
-    int cm = -0x8000, sm = -0x8000;
+    int low = kFxNonFinite, cm = -0x8000, sm = -0x8000;
 #pragma unroll 1
     for (int t = lane; t < n; t += 32) {
-        cm = max(cm, (int)__ldcg(c + t));
+        const int ct = __ldcg(c + t);
+        low = min(low, ct);
+        cm = max(cm, ct);
         sm = max(sm, (int)__ldcg(s + t));
     }
+    low = __reduce_min_sync(0xffffffffu, low);
     cm = __reduce_max_sync(0xffffffffu, cm);
     sm = __reduce_max_sync(0xffffffffu, sm);
     unsigned sum = 0;
 #pragma unroll 1
     for (int t = lane; t < n; t += 32) sum += (1u << 20) >> min(sm - (int)__ldcg(s + t), 20);
     sum = __reduce_add_sync(0xffffffffu, sum);
-    return fx_units<H2>(cm, sm - 20 + 32 - __clz(sum - 1));
+    return fx_units<H2>(low, cm, sm - 20 + 32 - __clz(sum - 1));
 }
 
 // This thread's entries (round-0 layout, block = entry index mod 2^H2) from
@@ -476,7 +480,18 @@ struct FxAlign {
                 *reinterpret_cast<int4 *>(q + j) = __ldcg(reinterpret_cast<const int4 *>(p + j));
         }
     }
-    __device__ __forceinline__ void operator()(cx_t<fx> (&v)[16], int k) const {
+    __device__ __forceinline__ void operator()(cx_t<fx> (&v)[16], const FxUnits<H2> &u) const {
+        const int k = u.k[0];
+        // all but strongly decaying states (below four bits the units are uniform,
+        // and two paths only cost registers)
+        if (H2 >= 4 && k - u.low <= 8) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int d = k - q[i & (n - 1)];
+                v[i] = make_longlong2(fx_shift_few(v[i].x, d), fx_shift_few(v[i].y, d));
+            }
+            return;
+        }
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int d = k - q[i & (n - 1)];

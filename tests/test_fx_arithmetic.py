@@ -49,5 +49,5 @@ def test_shift_rounds_half_up_over_the_whole_range(shifted):
 
 def test_short_shift_rounds_alike_below_the_top(shifted):
     top = (1 << 63) - (1 << 10)
-    pairs = [(s * v, q) for s in (1, -1) for v in (0, 1, 7, 128, 99991, 1 << 50, top - 1, top) for q in range(1, 9)]
+    pairs = [(s * v, q) for s in (1, -1) for v in (0, 1, 7, 128, 99991, 1 << 50, top - 1, top) for q in range(0, 9)]
     assert shifted(pairs, 1) == shifted(pairs)
