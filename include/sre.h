@@ -75,7 +75,8 @@ typedef enum {
  * |A|^4; the cross-shift accumulation, the norm and the final log are FP64
  * in every mode.  The split modes apply to complex64 states and take the
  * halved shifts (x >= 4096) of 16-byte aligned states with 16 <= N <= 20
- * (other sizes run wholly in FP32) through two
+ * (other sizes run wholly in FP32; at N = 16 the FP32 mode is twice as fast
+ * as these and more exact, at N = 17 as fast) through two
  * tensor-core Hadamard stages of 128 x 128: each operand is scaled by a
  * power of two and split into an integer high piece (|hi| <= 2^8 for bf16,
  * 2^11 for fp16) and the remainder rounded to the 16-bit type as the low
@@ -83,8 +84,9 @@ typedef enum {
  * the FP32 accumulator and the low piece adds the next 8 (bf16) or 11
  * (fp16) significant bits; the remaining shifts run in FP32.  The FP64 mode
  * forms products and powers in FP64 and runs the butterflies between them in
- * 64-bit fixed point, on units that bound the whole transform (no rounding in
- * a butterfly but the rescaling between groups of stages).  Value 3 is unused
+ * 64-bit fixed point, on units that bound the next stages (no rounding in a
+ * butterfly but the rescaling between groups of stages); its sums, those of
+ * single shifts too, are as exact as with FP64 butterflies.  Value 3 is unused
  * (a tf32 split would need the same two pieces at half the bf16 tensor rate
  * and twice the operand bytes). */
 typedef enum {
@@ -233,13 +235,13 @@ SRE_API sre_status_t sre_sum4_range(sre_plan_t plan, const void *d_state, int N,
  * for the normalised state, i.e. log2(S_alpha / (d n2^{2 alpha})) / (1 - alpha)
  * with S_alpha = sum_{x,z} |A_x(z)|^{2 alpha} of the stored state.  The same
  * XOR-FWHT pass as M2 (Algorithm 1) with the exponent 2 alpha in place of 4;
- * for x >= 4096 the conjugate symmetry gives sum_z |A_x(z)|^{2 alpha} =
+ * the conjugate symmetry gives sum_z |A_x(z)|^{2 alpha} =
  * 2^{2 alpha} sum_{z'} [(Re W)^{2 alpha} + (Im W)^{2 alpha}].  alpha = 2 is M2
  * (bitwise the same as sre_m2).  2 <= alpha <= SRE_MAX_ORDER, else
  * SRE_EINVAL.  SYNCHRONOUS; result in *m_host; other arguments and errors as
- * sre_m2.  FP32 modes: terms below the FP32 range (|A|^{2 alpha} < ~1e-45)
- * count as zero; for a normalised state they are far below the result's
- * rounding.
+ * sre_m2.  FP32 modes: terms below the FP32 range (|A|^{2 alpha} < ~1e-45,
+ * for x >= 4096 |A/2|^{2 alpha}) count as zero; for a normalised state they are
+ * far below the result's rounding.
  */
 SRE_API sre_status_t sre_m_alpha(sre_plan_t plan, const void *d_state, int N, int alpha,
                                  sre_stream_t stream, double *m_host);

@@ -354,10 +354,10 @@ LargeCfg choose_large_cfg(const DeviceInfo &dev, int N, int elem_bytes) {
     while (C_log > 0 && (double)c.R * (double)(1 << C_log) * per_x > budget) --C_log;
     c.C_log = C_log;
     c.G2_log = std::min(C_log, h2);
-    // pass 2 staged through TMA (FP32, h2 = 7 and 8) overlaps the copy of
-    // tile g + 2 with tile g: give each item four tiles or more
     c.stage1 = 1;
     c.stage2 = 1;
+    // items of four tiles or more: tiles by tensor copy (FP32, h2 = 7 and 8, and
+    // the tensor-core kernel) overlap the copy of tile g + 2 with tile g
     if (elem_bytes == 8 && h2 >= 5 && h2 <= 8) c.G2_log = std::min(C_log + 2, h2);
     c.B1_log = 0;
     return c;

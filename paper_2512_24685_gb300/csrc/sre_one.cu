@@ -14,9 +14,9 @@
 // memory, three shuffles; per 32 entries some 12 cycles of the L1 pipe and 10
 // of the FP32 pipes), with 16 warps per SM to cover latency.  Measured on
 // GB300, all shifts of one state: N = 16 4.6 ms (the two-pass kernel with 16
-// entries per thread and full transforms below x = 4096: 9.9 ms), N = 15 1.27
+// entries per thread and full transforms below x = 4096: 9.9 ms), N = 15 1.24
 // ms (2.04 ms, a CTA per SM parking three 4096-entry blocks in shared memory),
-// N = 14 in a batch of 60 0.32 ms per state (0.45 ms); 20.6 SM cycles per 32
+// N = 14 in a batch of 60 0.31 ms per state (0.45 ms); 20.6 SM cycles per 32
 // complex entries at N = 16.
 //
 // Tiles (one block's shifts, or one shift) are claimed from one counter: the

@@ -18,12 +18,12 @@
 // per pass or more).  A chunk owns one ring slot from its first
 // pass-1 item to its last pass-2 item.
 //
-// What bounds it: about 31 SM cycles per 32 entries of the halved transform at
+// What bounds it: about 30 SM cycles per 32 entries of the halved transform at
 // N = 18, of which the transforms themselves take 20 (sre_one.cu); the rest are
 // the row stores and loads through L2, the factor loads and the GPU-scope
 // fence of each item.  DRAM carries 3.4 TB/s of ring traffic that L2 does not
-// hold.  Measured on GB300: N = 18 112 ms for all shifts (16 entries per
-// thread, 4096-entry blocks and a fixed item order: 196 ms), N = 19 51.8 ms for
+// hold.  Measured on GB300: N = 18 109 ms for all shifts (16 entries per
+// thread, 4096-entry blocks and a fixed item order: 196 ms), N = 19 50.6 ms for
 // 58255 shifts (76.7 ms).
 #include <cuda_runtime.h>
 #include <stdint.h>
